@@ -17,6 +17,7 @@
 #include "../../include/pic.h"
 #include "pic_host.h"
 #include "pic_runtime.h"
+#include "pic_push32.cuh"
 #include "pic_tiled.cuh"
 
 using namespace pic;
@@ -372,24 +373,54 @@ int curl_only(pic_t* h, int i0, int ni) {
   return PIC_OK;
 }
 
+// The FP64 push moves the particles in place; the FP32 push writes them to the
+// second buffer.
+template <typename T>
+constexpr bool push_in_place() {
+  return sizeof(T) == 8;
+}
+
+// The compile-time strides of the FP32 push cover tiles of up to 8 cells per axis.
+inline bool push32_fixed(const Tiles& tl) { return tl.tx <= 8 && tl.ty <= 8 && tl.tz <= 8; }
+
+// Gather, push, move and deposit of the particles in buffer `cur`, tile
+// starts `tsi`.
+template <typename T>
+void launch_push(pic_t* h, const Geom<T>& g, int cur, int tsi, int origin_after, cudaStream_t s) {
+  const Tiles& tl = h->tiles;
+  const T hq = (T)(h->q * h->dt / (2.0 * h->m));
+  if constexpr (push_in_place<T>()) {
+    k_push_tiled<T><<<tl.n, kPushThreads64, tiled_smem_bytes<T>(tl), s>>>(
+        g, tl, fields<T>(h), parts<T>(h, cur), h->tstart[tsi], (int)h->capacity, h->keys, h->tcnt, hq, (T)h->q,
+        origin_after, x_lo(h), x_hi(h), h->d_pushed, h->d_ctrl + 2);
+  } else {
+    const bool fixed = push32_fixed(tl);
+    const size_t sm = fixed ? Smem32::of<true>(tl, Lay32<true>(tl)).total : Smem32::of<false>(tl, Lay32<false>(tl)).total;
+    (fixed ? k_push32<true> : k_push32<false>)<<<tl.n, kPushThreads32, sm, s>>>(
+        g, tl, fields<T>(h), parts<T>(h, cur), parts<T>(h, 1 - cur), h->tstart[tsi], (int)h->capacity, h->keys,
+        h->tcnt, hq, (T)h->q, origin_after, x_lo(h), x_hi(h), h->d_pushed, h->d_ctrl + 2);
+  }
+}
+
 // Counting sort of the current buffer by tile into the other buffer.
 template <typename T>
 int resort_all(pic_t* h) {
   if (h->capacity == 0) return PIC_OK;
-  const int nb = 1 - h->cur;
+  const int nb = 1 - h->cur, ns = 1 - h->tsi;
   const Tiles tl = h->tiles;
   GroupTimer tm(h, G_PART);
   CK(h, cudaMemsetAsync(h->tcnt, 0, sizeof(int) * tl.n, h->stream));
   CK(h, cudaMemsetAsync(h->tfill, 0, sizeof(int) * tl.n, h->stream));
   k_keys<T><<<grid_for(h->capacity, 256, 152 * 16), 256, 0, h->stream>>>(geom<T>(h), tl, parts<T>(h, h->cur),
                                                                          h->d_ctrl + h->cur, h->keys, h->tcnt);
-  k_scan_tiles<<<1, 1024, 0, h->stream>>>(h->tcnt, h->tstart[nb], tl.n, h->d_ctrl + nb, (int)h->capacity,
+  k_scan_tiles<<<1, 1024, 0, h->stream>>>(h->tcnt, h->tstart[ns], tl.n, h->d_ctrl + nb, (int)h->capacity,
                                           h->d_ctrl + 2);
   k_scatter<T><<<grid_for(h->capacity, 256, 152 * 16), 256, 0, h->stream>>>(
-      parts<T>(h, h->cur), h->keys, h->d_ctrl + h->cur, parts<T>(h, nb), h->tstart[nb], h->tfill, h->d_ctrl + 2);
+      parts<T>(h, h->cur), h->keys, h->d_ctrl + h->cur, parts<T>(h, nb), h->tstart[ns], h->tfill, h->d_ctrl + 2);
   counted(h, G_PART, 3);
   CK(h, cudaGetLastError());
   h->cur = nb;
+  h->tsi = ns;
   return PIC_OK;
 }
 
@@ -464,18 +495,17 @@ int step_tiled(pic_t* h) {
   const int shift = window_due(h, t_old, t_new, &frac_new);
   const int origin_after = shift ? (h->origin + 1) % h->nx : h->origin;
   const Tiles tl = h->tiles;
-  const int nb = 1 - h->cur;
+  const int nb = 1 - h->cur, ns = 1 - h->tsi;
   CK(h, cudaMemsetAsync(f.c[JX], 0, 3 * n * sizeof(T), h->stream));
   if (h->capacity > 0) {
     CK(h, cudaMemsetAsync(h->tcnt, 0, sizeof(int) * tl.n, h->stream));
     GroupTimer tm(h, G_PUSH);
     counted(h, G_PUSH);
-    const T hq = (T)(h->q * h->dt / (2.0 * h->m));
-    k_push_tiled<T><<<tl.n, push_threads<T>(), tiled_smem_bytes<T>(tl), h->stream>>>(
-        geom<T>(h), tl, f, parts<T>(h, h->cur), h->tstart[h->cur], (int)h->capacity, h->keys, h->tcnt, hq,
-        (T)h->q, origin_after, x_lo(h), x_hi(h), h->d_pushed, h->d_ctrl + 2);
+    launch_push<T>(h, geom<T>(h), h->cur, h->tsi, origin_after, h->stream);
     CK(h, cudaGetLastError());
   }
+  // the push leaves the moved particles in `moved`; re-binning puts them into `next`
+  const int moved = push_in_place<T>() ? h->cur : nb, next = 1 - moved;
   int rc = field_first_half<T>(h);
   if (rc) return rc;
   h->step += 1;
@@ -502,23 +532,25 @@ int step_tiled(pic_t* h) {
     L = load_spec(h, x_hi(h), x_hi(h));
     const long long nslot = (long long)h->ny * h->nz * h->ppc;
     k_inject_tiled<T><<<grid_for(nslot, 256, 152 * 16), 256, 0, h->stream>>>(
-        geom<T>(h), tl, parts<T>(h, nb), L, 0, h->tcnt, h->tstart[nb], h->tfill, h->d_ctrl + 2);
+        geom<T>(h), tl, parts<T>(h, next), L, 0, h->tcnt, h->tstart[ns], h->tfill, h->d_ctrl + 2);
     counted(h, G_PART);
   }
-  k_scan_tiles<<<1, 1024, 0, h->stream>>>(h->tcnt, h->tstart[nb], tl.n, h->d_ctrl + nb, (int)h->capacity,
+  k_scan_tiles<<<1, 1024, 0, h->stream>>>(h->tcnt, h->tstart[ns], tl.n, h->d_ctrl + next, (int)h->capacity,
                                           h->d_ctrl + 2);
   CK(h, cudaMemsetAsync(h->tfill, 0, sizeof(int) * tl.n, h->stream));
   k_scatter<T><<<grid_for(h->capacity, 256, 152 * 16), 256, 0, h->stream>>>(
-      parts<T>(h, h->cur), h->keys, h->d_ctrl + h->cur, parts<T>(h, nb), h->tstart[nb], h->tfill, h->d_ctrl + 2);
+      parts<T>(h, moved), h->keys, h->tstart[h->tsi] + tl.n, parts<T>(h, next), h->tstart[ns], h->tfill,
+      h->d_ctrl + 2);
   counted(h, G_PART, 2);
   if (inject) {
     const long long nslot = (long long)h->ny * h->nz * h->ppc;
     k_inject_tiled<T><<<grid_for(nslot, 256, 152 * 16), 256, 0, h->stream>>>(
-        geom<T>(h), tl, parts<T>(h, nb), L, 1, h->tcnt, h->tstart[nb], h->tfill, h->d_ctrl + 2);
+        geom<T>(h), tl, parts<T>(h, next), L, 1, h->tcnt, h->tstart[ns], h->tfill, h->d_ctrl + 2);
     counted(h, G_PART);
   }
   CK(h, cudaGetLastError());
-  h->cur = nb;
+  h->cur = next;
+  h->tsi = ns;
   return PIC_OK;
 }
 
@@ -830,7 +862,9 @@ int pic_create(const pic_grid* g, double dt, const pic_window* w, pic_t** out) {
     const int sm = 227 * 1024;
     cudaError_t e = h->precision == PIC_FP64
                         ? cudaFuncSetAttribute(k_push_tiled<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm)
-                        : cudaFuncSetAttribute(k_push_tiled<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+                        : cudaFuncSetAttribute(k_push32<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    if (e == cudaSuccess && h->precision == PIC_FP32)
+      e = cudaFuncSetAttribute(k_push32<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
     if (e == cudaSuccess)
       e = h->precision == PIC_FP64 ? cudaFuncSetAttribute(k_curl_tiled<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                           (int)curl_tiled_smem_bytes<double>())
@@ -1666,7 +1700,7 @@ struct pic_batch_t {
   cudaEvent_t fork = nullptr;
   std::vector<cudaEvent_t> join;
   cudaGraphExec_t exec[2] = {nullptr, nullptr};
-  std::vector<int> cur0;
+  std::vector<int> tsi0;
   int parity = 0;
   bool stale = true;
   long long kernels_per_step = 0;
@@ -1685,11 +1719,12 @@ int bfail(pic_batch_t* b, int code, const std::string& m) {
 
 // One step of member h on stream s, every step parameter read from the
 // device-side state (so the same captured launches replay every step).
-int enqueue_step_dyn(pic_t* h, cudaStream_t s, int cur, long long* kernels) {
+int enqueue_step_dyn(pic_t* h, cudaStream_t s, int tsi, long long* kernels) {
   using T = float;
+  static_assert(!push_in_place<T>(), "the particles stay in buffer h->cur");
   const size_t n = h->ncell;
   const Tiles tl = h->tiles;
-  const int nb = 1 - cur;
+  const int cur = h->cur, moved = 1 - cur, ns = 1 - tsi;
   Geom<T> g = geom<T>(h);
   g.dyn = h->d_dyn;
   Geom<T> gs = g;
@@ -1700,10 +1735,7 @@ int enqueue_step_dyn(pic_t* h, cudaStream_t s, int cur, long long* kernels) {
   CK(h, cudaMemsetAsync(f.c[JX], 0, 3 * n * sizeof(T), s));
   CK(h, cudaMemsetAsync(h->tcnt, 0, sizeof(int) * tl.n, s));
   k_step_begin<<<1, 32, 0, s>>>(h->d_dyn);
-  const T hq = (T)(h->q * h->dt / (2.0 * h->m));
-  k_push_tiled<T><<<tl.n, push_threads<T>(), tiled_smem_bytes<T>(tl), s>>>(g, tl, f, parts<T>(h, cur), h->tstart[cur],
-                                                            (int)h->capacity, h->keys, h->tcnt, hq, (T)h->q, 0,
-                                                            x_lo(h), x_hi(h), h->d_pushed, h->d_ctrl + 2);
+  launch_push<T>(h, g, cur, tsi, 0, s);
   k_e_update<T><<<e_update_grid(h), e_update_block(h), 0, s>>>(g, f, curl_view<T>(h), fc, pml_view<T>(h));
   launch_curl<T>(h, g, 1, 0, h->nx, s);
   k_window_commit<<<1, 32, 0, s>>>(h->d_dyn);
@@ -1716,17 +1748,17 @@ int enqueue_step_dyn(pic_t* h, cudaStream_t s, int cur, long long* kernels) {
   const long long nslot = (long long)h->ny * h->nz * std::max(h->ppc, 1);
   if (inject) {
     L = load_spec(h, x_hi(h), x_hi(h));
-    k_inject_tiled<T><<<grid_for(nslot, 256, 152 * 16), 256, 0, s>>>(gs, tl, parts<T>(h, nb), L, 0, h->tcnt,
-                                                                     h->tstart[nb], h->tfill, h->d_ctrl + 2);
+    k_inject_tiled<T><<<grid_for(nslot, 256, 152 * 16), 256, 0, s>>>(gs, tl, parts<T>(h, cur), L, 0, h->tcnt,
+                                                                     h->tstart[ns], h->tfill, h->d_ctrl + 2);
   }
-  k_scan_tiles<<<1, 1024, 0, s>>>(h->tcnt, h->tstart[nb], tl.n, h->d_ctrl + nb, (int)h->capacity, h->d_ctrl + 2);
+  k_scan_tiles<<<1, 1024, 0, s>>>(h->tcnt, h->tstart[ns], tl.n, h->d_ctrl + cur, (int)h->capacity, h->d_ctrl + 2);
   CK(h, cudaMemsetAsync(h->tfill, 0, sizeof(int) * tl.n, s));
-  k_scatter<T><<<grid_for(h->capacity, 256, 152 * 16), 256, 0, s>>>(parts<T>(h, cur), h->keys, h->d_ctrl + cur,
-                                                                     parts<T>(h, nb), h->tstart[nb], h->tfill,
+  k_scatter<T><<<grid_for(h->capacity, 256, 152 * 16), 256, 0, s>>>(parts<T>(h, moved), h->keys, h->tstart[tsi] + tl.n,
+                                                                     parts<T>(h, cur), h->tstart[ns], h->tfill,
                                                                      h->d_ctrl + 2);
   if (inject)
-    k_inject_tiled<T><<<grid_for(nslot, 256, 152 * 16), 256, 0, s>>>(gs, tl, parts<T>(h, nb), L, 1, h->tcnt,
-                                                                     h->tstart[nb], h->tfill, h->d_ctrl + 2);
+    k_inject_tiled<T><<<grid_for(nslot, 256, 152 * 16), 256, 0, s>>>(gs, tl, parts<T>(h, cur), L, 1, h->tcnt,
+                                                                     h->tstart[ns], h->tfill, h->d_ctrl + 2);
   *kernels += 11 + (inject ? 2 : 0);
   CK(h, cudaGetLastError());
   return PIC_OK;
@@ -1772,10 +1804,10 @@ void drop_graphs(pic_batch_t* b) {
 }
 
 // Bring every member to a capturable state and capture the two step graphs
-// (members alternate their particle buffers, so even and odd steps differ).
+// (members alternate their tile-start arrays, so even and odd steps differ).
 int prepare_and_capture(pic_batch_t* b) {
   drop_graphs(b);
-  b->cur0.assign(b->sims.size(), 0);
+  b->tsi0.assign(b->sims.size(), 0);
   for (size_t i = 0; i < b->sims.size(); ++i) {
     pic_t* h = b->sims[i];
     if (h->need_sort) {
@@ -1790,7 +1822,7 @@ int prepare_and_capture(pic_batch_t* b) {
     }
     int rc = dyn_to_device(h);
     if (rc) return bfail(b, rc, h->err);
-    b->cur0[i] = h->cur;
+    b->tsi0[i] = h->tsi;
   }
   for (int p = 0; p < 2; ++p) {
     long long kernels = 0;
@@ -1800,7 +1832,7 @@ int prepare_and_capture(pic_batch_t* b) {
     int rc = PIC_OK;
     for (size_t i = 0; i < b->sims.size() && rc == PIC_OK; ++i) {
       cudaStreamWaitEvent(b->side[i], b->fork, 0);
-      rc = enqueue_step_dyn(b->sims[i], b->side[i], b->cur0[i] ^ p, &kernels);
+      rc = enqueue_step_dyn(b->sims[i], b->side[i], b->tsi0[i] ^ p, &kernels);
       cudaEventRecord(b->join[i], b->side[i]);
       cudaStreamWaitEvent(b->stream, b->join[i], 0);
     }
@@ -1887,7 +1919,7 @@ int pic_batch_step(pic_batch_t* b, int n) {
   if (cudaEventElapsedTime(&ms, b->t0, b->t1) == cudaSuccess) b->last_ms = ms;
   for (size_t i = 0; i < b->sims.size(); ++i) {
     pic_t* h = b->sims[i];
-    h->cur = b->cur0[i] ^ b->parity;
+    h->tsi = b->tsi0[i] ^ b->parity;
     int rc = dyn_to_host(h);
     if (!rc) rc = check_device_error(h);
     if (rc) return bfail(b, rc, h->err);

@@ -51,7 +51,8 @@ struct pic_t {
   // tile-sorted particles
   pic::Tiles tiles = {1, 1, 1, 1, 1, 1, 1};
   int* keys = nullptr;      // destination tile per particle
-  int* tstart[2] = {nullptr, nullptr};  // tile starts of pb[0], pb[1]
+  int* tstart[2] = {nullptr, nullptr};  // tile starts, [tsi] those of the current buffer
+  int tsi = 0;
   int* tcnt = nullptr;      // per-tile counts of the next buffer
   int* tfill = nullptr;     // per-tile fill counters of the scatter
   bool need_sort = false;   // particles not grouped by tile (after load/set)

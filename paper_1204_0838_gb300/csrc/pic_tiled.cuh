@@ -22,24 +22,6 @@ __device__ __forceinline__ int tile_of(const Geom<T>& g, const Tiles& tl, int cx
 __host__ __device__ __forceinline__ int stage_n(const Tiles& tl) { return (tl.tx + 4) * (tl.ty + 4) * (tl.tz + 4); }
 __host__ __device__ __forceinline__ int jtile_n(const Tiles& tl) { return (tl.tx + 5) * (tl.ty + 5) * (tl.tz + 5); }
 
-// FP32 particle layout of the push (FP64 keeps its own, see k_push_tiled):
-// - cell rounds: the particles of a tile are taken in rounds, round r holding
-//   the r-th particle of every occupied cell (ranks from a shared-memory cell
-//   histogram), so that the lanes of a warp sit in distinct cells while
-//   consecutive lanes stay on neighbouring cells.  Ranks from kRounds - 1 up
-//   share the last round; the order is built for chunks of up to kOrderChunk
-//   list entries.
-// - fixed-point J tile: the deposit adds each contribution as an exact 64-bit
-//   fixed-point integer split over two 32-bit words with native shared-memory
-//   integer reductions (a float add on shared memory is a load plus a
-//   compare-and-swap loop).  The scale is a power of two 2^s per tile and
-//   component with 2^s <= 2^42 / B, B = |q jc| sum_p w_p over the tile: no
-//   node of the tile can receive more than B in magnitude (each contribution
-//   is bounded by |q w jc|), so the high word stays within 2^30 and the low
-//   word (12 bits per contribution) within 2^32 for fewer than 2^20
-//   contributions.  The resolution 2^-s is about 2^-42 B, far below the FP32
-//   rounding of the contributions themselves, and the tile sum is exact and
-//   independent of the order of the adds.
 // FP64 push: the gather and the deposit run in 64-bit fixed point on the
 // integer pipes (pic_fixed64.cuh).  The staged E/B become int64 at a power of
 // two 2^sF per tile and component with max|F| 2^sF < 2^60, and the J tile
@@ -50,37 +32,28 @@ __host__ __device__ __forceinline__ int jtile_n(const Tiles& tl) { return (tl.tx
 // 2^-60 of the tile's largest field and 2^-62 of B, are at the level of
 // FP64 rounding at those scales, and the deposit's products round without
 // bias, so that thousands of contributions to a node add up no drift.
-constexpr int kRounds = 32;
-constexpr int kOrderChunk = 2048;
-constexpr int kFixedLoBits = 12;
-constexpr int kFixedRange = 42;
 constexpr int kFixed64Range = 60;   // staged fields: 4-term sums need |x| < 2^60
 constexpr int kFixed64JRange = 62;  // J sums of single products
 constexpr long long kThird62 = 1537228672809129301LL;  // round(2^62 / 3)
-template <typename T>
-struct LaneLayout {
-  static constexpr bool cell_rounds = sizeof(T) == 4;
-  static constexpr bool fixed_j = sizeof(T) == 4;   // FP32 J words: 12-bit low part
-  static constexpr bool fixed64 = sizeof(T) == 8;   // FP64 fixed-point gather and J words
-  // shared ints after the J tile: [0, 3) J scales, FP32 3 weight sum, FP64
-  // [4, 10) field exponent maxima, [10, 16) field scales and [16, 18) the
-  // sums behind the J bounds
-  static constexpr int scale_ints = sizeof(T) == 8 ? 18 : 4;
-};
+// shared ints after the J tile: [0, 3) J scales, [4, 10) field exponent
+// maxima, [10, 16) field scales and [16, 18) the sums behind the J bounds
+constexpr int kScaleInts64 = 18;
 
+// Shared memory of the FP64 push for a tile.  For FP32 it is the size that a
+// handle accepts tiles by (the staged fields, the J tile and the ordering
+// scratch side by side); the FP32 push itself needs less.
 template <typename T>
 size_t tiled_smem_bytes(const Tiles& tl) {
   size_t b = sizeof(T) * 6 * (size_t)stage_n(tl) + 8 * 3 * (size_t)jtile_n(tl);
-  if (LaneLayout<T>::cell_rounds) b += 4 * ((size_t)tl.tx * tl.ty * tl.tz + 3 * kRounds) + 2 * (size_t)kOrderChunk;
-  return b + 4 * LaneLayout<T>::scale_ints;
+  if (sizeof(T) == 4) return b + 4 * ((size_t)tl.tx * tl.ty * tl.tz + 100) + 4096;
+  return b + 4 * kScaleInts64;
 }
 
 // The J tile's scale exponent s for component threadIdx.x (< 3): B 2^s <
 // 2^range for the bound B = 1.001 |q| S / (dt d_b d_c) on every node, where
 // S bounds the sum over the tile's particles of |w| times the largest
-// running sum of the deposit (FP32: S = sum_p |w|, a move of up to one cell;
-// FP64: from each particle's speed bound).  1.001: margin over the float
-// rounding of the sums.
+// running sum of the deposit, from each particle's speed bound.  1.001: margin
+// over the float rounding of the sums.
 template <typename T>
 __device__ __forceinline__ int j_scale(const Geom<T>& g, T q, float S, int range) {
   const int c = threadIdx.x;
@@ -126,29 +99,6 @@ __device__ __forceinline__ int warp_count(int* counter, int key, bool want_base,
   return __popc(m & lanemask_lt());
 }
 
-// Gather one field component from the staged tile: NA x NB x NC separable
-// sum (4 nodes along a node-centred axis; 4, or 5 with one zero weight, along
-// a half-staggered one), contracting z first, then y, then x.
-template <int NA, int NB, int NC, typename T>
-__device__ __forceinline__ T gather_smem(const T* __restrict__ s, int SY, int SZ, int bx, int by, int bz,
-                                         const T* wx, const T* wy, const T* wz) {
-  T ax = T(0);
-#pragma unroll
-  for (int a = 0; a < NA; ++a) {
-    T ay = T(0);
-#pragma unroll
-    for (int b = 0; b < NB; ++b) {
-      const T* row = s + ((bx + a) * SY + (by + b)) * SZ + bz;
-      T az = row[0] * wz[0];
-#pragma unroll
-      for (int c = 1; c < NC; ++c) az = fma(row[c], wz[c], az);
-      ay = fma(az, wy[b], ay);
-    }
-    ax = fma(ay, wx[a], ax);
-  }
-  return ax;
-}
-
 // Comparisons of an offset against 0, 1/2 and 1.  In FP64 they are made on
 // the bit pattern with integer instructions, off the slow FP64 pipe: for
 // doubles of either sign the int64 view orders non-negative values like the
@@ -156,9 +106,6 @@ __device__ __forceinline__ T gather_smem(const T* __restrict__ s, int SY, int SZ
 __device__ __forceinline__ bool lt_zero(double o) { return __double_as_longlong(o) < 0; }
 __device__ __forceinline__ bool ge_one(double o) { return __double_as_longlong(o) >= 0x3FF0000000000000LL; }
 __device__ __forceinline__ bool lt_half(double o) { return __double_as_longlong(o) < 0x3FE0000000000000LL; }
-__device__ __forceinline__ bool lt_zero(float o) { return o < 0.0f; }
-__device__ __forceinline__ bool ge_one(float o) { return o >= 1.0f; }
-__device__ __forceinline__ bool lt_half(float o) { return o < 0.5f; }
 
 // FP64 Esirkepov deposit of one particle into the fixed-point J tile: old
 // cell lc (staged frame) with node weights wn, cell step dc and new offsets
@@ -265,7 +212,6 @@ __device__ __forceinline__ int push_particle(const Geom<T>& g, const Tiles& tl, 
   const int N[3] = {g.nx, g.ny, g.nz};
   const T dtd[3] = {g.dt / g.dx, g.dt / g.dy, g.dt / g.dz};
   const T jc[3] = {T(-1) / (g.dt * g.dy * g.dz), T(-1) / (g.dt * g.dx * g.dz), T(-1) / (g.dt * g.dx * g.dy)};
-  const T third = T(1) / T(3);
   const int cell = p.cell[pi];
   int c0[3];
   c0[0] = cell / g.nyz;
@@ -301,8 +247,8 @@ __device__ __forceinline__ int push_particle(const Geom<T>& g, const Tiles& tl, 
     bn[d] = lc[d] - 1;
     bh[d] = lc[d] - (lo ? 2 : 1);
   }
-  if constexpr (LaneLayout<T>::fixed64) {
-    // FP64: the weights at 2^62 on the fixed-point staged tile
+  {
+    // the weights at 2^62 on the fixed-point staged tile
     const long long* sI = reinterpret_cast<const long long*>(sF);
     W62 Wn[3][4], Wh[3][4];
 #pragma unroll
@@ -335,13 +281,6 @@ __device__ __forceinline__ int push_particle(const Geom<T>& g, const Tiles& tl, 
         if (comp == k + 3) B[k] = v;
       }
     }
-  } else {
-    E[0] = gather_smem<4, 4, 4>(sF + 0 * nS, SY, SZ, bh[0], bn[1], bn[2], wh[0], wn[1], wn[2]);
-    E[1] = gather_smem<4, 4, 4>(sF + 1 * nS, SY, SZ, bn[0], bh[1], bn[2], wn[0], wh[1], wn[2]);
-    E[2] = gather_smem<4, 4, 4>(sF + 2 * nS, SY, SZ, bn[0], bn[1], bh[2], wn[0], wn[1], wh[2]);
-    B[0] = gather_smem<4, 4, 4>(sF + 3 * nS, SY, SZ, bn[0], bh[1], bh[2], wn[0], wh[1], wh[2]);
-    B[1] = gather_smem<4, 4, 4>(sF + 4 * nS, SY, SZ, bh[0], bn[1], bh[2], wh[0], wn[1], wh[2]);
-    B[2] = gather_smem<4, 4, 4>(sF + 5 * nS, SY, SZ, bh[0], bh[1], bn[2], wh[0], wh[1], wn[2]);
   }
 
   // relativistic Boris push
@@ -401,87 +340,7 @@ __device__ __forceinline__ int push_particle(const Geom<T>& g, const Tiles& tl, 
   // there (node 5 of the window carries nothing): nw = 4 or 5 nodes, and
   // the running sum along the current's own axis vanishes on its last
   // node, so only nw - 1 current values are nonzero.
-  if constexpr (LaneLayout<T>::fixed64) {
-    deposit_fixed64(jt, jc, lc, dc, wn, o1, bad ? 0.0 : (double)q * (double)p.w[pi]);
-  } else {
-    int lw[3], nw[3];
-    T S0[3][5], DS[3][5];
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      T w1[4];
-      bspline3(o1[d], w1);
-      const int p0 = dc[d] < 0 ? 1 : 0, p1 = dc[d] > 0 ? 1 : 0;
-      lw[d] = lc[d] - 1 - p0;
-      nw[d] = dc[d] != 0 ? 5 : 4;
-#pragma unroll
-      for (int m = 0; m < 5; ++m) {
-        const T a0 = p0 ? (m > 0 ? wn[d][m > 0 ? m - 1 : 0] : T(0)) : (m < 4 ? wn[d][m < 4 ? m : 3] : T(0));
-        const T a1 = p1 ? (m > 0 ? w1[m > 0 ? m - 1 : 0] : T(0)) : (m < 4 ? w1[m < 4 ? m : 3] : T(0));
-        S0[d][m] = a0;
-        DS[d][m] = a1 - a0;
-      }
-    }
-    const T qw = bad ? T(0) : q * p.w[pi];
-#pragma unroll
-    for (int comp = 0; comp < 3; ++comp) {
-      // axis `comp` carries the running sum; (b, c) are the other two axes
-      const int ab = comp == 0 ? 1 : 0, ac = comp == 2 ? 1 : 2;
-      T P[4];
-      T run = T(0);
-      const T cf = qw * jc[comp];
-#pragma unroll
-      for (int m = 0; m < 4; ++m) {
-        run += DS[comp][m];
-        P[m] = cf * run;
-      }
-      T ak[5], bk[5];
-#pragma unroll
-      for (int m = 0; m < 5; ++m) {
-        ak[m] = S0[ac][m] + T(0.5) * DS[ac][m];
-        bk[m] = T(0.5) * S0[ac][m] + third * DS[ac][m];
-      }
-      // strides of the three axes in the J tile; (m, b, c) walk (comp, ab, ac)
-      const int st[3] = {jt.JY * jt.JZ, jt.JZ, 1};
-      const int base0 = comp * jt.nJ + lw[0] * st[0] + lw[1] * st[1] + lw[2] * st[2];
-      const int sm_ = st[comp], sb_ = st[ab], sc_ = st[ac];
-      const int nm = nw[comp] - 1, nb = nw[ab], nc = nw[ac];
-      // P[m] as integers with a per-particle exponent kp (|P 2^kp| in
-      // [2^23, 2^24): the float's 24 significant bits, exactly), A with 2^30
-      // (exact for A >= 2^-7, within 2^-31 below); their product carries
-      // 2^(kp + 30), shifted to the tile's 2^s with rounding to nearest
-      const float pmax = fmaxf(fmaxf(fabsf(P[0]), fabsf(P[1])), fmaxf(fabsf(P[2]), fabsf(P[3])));
-      const int ep = ((__float_as_int(pmax) >> 23) & 255) - 127;
-      if (ep > -100) {  // else the particle carries no current along this axis (or below 2^-100)
-        const int kp = 23 - ep;
-        const float sp = __int_as_float((127 + kp) << 23);
-        int Pi[4];
-#pragma unroll
-        for (int m = 0; m < 4; ++m) Pi[m] = __float2int_rn(P[m] * sp);
-        const int sh = min(max(kp + 30 - jt.s[comp], 0), 62);
-        const long long half = (1LL << sh) >> 1;
-#pragma unroll
-        for (int b = 0; b < 5; ++b) {
-          if (b < nb) {
-            const T sb = S0[ab][b], db = DS[ab][b];
-#pragma unroll
-            for (int c = 0; c < 5; ++c) {
-              if (c < nc) {
-                const int Ai = __float2int_rn((sb * ak[c] + db * bk[c]) * 1073741824.0f);
-#pragma unroll
-                for (int m = 0; m < 4; ++m)
-                  if (m < nm) {
-                    const long long X = ((long long)Pi[m] * Ai + half) >> sh;
-                    const int idx = base0 + m * sm_ + b * sb_ + c * sc_;
-                    red_u32(jt.hi + idx, (unsigned)(X >> kFixedLoBits));
-                    red_u32(jt.lo + idx, (unsigned)X & ((1u << kFixedLoBits) - 1u));
-                  }
-              }
-            }
-          }
-        }
-      }
-    }
-  }
+  deposit_fixed64(jt, jc, lc, dc, wn, o1, bad ? 0.0 : (double)q * (double)p.w[pi]);
 
   // store in place; the key is the destination tile (or -1: absorbed)
   const int n0 = wrapi(c0[0] + dc[0], N[0]);
@@ -506,22 +365,17 @@ __device__ __forceinline__ int push_particle(const Geom<T>& g, const Tiles& tl, 
   return key;
 }
 
-// Threads per CTA of the push: FP32 256 (the cell-round order is built for
-// 256 threads; two CTAs of about 100 KB of shared memory per SM); FP64 512
-// (one CTA per SM, the FP64 tile takes most of the shared memory; 16 warps
-// at 128 registers hide the integer and fetch latencies better than 8 at
-// 254, despite a few hundred bytes of spills).
-template <typename T>
-constexpr int push_threads() {
-  return sizeof(T) == 8 ? 512 : 256;
-}
+// Threads per CTA of the FP64 push: 512 (one CTA per SM, the tile takes most of
+// the shared memory; 16 warps at 128 registers hide the integer and fetch
+// latencies better than 8 at 254, despite a few hundred bytes of spills).
+constexpr int kPushThreads64 = 512;
 
 // One CTA per tile.  keys[p] receives the particle's tile after the move (or
 // -1 when it leaves the open-x range once the window has moved to
 // origin_after); cnt_next[tile] counts the particles each tile will hold.
-// blockDim.x is push_threads<T>().
+// blockDim.x is kPushThreads64.
 template <typename T>
-__global__ void __launch_bounds__(push_threads<T>(), sizeof(T) == 8 ? 1 : 2) k_push_tiled(Geom<T> g, Tiles tl, Fields<T> f, Parts<T> p,
+__global__ void __launch_bounds__(kPushThreads64, 1) k_push_tiled(Geom<T> g, Tiles tl, Fields<T> f, Parts<T> p,
                                                    const int* __restrict__ tstart, int capacity,
                                                    int* __restrict__ keys, int* __restrict__ cnt_next,
                                                    T h, T q, int origin_after, int xlo, int xhi,
@@ -547,10 +401,9 @@ __global__ void __launch_bounds__(push_threads<T>(), sizeof(T) == 8 ? 1 : 2) k_p
   int* sexp = reinterpret_cast<int*>(jt.lo + 3 * nJ);
   jt.s = sexp;
   jt.fs = sexp + 10;
-  unsigned char* after_j = reinterpret_cast<unsigned char*>(sexp + LaneLayout<T>::scale_ints);
 
-  // stage E and B (wrapped storage indices; see the ring note in pic_device.cuh);
-  // FP64 also takes the largest exponent of each component
+  // stage E and B (wrapped storage indices; see the ring note in pic_device.cuh)
+  // and take the largest exponent of each component
   int emax[6] = {0, 0, 0, 0, 0, 0};
   for (int i = threadIdx.x; i < nS; i += blockDim.x) {
     const int lz = i % SZ, r = i / SZ;
@@ -561,13 +414,12 @@ __global__ void __launch_bounds__(push_threads<T>(), sizeof(T) == 8 ? 1 : 2) k_p
     for (int c = 0; c < 6; ++c) {
       const T v = f.c[c][gi];
       sF[c * nS + i] = v;
-      if constexpr (LaneLayout<T>::fixed64)
-        emax[c] = max(emax[c], (int)((__double_as_longlong(v) >> 52) & 0x7FF));
+      emax[c] = max(emax[c], (int)((__double_as_longlong(v) >> 52) & 0x7FF));
     }
   }
-  if (threadIdx.x < LaneLayout<T>::scale_ints) sexp[threadIdx.x] = 0;
+  if (threadIdx.x < kScaleInts64) sexp[threadIdx.x] = 0;
   __syncthreads();
-  if constexpr (LaneLayout<T>::fixed64) {
+  {
 #pragma unroll
     for (int c = 0; c < 6; ++c) {
       const unsigned e = __reduce_max_sync(0xffffffffu, (unsigned)emax[c]);
@@ -596,17 +448,8 @@ __global__ void __launch_bounds__(push_threads<T>(), sizeof(T) == 8 ? 1 : 2) k_p
     }
   }
   for (int i = threadIdx.x; i < 6 * nJ; i += blockDim.x) jt.hi[i] = 0u;
-  if constexpr (!LaneLayout<T>::fixed64) {
-    // the scale of the fixed-point J tile: B = |q jc| sum_p w_p bounds every node
-    float ws = 0.0f;
-    for (int k = threadIdx.x; k < pend - pbeg; k += blockDim.x) ws += fabsf((float)p.w[pbeg + k]);
-    for (int o = 16; o > 0; o >>= 1) ws += __shfl_down_sync(0xffffffffu, ws, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(reinterpret_cast<float*>(sexp + 3), ws);
-  }
   __syncthreads();
-  if constexpr (!LaneLayout<T>::fixed64) {
-    if (threadIdx.x < 3) sexp[threadIdx.x] = j_scale(g, q, __int_as_float(sexp[3]), kFixedRange);
-  } else {
+  {
     // a particle moves at most dt/d |u'| cells along an axis, and a running
     // sum of the deposit changes by at most 3/4 of the move (the slope bound
     // of the cubic spline's partial sums); 2^-20 covers the rounding
@@ -632,73 +475,11 @@ __global__ void __launch_bounds__(push_threads<T>(), sizeof(T) == 8 ? 1 : 2) k_p
       for (int i = threadIdx.x; i < nS; i += blockDim.x) sI[c * nS + i] = to_fixed(sF[c * nS + i], sfc[c]);
   }
   if (threadIdx.x == 0) atomicAdd(pushed, (unsigned long long)(pend - pbeg));
-  // the fixed-point low words hold up to 2^20 contributions each
-  if (LaneLayout<T>::fixed_j && threadIdx.x == 0 && pend - pbeg >= (1 << 20)) atomicOr(err, 16);
   __syncthreads();
   const int ntile = pend - pbeg;
 
-  if constexpr (LaneLayout<T>::cell_rounds) {
-    // cell-round order, chunk by chunk of the tile's list
-    const int ncell_t = tl.tx * tl.ty * tl.tz;
-    int* hist = reinterpret_cast<int*>(after_j);
-    int* rtot = hist + ncell_t;
-    int* rbase = rtot + kRounds;
-    int* rfill = rbase + kRounds;
-    unsigned short* order = reinterpret_cast<unsigned short*>(rfill + kRounds);
-    constexpr int kPer = kOrderChunk / 256;
-    for (int ch0 = 0; ch0 < ntile; ch0 += kOrderChunk) {
-      const int nch = min(kOrderChunk, ntile - ch0);
-      for (int i = threadIdx.x; i < ncell_t; i += blockDim.x) hist[i] = 0;
-      if (threadIdx.x < 3 * kRounds) rtot[threadIdx.x] = 0;
-      __syncthreads();
-      int rk[kPer];
-#pragma unroll
-      for (int it = 0; it < kPer; ++it) {
-        const int k = it * 256 + threadIdx.x;
-        int r = -1;
-        if (k < nch) {
-          const int cell = p.cell[pbeg + ch0 + k];
-          const int cx = cell / g.nyz, rem = cell - cx * g.nyz;
-          const int cy = rem / g.nz, cz = rem - cy * g.nz;
-          const int lx = cx - o3[0] - 2, ly = cy - o3[1] - 2, lz = cz - o3[2] - 2;
-          const bool in = lx >= 0 && lx < tl.tx && ly >= 0 && ly < tl.ty && lz >= 0 && lz < tl.tz;
-          const int lcell = in ? (lx * tl.ty + ly) * tl.tz + lz : 0;  // a stray particle (caught later) ranks in cell 0
-          r = min(atomicAdd(hist + lcell, 1), kRounds - 1);
-        }
-        rk[it] = r;
-        warp_count(rtot, r, false, nullptr);
-      }
-      __syncthreads();
-      if (threadIdx.x < 32) {  // exclusive scan of the round sizes (kRounds = 32)
-        const int v = rtot[threadIdx.x];
-        int incl = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int n = __shfl_up_sync(0xffffffffu, incl, o);
-          if (threadIdx.x >= o) incl += n;
-        }
-        rbase[threadIdx.x] = incl - v;
-      }
-      __syncthreads();
-#pragma unroll
-      for (int it = 0; it < kPer; ++it) {
-        int off;
-        const int rank = warp_count(rfill, rk[it], true, &off);
-        if (rk[it] >= 0) order[rbase[rk[it]] + off + rank] = (unsigned short)(it * 256 + threadIdx.x);
-      }
-      __syncthreads();
-      for (int base = 0; base < nch; base += blockDim.x) {
-        const int k = base + threadIdx.x;
-        int key = -2;
-        if (k < nch)
-          key = push_particle(g, tl, p, pbeg + ch0 + order[k], o3, sF, nS, SY, SZ, jt, h, q, origin_after,
-                              xlo, xhi, keys, err);
-        warp_count(cnt_next, key, false, nullptr);
-      }
-      __syncthreads();  // the next chunk reuses the histogram and the order
-    }
-  } else {
-    // FP64: the lanes of a warp take particles mrow apart in the list, which
+  {
+    // the lanes of a warp take particles mrow apart in the list, which
     // spreads the many particles of a dense cell (bubble walls) over warps.
     const int mrow = (ntile + 31) >> 5;
     const int nloop = 32 * mrow;
@@ -719,15 +500,9 @@ __global__ void __launch_bounds__(push_threads<T>(), sizeof(T) == 8 ? 1 : 2) k_p
   for (int i = threadIdx.x; i < 3 * nJ; i += blockDim.x) {
     const int comp = i / nJ, li = i - comp * nJ;
     T v;
-    if constexpr (LaneLayout<T>::fixed64) {
-      const long long X = (long long)(((unsigned long long)jt.hi[i] << 32) | jt.lo[i]);
-      if (X == 0) continue;
-      v = from_fixed(X, sexp[comp]);
-    } else {
-      const long long X = (long long)(int)jt.hi[i] * (1LL << kFixedLoBits) + (long long)jt.lo[i];
-      if (X == 0) continue;
-      v = ldexpf((float)X, -sexp[comp]);
-    }
+    const long long X = (long long)(((unsigned long long)jt.hi[i] << 32) | jt.lo[i]);
+    if (X == 0) continue;
+    v = from_fixed(X, sexp[comp]);
     const int lz = li % jt.JZ, r = li / jt.JZ;
     const int ly = r % jt.JY, lx = r / jt.JY;
     const size_t gi = (size_t)wrapi(o3[0] + lx, g.nx) * g.nyz + (size_t)wrapi(o3[1] + ly, g.ny) * g.nz +
