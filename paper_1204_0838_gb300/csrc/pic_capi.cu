@@ -18,6 +18,7 @@
 #include "pic_host.h"
 #include "pic_runtime.h"
 #include "pic_push32.cuh"
+#include "pic_push64.cuh"
 #include "pic_tiled.cuh"
 
 using namespace pic;
@@ -373,33 +374,29 @@ int curl_only(pic_t* h, int i0, int ni) {
   return PIC_OK;
 }
 
-// The FP64 push moves the particles in place; the FP32 push writes them to the
-// second buffer.
-template <typename T>
-constexpr bool push_in_place() {
-  return sizeof(T) == 8;
-}
+// The compile-time strides of the push cover tiles of up to 8 cells per axis.
+inline bool push_fixed(const Tiles& tl) { return tl.tx <= 8 && tl.ty <= 8 && tl.tz <= 8; }
 
-// The compile-time strides of the FP32 push cover tiles of up to 8 cells per axis.
-inline bool push32_fixed(const Tiles& tl) { return tl.tx <= 8 && tl.ty <= 8 && tl.tz <= 8; }
-
-// Gather, push, move and deposit of the particles in buffer `cur`, tile
-// starts `tsi`.
 template <typename T>
-void launch_push(pic_t* h, const Geom<T>& g, int cur, int tsi, int origin_after, cudaStream_t s) {
+using PushKernel = void (*)(Geom<T>, Tiles, Fields<T>, Parts<T>, Parts<T>, const int*, int, int*, int*, T, T, int, int,
+                            int, unsigned long long*, int*);
+template <typename T>
+PushKernel<T> push_kernel(bool fixed);
+template <>
+PushKernel<float> push_kernel<float>(bool fixed) { return fixed ? k_push32<true> : k_push32<false>; }
+template <>
+PushKernel<double> push_kernel<double>(bool fixed) { return fixed ? k_push64<true> : k_push64<false>; }
+
+// Gather, push, move and deposit of the particles of the current buffer, with
+// tile starts `tsi`; the moved particles go to the other buffer.
+template <typename T>
+void launch_push(pic_t* h, const Geom<T>& g, int tsi, int origin_after, cudaStream_t s) {
   const Tiles& tl = h->tiles;
-  const T hq = (T)(h->q * h->dt / (2.0 * h->m));
-  if constexpr (push_in_place<T>()) {
-    k_push_tiled<T><<<tl.n, kPushThreads64, tiled_smem_bytes<T>(tl), s>>>(
-        g, tl, fields<T>(h), parts<T>(h, cur), h->tstart[tsi], (int)h->capacity, h->keys, h->tcnt, hq, (T)h->q,
-        origin_after, x_lo(h), x_hi(h), h->d_pushed, h->d_ctrl + 2);
-  } else {
-    const bool fixed = push32_fixed(tl);
-    const size_t sm = fixed ? Smem32::of<true>(tl, Lay32<true>(tl)).total : Smem32::of<false>(tl, Lay32<false>(tl)).total;
-    (fixed ? k_push32<true> : k_push32<false>)<<<tl.n, kPushThreads32, sm, s>>>(
-        g, tl, fields<T>(h), parts<T>(h, cur), parts<T>(h, 1 - cur), h->tstart[tsi], (int)h->capacity, h->keys,
-        h->tcnt, hq, (T)h->q, origin_after, x_lo(h), x_hi(h), h->d_pushed, h->d_ctrl + 2);
-  }
+  const bool fixed = push_fixed(tl);
+  const size_t sm = fixed ? PushSmem::of<T, true>(tl).total : PushSmem::of<T, false>(tl).total;
+  push_kernel<T>(fixed)<<<tl.n, kPushThreads, sm, s>>>(
+      g, tl, fields<T>(h), parts<T>(h, h->cur), parts<T>(h, 1 - h->cur), h->tstart[tsi], (int)h->capacity, h->keys,
+      h->tcnt, (T)(h->q * h->dt / (2.0 * h->m)), (T)h->q, origin_after, x_lo(h), x_hi(h), h->d_pushed, h->d_ctrl + 2);
 }
 
 // Counting sort of the current buffer by tile into the other buffer.
@@ -495,17 +492,16 @@ int step_tiled(pic_t* h) {
   const int shift = window_due(h, t_old, t_new, &frac_new);
   const int origin_after = shift ? (h->origin + 1) % h->nx : h->origin;
   const Tiles tl = h->tiles;
-  const int nb = 1 - h->cur, ns = 1 - h->tsi;
+  const int cur = h->cur, moved = 1 - cur, ns = 1 - h->tsi;  // re-binning brings the moved particles back
   CK(h, cudaMemsetAsync(f.c[JX], 0, 3 * n * sizeof(T), h->stream));
   if (h->capacity > 0) {
     CK(h, cudaMemsetAsync(h->tcnt, 0, sizeof(int) * tl.n, h->stream));
     GroupTimer tm(h, G_PUSH);
     counted(h, G_PUSH);
-    launch_push<T>(h, geom<T>(h), h->cur, h->tsi, origin_after, h->stream);
+    launch_push<T>(h, geom<T>(h), h->tsi, origin_after, h->stream);
     CK(h, cudaGetLastError());
   }
-  // the push leaves the moved particles in `moved`; re-binning puts them into `next`
-  const int moved = push_in_place<T>() ? h->cur : nb, next = 1 - moved;
+
   int rc = field_first_half<T>(h);
   if (rc) return rc;
   h->step += 1;
@@ -532,24 +528,23 @@ int step_tiled(pic_t* h) {
     L = load_spec(h, x_hi(h), x_hi(h));
     const long long nslot = (long long)h->ny * h->nz * h->ppc;
     k_inject_tiled<T><<<grid_for(nslot, 256, 152 * 16), 256, 0, h->stream>>>(
-        geom<T>(h), tl, parts<T>(h, next), L, 0, h->tcnt, h->tstart[ns], h->tfill, h->d_ctrl + 2);
+        geom<T>(h), tl, parts<T>(h, cur), L, 0, h->tcnt, h->tstart[ns], h->tfill, h->d_ctrl + 2);
     counted(h, G_PART);
   }
-  k_scan_tiles<<<1, 1024, 0, h->stream>>>(h->tcnt, h->tstart[ns], tl.n, h->d_ctrl + next, (int)h->capacity,
+  k_scan_tiles<<<1, 1024, 0, h->stream>>>(h->tcnt, h->tstart[ns], tl.n, h->d_ctrl + cur, (int)h->capacity,
                                           h->d_ctrl + 2);
   CK(h, cudaMemsetAsync(h->tfill, 0, sizeof(int) * tl.n, h->stream));
   k_scatter<T><<<grid_for(h->capacity, 256, 152 * 16), 256, 0, h->stream>>>(
-      parts<T>(h, moved), h->keys, h->tstart[h->tsi] + tl.n, parts<T>(h, next), h->tstart[ns], h->tfill,
+      parts<T>(h, moved), h->keys, h->tstart[h->tsi] + tl.n, parts<T>(h, cur), h->tstart[ns], h->tfill,
       h->d_ctrl + 2);
   counted(h, G_PART, 2);
   if (inject) {
     const long long nslot = (long long)h->ny * h->nz * h->ppc;
     k_inject_tiled<T><<<grid_for(nslot, 256, 152 * 16), 256, 0, h->stream>>>(
-        geom<T>(h), tl, parts<T>(h, next), L, 1, h->tcnt, h->tstart[ns], h->tfill, h->d_ctrl + 2);
+        geom<T>(h), tl, parts<T>(h, cur), L, 1, h->tcnt, h->tstart[ns], h->tfill, h->d_ctrl + 2);
     counted(h, G_PART);
   }
   CK(h, cudaGetLastError());
-  h->cur = next;
   h->tsi = ns;
   return PIC_OK;
 }
@@ -860,11 +855,11 @@ int pic_create(const pic_grid* g, double dt, const pic_window* w, pic_t** out) {
     // the limit is a property of the kernel, shared by every handle: allow the
     // largest tile any handle may pick (227 KB); each launch asks for its own
     const int sm = 227 * 1024;
-    cudaError_t e = h->precision == PIC_FP64
-                        ? cudaFuncSetAttribute(k_push_tiled<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm)
-                        : cudaFuncSetAttribute(k_push32<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-    if (e == cudaSuccess && h->precision == PIC_FP32)
-      e = cudaFuncSetAttribute(k_push32<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    cudaError_t e = cudaSuccess;
+    for (int fixed = 0; fixed < 2 && e == cudaSuccess; ++fixed)
+      e = h->precision == PIC_FP64
+              ? cudaFuncSetAttribute(push_kernel<double>(fixed), cudaFuncAttributeMaxDynamicSharedMemorySize, sm)
+              : cudaFuncSetAttribute(push_kernel<float>(fixed), cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
     if (e == cudaSuccess)
       e = h->precision == PIC_FP64 ? cudaFuncSetAttribute(k_curl_tiled<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                           (int)curl_tiled_smem_bytes<double>())
@@ -1721,7 +1716,6 @@ int bfail(pic_batch_t* b, int code, const std::string& m) {
 // device-side state (so the same captured launches replay every step).
 int enqueue_step_dyn(pic_t* h, cudaStream_t s, int tsi, long long* kernels) {
   using T = float;
-  static_assert(!push_in_place<T>(), "the particles stay in buffer h->cur");
   const size_t n = h->ncell;
   const Tiles tl = h->tiles;
   const int cur = h->cur, moved = 1 - cur, ns = 1 - tsi;
@@ -1735,7 +1729,7 @@ int enqueue_step_dyn(pic_t* h, cudaStream_t s, int tsi, long long* kernels) {
   CK(h, cudaMemsetAsync(f.c[JX], 0, 3 * n * sizeof(T), s));
   CK(h, cudaMemsetAsync(h->tcnt, 0, sizeof(int) * tl.n, s));
   k_step_begin<<<1, 32, 0, s>>>(h->d_dyn);
-  launch_push<T>(h, g, cur, tsi, 0, s);
+  launch_push<T>(h, g, tsi, 0, s);
   k_e_update<T><<<e_update_grid(h), e_update_block(h), 0, s>>>(g, f, curl_view<T>(h), fc, pml_view<T>(h));
   launch_curl<T>(h, g, 1, 0, h->nx, s);
   k_window_commit<<<1, 32, 0, s>>>(h->d_dyn);

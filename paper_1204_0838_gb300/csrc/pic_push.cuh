@@ -1,0 +1,296 @@
+// pic_push.cuh -- what the FP32 and FP64 particle pushes share: the layout of
+// a tile's fields and current in shared memory, and the ranking of a tile's
+// particles per cell.  One CTA takes one tile, in passes of up to kChunk
+// particles:
+//   stage E, B; rank the particles per cell and list them in (rank, cell)
+//   order; gather, push, move, writing the moved particles in that order to the
+//   second buffer; turn the staged fields' memory into the J tile; deposit the
+//   particles that stayed in their cell, then the others; add the tile to J.
+// In (rank, cell) order the lanes of a warp hold distinct neighbouring cells,
+// so that their reads and adds at one offset from their own cells collide
+// little, and the writes are coalesced and nearly sorted for the next step.
+#pragma once
+
+#include "pic_tiled.cuh"
+
+namespace pic {
+
+constexpr int kPushThreads = 256;  // two CTAs per SM at 128 registers
+constexpr int kChunk = 3072;       // particles per pass over a tile
+constexpr int kRanks = 32;         // ranks per cell that are ordered; later ones follow in any order
+// entry of the order list: particle of the pass (12 bits), cell slot (12
+// bits), cell steps + 1 per axis (6 bits) and two flags
+constexpr unsigned kCross = 1u << 31;  // does not deposit with the ordered particles
+constexpr unsigned kStray = 1u << 30;  // outside the tile: dropped, error bit set
+
+// The shared-memory region.  Components are stored with their axes rotated,
+// [i_d][i_e][i_f] with (e, f) the axes after d in cyclic order, so that one
+// body serves the three rotations with the same offsets (three unrolled bodies
+// overflow the instruction cache): two field components per d, in T or 64-bit
+// words, and J as [d][hi, lo] in 32-bit words.  FIXED: tiles of up to 8 cells
+// per axis, strides known to the compiler; otherwise any tile.  The fixed
+// strides keep a warp on 4x8 neighbouring cells within two wavefronts per
+// 32-bit access, one for one of the three rotations (12 and 17 modulo 32 for
+// the fields, 13 and 12 modulo 32 for J), and within 4.3 of the 2 that a 64-bit
+// access needs when the lanes start at either half cell (12 and 9 modulo 16).
+template <typename T, bool FIXED>
+struct PushLayout {
+  int t[3];
+  __host__ __device__ explicit PushLayout(const Tiles& tl) : t{tl.tx, tl.ty, tl.tz} {}
+  // pad = 4: staged fields, 5: J
+  __host__ __device__ __forceinline__ int se(int d, int pad) const { return FIXED ? 8 + pad : t[(d + 2) % 3] + pad; }
+  __host__ __device__ __forceinline__ int sd(int d, int pad) const {
+    return FIXED ? (pad == 4 ? (sizeof(T) == 8 ? 153 : 145) : 172) : (t[(d + 1) % 3] + pad) * se(d, pad);
+  }
+  __host__ __device__ __forceinline__ int part(int d, int pad) const {
+    return FIXED ? (8 + pad) * sd(d, pad) : (t[d] + pad) * sd(d, pad);
+  }
+  __host__ __device__ __forceinline__ int start(int d, int pad) const { return FIXED ? 2 * d * part(0, pad) : 2 * d * part(d, pad); }
+  __host__ __device__ int region(int pad) const { return 6 * part(0, pad); }
+  // cell slots: a warp's 32 are 4x8 cells (fixed) or consecutive cells
+  __host__ __device__ int words() const { return FIXED ? 2 * t[0] : (t[0] * t[1] * t[2] + 31) / 32; }
+  __device__ __forceinline__ int slot(int lx, int ly, int lz) const {
+    return FIXED ? lx * 64 + ly * 8 + lz : (lx * t[1] + ly) * t[2] + lz;
+  }
+  __device__ __forceinline__ void cell(int s, int (&l)[3]) const {
+    if (FIXED) {
+      l[0] = s >> 6;
+      l[1] = (s >> 3) & 7;
+      l[2] = s & 7;
+    } else {
+      l[0] = s / (t[1] * t[2]);
+      const int r = s - l[0] * t[1] * t[2];
+      l[1] = r / t[2];
+      l[2] = r - l[1] * t[2];
+    }
+  }
+};
+
+// Shared memory: the region (staged fields and the ranking's scratch, then J),
+// the order list (32-bit entries), the FP32 pair list, the list of crossing
+// particles, the wrapped grid offsets per axis, and 64 ints of scalars.
+struct PushSmem {
+  size_t hist, mask, base, order, pair, cross, tab, scal, total;
+  template <typename T, bool FIXED>
+  __host__ __device__ static PushSmem of(const Tiles& tl) {
+    const PushLayout<T, FIXED> L(tl);
+    PushSmem s;
+    const size_t w = L.words();
+    size_t a = ((size_t)L.region(4) * sizeof(T) + 15) / 16 * 16;
+    s.hist = a;
+    a += 4 * 32 * w;
+    s.mask = a;
+    a += 4 * kRanks * w;
+    s.base = a;
+    a += (2 * kRanks * w + 15) / 16 * 16;
+    const size_t j = (size_t)L.region(5) * 4;
+    a = ((a > j ? a : j) + 15) / 16 * 16;
+    s.order = a;
+    a += 4 * (size_t)kChunk;
+    s.pair = a;
+    if (sizeof(T) == 4) a += 2 * (size_t)kChunk;  // FP64 takes the particles one by one
+    s.cross = a;
+    a += 2 * (size_t)kChunk;
+    s.tab = a;
+    a += 4 * (size_t)(tl.tx + tl.ty + tl.tz + 15);
+    s.scal = (a + 15) / 16 * 16;
+    s.total = s.scal + 4 * 64;
+    return s;
+  }
+};
+
+// Pointers into the shared memory of a CTA, and the scalars: [0] particles
+// without an ordered rank, [1] particles that left their cell, [2, 4) sums or
+// maxima over the pass, [4, 7) J scale per component, [8, 16) scan partials,
+// [16, 33) first pair of each pair of ranks, [33] ordered particles, [34, 50)
+// first position of each pair of ranks, [50, 62) field scales (FP64).
+struct PushTile {
+  int* hist;
+  unsigned* mask;         // [rank][word]: cells that hold more than `rank` particles
+  unsigned short* base;   // [rank][word]: position of the word's first particle
+  unsigned* order;
+  unsigned short* cross;
+  int *tabx, *taby, *tabz;  // wrapped grid offsets of the staged cells
+  int* sc;
+  int x0, y0, z0;         // tile corner (cells)
+
+  // position of rank r of the cell in slot s
+  __device__ __forceinline__ int position(int W, int r, int s) const {
+    const int i = r * W + (s >> 5);
+    return base[i] + __popc(mask[i] & ((1u << (s & 31)) - 1u));
+  }
+};
+
+template <typename T, bool FIXED>
+__device__ __forceinline__ PushTile push_tile(unsigned char* smem, const Geom<T>& g, const Tiles& tl, int t) {
+  const PushSmem so = PushSmem::of<T, FIXED>(tl);
+  PushTile P;
+  P.hist = reinterpret_cast<int*>(smem + so.hist);
+  P.mask = reinterpret_cast<unsigned*>(smem + so.mask);
+  P.base = reinterpret_cast<unsigned short*>(smem + so.base);
+  P.order = reinterpret_cast<unsigned*>(smem + so.order);
+  P.cross = reinterpret_cast<unsigned short*>(smem + so.cross);
+  P.tabx = reinterpret_cast<int*>(smem + so.tab);
+  P.taby = P.tabx + tl.tx + 5;
+  P.tabz = P.taby + tl.ty + 5;
+  P.sc = reinterpret_cast<int*>(smem + so.scal);
+  const int rest = t / tl.ntz;
+  P.x0 = (rest / tl.nty) * tl.tx;
+  P.y0 = (rest % tl.nty) * tl.ty;
+  P.z0 = (t % tl.ntz) * tl.tz;
+  // origin tile - 2; J reaches one cell further than E, B
+  for (int i = threadIdx.x; i < tl.tx + tl.ty + tl.tz + 15; i += kPushThreads) {
+    int v;
+    if (i < tl.tx + 5)
+      v = wrapi(P.x0 - 2 + i, g.nx) * g.nyz;
+    else if (i < tl.tx + tl.ty + 10)
+      v = wrapi(P.y0 - 2 + i - (tl.tx + 5), g.ny) * g.nz;
+    else
+      v = wrapi(P.z0 - 2 + i - (tl.tx + tl.ty + 10), g.nz);
+    P.tabx[i] = v;
+  }
+  return P;
+}
+
+// Clear the ranking's scratch for a pass (a barrier must follow).
+__device__ __forceinline__ void rank_clear(const PushTile& P, int W) {
+  for (int i = threadIdx.x; i < 32 * W; i += kPushThreads) P.hist[i] = 0;
+  for (int i = threadIdx.x; i < kRanks * W; i += kPushThreads) P.mask[i] = 0u;
+  if (threadIdx.x < 64) P.sc[threadIdx.x] = 0;
+}
+
+constexpr int kPerThread = kChunk / kPushThreads;
+
+// Count the pass's particles [c0, c0 + nch) per cell: sr[] = slot and rank of
+// this thread's particles (-2: outside the tile).  A barrier must follow.
+template <typename T, bool FIXED>
+__device__ __forceinline__ void rank_count(const PushTile& P, const PushLayout<T, FIXED>& L, const Geom<T>& g,
+                                           const Tiles& tl, const int* __restrict__ cells, int c0, int nch,
+                                           int (&sr)[kPerThread], int* err) {
+  const float inv_nyz = 1.0f / (float)g.nyz, inv_nz = 1.0f / (float)g.nz;
+#pragma unroll
+  for (int it = 0; it < kPerThread; ++it) {
+    const int k = it * kPushThreads + threadIdx.x;
+    sr[it] = -1;
+    if (k < nch) {
+      // cell - (tile corner) split by quotient estimates, then checked exactly
+      const int rel = cells[c0 + k] - P.x0 * g.nyz - P.y0 * g.nz - P.z0;
+      int lx = __float2int_rn((float)rel * inv_nyz);
+      int rem = rel - lx * g.nyz;
+      if (rem < 0) {
+        lx -= 1;
+        rem += g.nyz;
+      }
+      int ly = __float2int_rn((float)rem * inv_nz);
+      int lz = rem - ly * g.nz;
+      if (lz < 0) {
+        ly -= 1;
+        lz += g.nz;
+      }
+      const bool in = lx >= 0 && lx < tl.tx && ly >= 0 && ly < tl.ty && lz >= 0 && lz < tl.tz &&
+                      (lx * g.ny + ly) * g.nz + lz == rel;
+      if (in) {
+        const int s = L.slot(lx, ly, lz);
+        sr[it] = s | (atomicAdd(P.hist + s, 1) << 12);
+      } else {  // never expected: keeps every index in range
+        atomicOr(err, 4);
+        sr[it] = -2;
+      }
+    }
+  }
+}
+
+// Occupancy of every rank: bit of a slot set in mask[r][word] if the cell holds
+// more than r particles.  A barrier must follow.
+__device__ __forceinline__ void rank_masks(const PushTile& P, int W) {
+  for (int i = threadIdx.x; i < 32 * W; i += kPushThreads) {
+    const int n = min(P.hist[i], kRanks);
+    for (int r = 0;; ++r) {
+      const unsigned m = __ballot_sync(0xffffffffu, n > r);
+      if (!m) break;
+      if ((threadIdx.x & 31) == 0) P.mask[r * W + (i >> 5)] = m;
+    }
+  }
+}
+
+// Positions: an exclusive scan of the populations over (rank, word), then the
+// order list.  Ends with the list written (a barrier must follow).
+__device__ __forceinline__ void rank_order(const PushTile& P, int W, int nch, const int (&sr)[kPerThread]) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  {
+    const int n = kRanks * W, per = (n + kPushThreads - 1) / kPushThreads;
+    const int b = min(tid * per, n), e = min(b + per, n);
+    int s = 0;
+    for (int i = b; i < e; ++i) s += __popc(P.mask[i]);
+    int incl = s;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += v;
+    }
+    if (lane == 31) P.sc[8 + (tid >> 5)] = incl;
+    __syncthreads();
+    int run = incl - s;
+    for (int k = 0; k < (tid >> 5); ++k) run += P.sc[8 + k];
+    for (int i = b; i < e; ++i) {
+      P.base[i] = (unsigned short)run;
+      run += __popc(P.mask[i]);
+    }
+    if (tid == kPushThreads - 1) P.sc[33] = run;
+  }
+  __syncthreads();
+  const int ranked = P.sc[33];
+#pragma unroll
+  for (int it = 0; it < kPerThread; ++it) {
+    const int k = it * kPushThreads + tid;
+    if (k < nch) {
+      const int v = sr[it], s = v & 4095, r = v >> 12;
+      const bool stray = v == -2;
+      const int pos = !stray && r < kRanks ? P.position(W, r, s) : ranked + atomicAdd(P.sc, 1);
+      P.order[pos] = stray ? (unsigned)k | kStray : (unsigned)k | ((unsigned)s << 12);
+    }
+  }
+}
+
+// Store a moved particle's cell and key.  l: its cell in the tile, dc: its
+// steps (at most one cell per axis, periodic in the storage frame).  Returns
+// the destination tile or -1 (absorbed), and lists a particle that left its
+// cell at position pos.
+template <typename T>
+__device__ __forceinline__ int place_moved(const PushTile& P, const Geom<T>& g, const Tiles& tl, int t,
+                                           const int (&l)[3], const int (&dc)[3], bool good, int origin_after,
+                                           int xlo, int xhi, int pos, unsigned ent, int* cell_out, int* key_out) {
+  int n0 = P.x0 + l[0] + dc[0], n1 = P.y0 + l[1] + dc[1], n2 = P.z0 + l[2] + dc[2];
+  int key = t;
+  if (dc[0] | dc[1] | dc[2]) {
+    n0 = wrapi(n0, g.nx), n1 = wrapi(n1, g.ny), n2 = wrapi(n2, g.nz);
+    if ((unsigned)(n0 - P.x0) >= (unsigned)tl.tx || (unsigned)(n1 - P.y0) >= (unsigned)tl.ty ||
+        (unsigned)(n2 - P.z0) >= (unsigned)tl.tz)
+      key = tile_of(g, tl, n0, n1, n2);
+    P.order[pos] = ent | kCross | ((unsigned)(dc[0] + 1) << 24) | ((unsigned)(dc[1] + 1) << 26) |
+                   ((unsigned)(dc[2] + 1) << 28);
+    P.cross[atomicAdd(P.sc + 1, 1)] = (unsigned short)pos;
+  }
+  *cell_out = (n0 * g.ny + n1) * g.nz + n2;
+  if (!g.periodic_x) {
+    int rel = n0 - origin_after;
+    if (rel < 0) rel += g.nx;
+    if (rel < xlo || rel > xhi) key = -1;
+  }
+  // absorbing layers: a particle that leaves the y, z cells [L, n - L) is absorbed
+  if (g.pml && (n1 < g.pml || n1 >= g.ny - g.pml || n2 < g.pml || n2 >= g.nz - g.pml)) key = -1;
+  if (!good) {  // absorbed without moving or depositing
+    key = -1;
+    P.order[pos] = ent | kCross;
+  }
+  *key_out = key;
+  return key;
+}
+
+// Count the particles that leave for other tiles (all 32 lanes call).
+__device__ __forceinline__ void count_leaving(int* cnt_next, int key, int t) {
+  const int k = key == t ? -2 : key;
+  if (__any_sync(0xffffffffu, k >= 0)) warp_count(cnt_next, k, false, nullptr);
+}
+
+}  // namespace pic

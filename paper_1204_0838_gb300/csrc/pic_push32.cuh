@@ -46,87 +46,9 @@
 // that the FP32 shape factors leave in P itself.
 #pragma once
 
-#include "pic_tiled.cuh"
+#include "pic_push.cuh"
 
 namespace pic {
-
-constexpr int kPushThreads32 = 256;
-constexpr int kChunk32 = 3072;  // particles per pass over a tile
-constexpr int kRanks32 = 32;    // ranks per cell that are ordered; later ones follow in any order
-constexpr unsigned kCross32 = 1u << 31, kStray32 = 1u << 30;
-
-// The shared-memory region in words.  Component d of E, B and J is stored with
-// its axes rotated, [i_d][i_e][i_f] with (e, f) the axes after d in cyclic
-// order, so that one body serves the three components with the same offsets
-// (three unrolled bodies overflow the instruction cache).  E, B: [d][E, B]
-// [...]; J: [d][hi, lo][...].  FIXED: tiles of up to 8 cells per axis, strides
-// known to the compiler; otherwise any tile.  The fixed strides (12 and 13
-// along e, 17 and 12 modulo 32 along d) keep a warp on 4x8 neighbouring cells
-// within two wavefronts per access, one for one of the three rotations.
-template <bool FIXED>
-struct Lay32 {
-  int t[3];
-  __host__ __device__ explicit Lay32(const Tiles& tl) : t{tl.tx, tl.ty, tl.tz} {}
-  // pad = 4: staged fields, 5: J
-  __host__ __device__ __forceinline__ int se(int d, int pad) const { return FIXED ? 8 + pad : t[(d + 2) % 3] + pad; }
-  __host__ __device__ __forceinline__ int sd(int d, int pad) const {
-    return FIXED ? (pad == 4 ? 145 : 172) : (t[(d + 1) % 3] + pad) * se(d, pad);
-  }
-  __host__ __device__ __forceinline__ int part(int d, int pad) const {
-    return FIXED ? (8 + pad) * sd(d, pad) : (t[d] + pad) * sd(d, pad);
-  }
-  __host__ __device__ __forceinline__ int start(int d, int pad) const { return FIXED ? 2 * d * part(0, pad) : 2 * d * part(d, pad); }
-  __host__ __device__ int region(int pad) const { return 6 * part(0, pad); }
-  // cell slots: a warp's 32 are 4x8 cells (fixed) or consecutive cells
-  __host__ __device__ int words() const { return FIXED ? 2 * t[0] : (t[0] * t[1] * t[2] + 31) / 32; }
-  __device__ __forceinline__ int slot(int lx, int ly, int lz) const {
-    return FIXED ? lx * 64 + ly * 8 + lz : (lx * t[1] + ly) * t[2] + lz;
-  }
-  __device__ __forceinline__ void cell(int s, int (&l)[3]) const {
-    if (FIXED) {
-      l[0] = s >> 6;
-      l[1] = (s >> 3) & 7;
-      l[2] = s & 7;
-    } else {
-      l[0] = s / (t[1] * t[2]);
-      const int r = s - l[0] * t[1] * t[2];
-      l[1] = r / t[2];
-      l[2] = r - l[1] * t[2];
-    }
-  }
-};
-
-// Shared memory: the region (staged fields and the ranking's scratch, then J),
-// the order list (32-bit entries), the pair list, the list of crossing
-// particles, the wrapped grid offsets per axis, and 64 ints of scalars.
-struct Smem32 {
-  size_t hist, mask, base, order, pair, cross, tab, scal, total;
-  template <bool FIXED>
-  __host__ __device__ static Smem32 of(const Tiles& tl, const Lay32<FIXED>& L) {
-    Smem32 s;
-    const size_t w = L.words();
-    size_t a = ((size_t)L.region(4) * 4 + 15) / 16 * 16;
-    s.hist = a;
-    a += 4 * 32 * w;
-    s.mask = a;
-    a += 4 * kRanks32 * w;
-    s.base = a;
-    a += (2 * kRanks32 * w + 15) / 16 * 16;
-    const size_t j = (size_t)L.region(5) * 4;
-    a = ((a > j ? a : j) + 15) / 16 * 16;
-    s.order = a;
-    a += 4 * (size_t)kChunk32;
-    s.pair = a;
-    a += 2 * (size_t)kChunk32;
-    s.cross = a;
-    a += 2 * (size_t)kChunk32;
-    s.tab = a;
-    a += 4 * (size_t)(tl.tx + tl.ty + tl.tz + 15);
-    s.scal = (a + 15) / 16 * 16;
-    s.total = s.scal + 4 * 64;
-    return s;
-  }
-};
 
 // Pairs of FP32 values (the two particles of a thread), one instruction for both.
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
@@ -263,7 +185,7 @@ constexpr float kA30 = 1073741824.0f;  // 2^30
 constexpr long long kHalf28 = 1LL << 28;
 
 template <bool FIXED>
-__global__ void __launch_bounds__(kPushThreads32, 2)
+__global__ void __launch_bounds__(kPushThreads, 2)
     k_push32(Geom<float> g, Tiles tl, Fields<float> f, Parts<float> p, Parts<float> pn,
              const int* __restrict__ tstart, int capacity, int* __restrict__ keys, int* __restrict__ cnt_next,
              float h, float q, int origin_after, int xlo, int xhi, unsigned long long* pushed, int* err) {
@@ -272,63 +194,37 @@ __global__ void __launch_bounds__(kPushThreads32, 2)
   const int t = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
   const int pbeg = min(tstart[t], capacity), pend = min(tstart[t + 1], capacity);
   if (pbeg >= pend) return;
-  const Lay32<FIXED> L(tl);
-  const Smem32 so = Smem32::of<FIXED>(tl, L);
+  const PushLayout<float, FIXED> L(tl);
+  const PushTile P = push_tile<float, FIXED>(smem_raw, g, tl, t);
+  const PushSmem so = PushSmem::of<float, FIXED>(tl);
   float* sF = reinterpret_cast<float*>(smem_raw);
   unsigned* sJ = reinterpret_cast<unsigned*>(smem_raw);
-  int* hist = reinterpret_cast<int*>(smem_raw + so.hist);
-  unsigned* mask = reinterpret_cast<unsigned*>(smem_raw + so.mask);
-  unsigned short* base = reinterpret_cast<unsigned short*>(smem_raw + so.base);
-  unsigned* order = reinterpret_cast<unsigned*>(smem_raw + so.order);
   unsigned short* pairB = reinterpret_cast<unsigned short*>(smem_raw + so.pair);
-  unsigned short* cross = reinterpret_cast<unsigned short*>(smem_raw + so.cross);
-  int* tabx = reinterpret_cast<int*>(smem_raw + so.tab);
-  int* taby = tabx + tl.tx + 5;
-  int* tabz = taby + tl.ty + 5;
-  // scalars: [0] tail count, [1] crossing count, [2] sum |w|, [3] max |w|
-  // (bits), [4, 7) kp, [8, 16) scan partials, [16, 33) first pair of a round,
-  // [33] ranked particles, [34, 50) first position of a round's first particles
-  int* sc = reinterpret_cast<int*>(smem_raw + so.scal);
+  unsigned* order = P.order;
+  int* sc = P.sc;
   const int W = L.words();
-  const int tzi = t % tl.ntz, rest = t / tl.ntz;
-  const int x0 = (rest / tl.nty) * tl.tx, y0 = (rest % tl.nty) * tl.ty, z0 = tzi * tl.tz;
-
-  // wrapped grid offsets of the staged cells (origin tile - 2; J reaches one
-  // cell further than E, B)
-  for (int i = tid; i < tl.tx + tl.ty + tl.tz + 15; i += kPushThreads32) {
-    int v;
-    if (i < tl.tx + 5)
-      v = wrapi(x0 - 2 + i, g.nx) * g.nyz;
-    else if (i < tl.tx + tl.ty + 10)
-      v = wrapi(y0 - 2 + i - (tl.tx + 5), g.ny) * g.nz;
-    else
-      v = wrapi(z0 - 2 + i - (tl.tx + tl.ty + 10), g.nz);
-    tabx[i] = v;
-  }
   const int ntile = pend - pbeg;
   if (tid == 0) {
     atomicAdd(pushed, (unsigned long long)ntile);
     if (ntile >= (1 << 20)) atomicOr(err, 16);
   }
-  const int npass = (ntile + kChunk32 - 1) / kChunk32, per_pass = (ntile + npass - 1) / npass;
+  const int npass = (ntile + kChunk - 1) / kChunk, per_pass = (ntile + npass - 1) / npass;
   const float dtd[3] = {g.dt / g.dx, g.dt / g.dy, g.dt / g.dz};
   int own = 0;
 
   for (int ch0 = 0; ch0 < ntile; ch0 += per_pass) {
     const int nch = min(per_pass, ntile - ch0), c0 = pbeg + ch0;
-    for (int i = tid; i < 32 * W; i += kPushThreads32) hist[i] = 0;
-    for (int i = tid; i < kRanks32 * W; i += kPushThreads32) mask[i] = 0u;
-    if (tid < 64) sc[tid] = 0;
+    rank_clear(P, W);
     __syncthreads();
 
     // stage E, B: a half warp per (x, y) row, the lanes along z
     {
       const int SY = tl.ty + 4, rows = (tl.tx + 4) * SY, SZ = tl.tz + 4;
-      for (int r = tid >> 4; r < rows; r += kPushThreads32 / 16) {
+      for (int r = tid >> 4; r < rows; r += kPushThreads / 16) {
         const int lx = r / SY, ly = r - lx * SY;
-        const int gi0 = tabx[lx] + taby[ly];
+        const int gi0 = P.tabx[lx] + P.taby[ly];
         for (int lz = tid & 15; lz < SZ; lz += 16) {
-          const int gi = gi0 + tabz[lz];
+          const int gi = gi0 + P.tabz[lz];
           const int i3[3] = {lx, ly, lz};
 #pragma unroll
           for (int d = 0; d < 3; ++d) {
@@ -343,137 +239,61 @@ __global__ void __launch_bounds__(kPushThreads32, 2)
       asm volatile("cp.async.commit_group;" ::: "memory");
     }
 
-    // rank the chunk's particles per cell; sum and maximum of |w|
-    constexpr int kPer = kChunk32 / kPushThreads32;
-    int sr[kPer];
-    float ws = 0.0f, wm = 0.0f;
-    const float inv_nyz = 1.0f / (float)g.nyz, inv_nz = 1.0f / (float)g.nz;
-#pragma unroll
-    for (int it = 0; it < kPer; ++it) {
-      const int k = it * kPushThreads32 + tid;
-      sr[it] = -1;
-      if (k < nch) {
-        const int cell = p.cell[c0 + k];
+    // rank the pass's particles per cell; sum and maximum of |w|
+    int sr[kPerThread];
+    rank_count(P, L, g, tl, p.cell, c0, nch, sr, err);
+    {
+      float ws = 0.0f, wm = 0.0f;
+      for (int k = tid; k < nch; k += kPushThreads) {
         const float wa = fabsf(p.w[c0 + k]);
         ws += wa;
         wm = fmaxf(wm, wa);
-        // cell - (tile corner) split by quotient estimates, then checked exactly
-        const int rel = cell - x0 * g.nyz - y0 * g.nz - z0;
-        int lx = __float2int_rn((float)rel * inv_nyz);
-        int rem = rel - lx * g.nyz;
-        if (rem < 0) {
-          lx -= 1;
-          rem += g.nyz;
-        }
-        int ly = __float2int_rn((float)rem * inv_nz);
-        int lz = rem - ly * g.nz;
-        if (lz < 0) {
-          ly -= 1;
-          lz += g.nz;
-        }
-        const bool in = lx >= 0 && lx < tl.tx && ly >= 0 && ly < tl.ty && lz >= 0 && lz < tl.tz &&
-                        (lx * g.ny + ly) * g.nz + lz == rel;
-        if (in) {
-          const int s = L.slot(lx, ly, lz);
-          sr[it] = s | (atomicAdd(hist + s, 1) << 12);
-        } else {  // never expected: keeps every index in range
-          atomicOr(err, 4);
-          sr[it] = -2;
-        }
       }
-    }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      ws += __shfl_down_sync(0xffffffffu, ws, o);
-      wm = fmaxf(wm, __shfl_down_sync(0xffffffffu, wm, o));
-    }
-    if (lane == 0) {
-      atomicAdd(reinterpret_cast<float*>(sc + 2), ws);
-      atomicMax(sc + 3, __float_as_int(wm));
+      for (int o = 16; o > 0; o >>= 1) {
+        ws += __shfl_down_sync(0xffffffffu, ws, o);
+        wm = fmaxf(wm, __shfl_down_sync(0xffffffffu, wm, o));
+      }
+      if (lane == 0) {
+        atomicAdd(reinterpret_cast<float*>(sc + 2), ws);
+        atomicMax(sc + 3, __float_as_int(wm));
+      }
     }
     __syncthreads();
-
-    // occupancy of every rank: bit of a slot set in mask[r][word] if the cell
-    // holds more than r particles
-    for (int i = tid; i < 32 * W; i += kPushThreads32) {
-      const int n = min(hist[i], kRanks32);
-      for (int r = 0;; ++r) {
-        const unsigned m = __ballot_sync(0xffffffffu, n > r);
-        if (!m) break;
-        if (lane == 0) mask[r * W + (i >> 5)] = m;
-      }
-    }
+    rank_masks(P, W);
     if (tid < 3) {
       // kp: |P| 2^kp < 2^31 for P <= 0.76 |q| max w jc, and B 2^(kp + 1) < 2^42
       const float jcc = tid == 0 ? g.dt * g.dy * g.dz : (tid == 1 ? g.dt * g.dx * g.dz : g.dt * g.dx * g.dy);
-      const float P = 0.76f * fabsf(q) * __int_as_float(sc[3]) / jcc;
+      const float Pm = 0.76f * fabsf(q) * __int_as_float(sc[3]) / jcc;
       const float B = 1.001f * fabsf(q) * __int_as_float(sc[2]) / jcc;
-      const int ep = ((__float_as_int(P) >> 23) & 255) - 127, eb = ((__float_as_int(B) >> 23) & 255) - 127;
+      const int ep = ((__float_as_int(Pm) >> 23) & 255) - 127, eb = ((__float_as_int(B) >> 23) & 255) - 127;
       sc[4 + tid] = B > 0.0f ? max(min(min(30 - ep, 40 - eb), 120), -120) : 0;
     }
     __syncthreads();
-    // exclusive scan of the population counts over (rank, word)
-    {
-      const int n = kRanks32 * W, per = (n + kPushThreads32 - 1) / kPushThreads32;
-      const int b = min(tid * per, n), e = min(b + per, n);
-      int s = 0;
-      for (int i = b; i < e; ++i) s += __popc(mask[i]);
-      int incl = s;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-      }
-      if (lane == 31) sc[8 + (tid >> 5)] = incl;
-      __syncthreads();
-      int run = incl - s;
-      for (int k = 0; k < (tid >> 5); ++k) run += sc[8 + k];
-      for (int i = b; i < e; ++i) {
-        base[i] = (unsigned short)run;
-        run += __popc(mask[i]);
-      }
-      if (tid == kPushThreads32 - 1) sc[33] = run;
-    }
-    __syncthreads();
-    // pairs of a round: as many as the round's first particles
+    rank_order(P, W, nch, sr);
+    // pairs of ranks 2k, 2k + 1: as many as particles of rank 2k
     if (tid < 32) {
-      const int r = 2 * min(lane, kRanks32 / 2 - 1);
-      const int first = base[r * W], next = base[(r + 1) * W];
-      const int n = lane < kRanks32 / 2 ? next - first : 0;
+      const int r = 2 * min(lane, kRanks / 2 - 1);
+      const int first = P.base[r * W], next = P.base[(r + 1) * W];
+      const int n = lane < kRanks / 2 ? next - first : 0;
       int incl = n;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         const int v = __shfl_up_sync(0xffffffffu, incl, o);
         if (lane >= o) incl += v;
       }
-      if (lane <= kRanks32 / 2) sc[16 + lane] = incl - n;
-      if (lane < kRanks32 / 2) sc[34 + lane] = first;
-    }
-    const int ranked = sc[33];
-#pragma unroll
-    for (int it = 0; it < kPer; ++it) {
-      const int k = it * kPushThreads32 + tid;
-      if (k < nch) {
-        const int v = sr[it];
-        const int s = v & 4095, r = v >> 12;
-        int pos;
-        unsigned e = (unsigned)k | ((unsigned)s << 12);
-        if (v == -2) e = (unsigned)k | kStray32;
-        if (v != -2 && r < kRanks32)
-          pos = base[r * W + (s >> 5)] + __popc(mask[r * W + (s >> 5)] & ((1u << (s & 31)) - 1u));
-        else
-          pos = ranked + atomicAdd(sc, 1);
-        order[pos] = e;
-      }
+      if (lane <= kRanks / 2) sc[16 + lane] = incl - n;
+      if (lane < kRanks / 2) sc[34 + lane] = first;
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
 
-    const int nround = sc[16 + kRanks32 / 2];       // pairs of the ordered ranks
+    const int ranked = sc[33];
+    const int nround = sc[16 + kRanks / 2];       // pairs of the ordered ranks
     const int nitem = nround + (nch - ranked);      // the rest goes one by one
     // ---- gather, push, move ----
     int round = 0;
-    for (int i0 = 0; i0 < nitem; i0 += kPushThreads32) {
+    for (int i0 = 0; i0 < nitem; i0 += kPushThreads) {
       const int i = i0 + tid;
       bool have[2] = {i < nitem, false};
       int pos[2] = {0, 0};
@@ -486,18 +306,16 @@ __global__ void __launch_bounds__(kPushThreads32, 2)
         }
       }
       unsigned ent[2];
-      ent[0] = have[0] ? order[pos[0]] : kStray32;
-      if (have[0] && (ent[0] & kStray32)) {  // dropped with the error bit set
+      ent[0] = have[0] ? order[pos[0]] : kStray;
+      if (have[0] && (ent[0] & kStray)) {  // dropped with the error bit set
         keys[c0 + pos[0]] = -1;
-        order[pos[0]] = ent[0] | kCross32;
+        order[pos[0]] = ent[0] | kCross;
       }
-      have[0] = have[0] && !(ent[0] & kStray32);
+      have[0] = have[0] && !(ent[0] & kStray);
       const int s = (ent[0] >> 12) & 4095;
       if (have[0] && i < nround) {
-        const int w = (2 * round + 1) * W + (s >> 5);
-        const unsigned m = mask[w];
-        have[1] = (m >> (s & 31)) & 1u;
-        pos[1] = base[w] + __popc(m & ((1u << (s & 31)) - 1u));
+        have[1] = (P.mask[(2 * round + 1) * W + (s >> 5)] >> (s & 31)) & 1u;
+        pos[1] = P.position(W, 2 * round + 1, s);
       }
       if (i < nitem) pairB[i] = have[1] ? (unsigned short)pos[1] : (unsigned short)0xffff;
       ent[1] = have[1] ? order[pos[1]] : ent[0];
@@ -560,39 +378,13 @@ __global__ void __launch_bounds__(kPushThreads32, 2)
           }
           pn.w[dst] = p.w[idx[k]];
           if (pn.id) pn.id[dst] = p.id[idx[k]];
-          // the new cell and its tile: a move is at most one cell, across the grid's end to the first or last tile
-          int n0 = x0 + l[0] + dc[0], n1 = y0 + l[1] + dc[1], n2 = z0 + l[2] + dc[2];
-          key[k] = t;
-          if (dc[0] | dc[1] | dc[2]) {
-            n0 = wrapi(n0, g.nx), n1 = wrapi(n1, g.ny), n2 = wrapi(n2, g.nz);
-            if ((unsigned)(n0 - x0) >= (unsigned)tl.tx || (unsigned)(n1 - y0) >= (unsigned)tl.ty ||
-                (unsigned)(n2 - z0) >= (unsigned)tl.tz)
-              key[k] = tile_of(g, tl, n0, n1, n2);
-            order[pos[k]] = ent[k] | kCross32 | ((unsigned)(dc[0] + 1) << 24) | ((unsigned)(dc[1] + 1) << 26) |
-                            ((unsigned)(dc[2] + 1) << 28);
-            cross[atomicAdd(sc + 1, 1)] = (unsigned short)pos[k];
-          }
-          pn.cell[dst] = (n0 * g.ny + n1) * g.nz + n2;
-          if (!g.periodic_x) {
-            int rel = n0 - origin_after;
-            if (rel < 0) rel += g.nx;
-            if (rel < xlo || rel > xhi) key[k] = -1;
-          }
-          // absorbing layers: a particle that leaves the y, z cells [L, n - L) is absorbed
-          if (g.pml && (n1 < g.pml || n1 >= g.ny - g.pml || n2 < g.pml || n2 >= g.nz - g.pml)) key[k] = -1;
-          if (!good) {
-            key[k] = -1;
-            order[pos[k]] = ent[k] | kCross32;
-          }
-          keys[dst] = key[k];
+          key[k] = place_moved(P, g, tl, t, l, dc, good, origin_after, xlo, xhi, pos[k], ent[k], pn.cell + dst,
+                               keys + dst);
           if (key[k] == t) own += 1;
         }
       }
 #pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        const int kk = key[k] == t ? -2 : key[k];
-        if (__any_sync(0xffffffffu, kk >= 0)) warp_count(cnt_next, kk, false, nullptr);
-      }
+      for (int k = 0; k < 2; ++k) count_leaving(cnt_next, key[k], t);
     }
     __syncthreads();
 
@@ -600,13 +392,13 @@ __global__ void __launch_bounds__(kPushThreads32, 2)
     {
       int4* z = reinterpret_cast<int4*>(smem_raw);
       const int n = (int)(so.order / 16);
-      for (int i = tid; i < n; i += kPushThreads32) z[i] = make_int4(0, 0, 0, 0);
+      for (int i = tid; i < n; i += kPushThreads) z[i] = make_int4(0, 0, 0, 0);
     }
     __syncthreads();
     const float third = 1.0f / 3.0f;
     const float jcc[3] = {g.dt * g.dy * g.dz, g.dt * g.dx * g.dz, g.dt * g.dx * g.dy};
     round = 0;
-    for (int i = tid; i < nitem; i += kPushThreads32) {
+    for (int i = tid; i < nitem; i += kPushThreads) {
       int posA;
       if (i < nround) {
         while (i >= sc[17 + round]) ++round;
@@ -617,7 +409,7 @@ __global__ void __launch_bounds__(kPushThreads32, 2)
       const int pb = pairB[i];
       const int pos[2] = {posA, pb == 0xffff ? posA : pb};
       const unsigned ent[2] = {order[pos[0]], order[pos[1]]};
-      const bool dep[2] = {!(ent[0] & kCross32), pb != 0xffff && !(ent[1] & kCross32)};
+      const bool dep[2] = {!(ent[0] & kCross), pb != 0xffff && !(ent[1] & kCross)};
       if (!(dep[0] || dep[1])) continue;
       int r[3];
       L.cell((ent[0] >> 12) & 4095, r);
@@ -640,7 +432,7 @@ __global__ void __launch_bounds__(kPushThreads32, 2)
       for (int d = 0; d < 3; ++d) {  // axes 0, 1, 2 of the arrays: d, e, f
         const int sd = L.sd(d, 5), se = L.se(d, 5), lo = L.part(d, 5);
         unsigned* j = sJ + L.start(d, 5) + (r[0] + 1) * sd + (r[1] + 1) * se + r[2] + 1;  // nodes c-1 .. c+2
-        int P[2][3];
+        int Pi[2][3];
         {
           const float scale = __int_as_float((127 + sc[4 + d]) << 23);
           const float jc = -1.0f / (d == 0 ? jcc[0] : (d == 1 ? jcc[1] : jcc[2]));
@@ -650,8 +442,8 @@ __global__ void __launch_bounds__(kPushThreads32, 2)
           for (int m = 0; m < 3; ++m) {
             run = add2(run, D[0][m]);
             const float2 v = mul2(c, run);
-            P[0][m] = __float2int_rn(v.x);
-            P[1][m] = __float2int_rn(v.y);
+            Pi[0][m] = __float2int_rn(v.x);
+            Pi[1][m] = __float2int_rn(v.y);
           }
         }
         // A(b, c) = S_e (S_f + D_f / 2) + D_e (S_f / 2 + D_f / 3)
@@ -669,7 +461,7 @@ __global__ void __launch_bounds__(kPushThreads32, 2)
             const int A0 = __float2int_rn(A.x), A1 = __float2int_rn(A.y);
 #pragma unroll
             for (int m = 0; m < 3; ++m)
-              add_current(j + m * sd + b * se + c, lo, kHalf28 + (long long)P[0][m] * A0 + (long long)P[1][m] * A1);
+              add_current(j + m * sd + b * se + c, lo, mad_wide(Pi[1][m], A1, mad_wide(Pi[0][m], A0, kHalf28)));
           }
         const int r0 = r[0];
         r[0] = r[1], r[1] = r[2], r[2] = r0;
@@ -683,8 +475,8 @@ __global__ void __launch_bounds__(kPushThreads32, 2)
     }
     // particles that left their cell: 5-node windows where they moved
     const int ncross = sc[1];
-    for (int i = tid; i < ncross; i += kPushThreads32) {
-      const int pos = cross[i];
+    for (int i = tid; i < ncross; i += kPushThreads) {
+      const int pos = P.cross[i];
       const unsigned e = order[pos];
       int r[3], n[3];
       L.cell((e >> 12) & 4095, r);
@@ -712,7 +504,7 @@ __global__ void __launch_bounds__(kPushThreads32, 2)
       for (int d = 0; d < 3; ++d) {
         const int sd = L.sd(d, 5), se = L.se(d, 5), lo = L.part(d, 5);
         unsigned* j = sJ + L.start(d, 5) + r[0] * sd + r[1] * se + r[2];
-        int P[4];
+        int Pi[4];
         {
           const float scale = __int_as_float((127 + sc[4 + d]) << 23);
           const float c = -1.0f / (d == 0 ? jcc[0] : (d == 1 ? jcc[1] : jcc[2])) * qw * scale;
@@ -720,7 +512,7 @@ __global__ void __launch_bounds__(kPushThreads32, 2)
 #pragma unroll
           for (int m = 0; m < 4; ++m) {
             run += D[0][m];
-            P[m] = __float2int_rn(c * run);
+            Pi[m] = __float2int_rn(c * run);
           }
         }
         float ak[5], bk[5];
@@ -738,7 +530,7 @@ __global__ void __launch_bounds__(kPushThreads32, 2)
                 const int A = __float2int_rn(S[1][b] * ak[c] + D[1][b] * bk[c]);
 #pragma unroll
                 for (int m = 0; m < 4; ++m)
-                  if (m < n[0] - 1) add_current(j + m * sd + b * se + c, lo, kHalf28 + (long long)P[m] * A);
+                  if (m < n[0] - 1) add_current(j + m * sd + b * se + c, lo, mad_wide(Pi[m], A, kHalf28));
               }
           }
         const int r0 = r[0], n0 = n[0];
@@ -757,9 +549,9 @@ __global__ void __launch_bounds__(kPushThreads32, 2)
     // flush: a half warp per (x, y) row, the lanes along z
     {
       const int NY = tl.ty + 5, rows = (tl.tx + 5) * NY, NZ = tl.tz + 5;
-      for (int r = tid >> 4; r < rows; r += kPushThreads32 / 16) {
+      for (int r = tid >> 4; r < rows; r += kPushThreads / 16) {
         const int lx = r / NY, ly = r - lx * NY;
-        const int gi0 = tabx[lx] + taby[ly];
+        const int gi0 = P.tabx[lx] + P.taby[ly];
         for (int lz = tid & 15; lz < NZ; lz += 16) {
           const int i3[3] = {lx, ly, lz};
 #pragma unroll
@@ -770,7 +562,7 @@ __global__ void __launch_bounds__(kPushThreads32, 2)
               // T = top 2^21 + low, both exact as floats: one rounding
               const long long T = (long long)(int)hi * 4096 + (long long)(lo - (hi << 12));
               const float v = fmaf((float)(int)(T >> 21), 2097152.0f, (float)(int)(T & 0x1fffff));
-              atomicAdd(f.c[JX + d] + gi0 + tabz[lz], v * __int_as_float((126 - sc[4 + d]) << 23));  // 2^-(kp + 1)
+              atomicAdd(f.c[JX + d] + gi0 + P.tabz[lz], v * __int_as_float((126 - sc[4 + d]) << 23));  // 2^-(kp + 1)
             }
           }
         }
