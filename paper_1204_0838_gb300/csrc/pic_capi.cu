@@ -806,10 +806,25 @@ int pic_create(const pic_grid* g, double dt, const pic_window* w, pic_t** out) {
     h->win_t0 = w->t_start * h->omega0;
   }
   {
-    int t3[3] = {8, 8, 8};
-    const char* ts = std::getenv("PIC_TILE");
-    if (ts) std::sscanf(ts, "%d,%d,%d", &t3[0], &t3[1], &t3[2]);
     const int n3[3] = {h->nx, h->ny, h->nz};
+    int t3[3] = {8, 8, 8};
+    // A grid of few 8x8x8 tiles leaves most of the 152 SMs idle: halve the tile
+    // until there are 1.5 tiles per SM, down to 4x4x4.  FP32 step of 83 k
+    // particles on 49x21x27 cells (84 tiles): 141 us with 8x8x8, 94 with 8x4x4,
+    // 104 with 4x4x4.  Above the line the smaller tile's extra halo costs more
+    // than it gains: FP64 on 128x32x32 (256 tiles) 251 us with 8x8x8, 286 with
+    // 4x8x8.
+    auto tiles = [&]() {
+      long long n = 1;
+      for (int d = 0; d < 3; ++d) n *= (n3[d] + t3[d] - 1) / t3[d];
+      return n;
+    };
+    for (int d = 2; d >= 0 && tiles() < 228; --d) t3[d] = 4;
+    const char* ts = std::getenv("PIC_TILE");
+    if (ts) {
+      t3[0] = t3[1] = t3[2] = 8;
+      std::sscanf(ts, "%d,%d,%d", &t3[0], &t3[1], &t3[2]);
+    }
     for (int d = 0; d < 3; ++d) t3[d] = std::max(1, std::min(t3[d], n3[d]));
     Tiles& tl = h->tiles;
     tl.tx = t3[0];
