@@ -378,8 +378,8 @@ int curl_only(pic_t* h, int i0, int ni) {
 inline bool push_fixed(const Tiles& tl) { return tl.tx <= 8 && tl.ty <= 8 && tl.tz <= 8; }
 
 template <typename T>
-using PushKernel = void (*)(Geom<T>, Tiles, Fields<T>, Parts<T>, Parts<T>, const int*, int, int*, int*, T, T, int, int,
-                            int, unsigned long long*, int*);
+using PushKernel = void (*)(Geom<T>, Tiles, Fields<T>, Parts<T>, Parts<T>, const int*, int, int*, int*, PushCoef<T>, int,
+                            int, int, unsigned long long*, int*);
 template <typename T>
 PushKernel<T> push_kernel(bool fixed);
 template <>
@@ -393,10 +393,18 @@ template <typename T>
 void launch_push(pic_t* h, const Geom<T>& g, int tsi, int origin_after, cudaStream_t s) {
   const Tiles& tl = h->tiles;
   const bool fixed = push_fixed(tl);
+  const double d[3] = {h->dx, h->dy, h->dz};
+  PushCoef<T> pc;
+  pc.h = (T)(h->q * h->dt / (2.0 * h->m));
+  pc.q = (T)h->q;
+  for (int a = 0; a < 3; ++a) {
+    pc.dtd[a] = (T)(h->dt / d[a]);
+    pc.jc[a] = (T)(-1.0 / (h->dt * d[(a + 1) % 3] * d[(a + 2) % 3]));
+  }
   const size_t sm = fixed ? PushSmem::of<T, true>(tl).total : PushSmem::of<T, false>(tl).total;
   push_kernel<T>(fixed)<<<tl.n, kPushThreads, sm, s>>>(
       g, tl, fields<T>(h), parts<T>(h, h->cur), parts<T>(h, 1 - h->cur), h->tstart[tsi], (int)h->capacity, h->keys,
-      h->tcnt, (T)(h->q * h->dt / (2.0 * h->m)), (T)h->q, origin_after, x_lo(h), x_hi(h), h->d_pushed, h->d_ctrl + 2);
+      h->tcnt, pc, origin_after, x_lo(h), x_hi(h), h->d_pushed, h->d_ctrl + 2);
 }
 
 // Counting sort of the current buffer by tile into the other buffer.

@@ -4,79 +4,110 @@
 // component) and the Esirkepov deposit (products of shape-factor sums) of the
 // FP64 push run as integer arithmetic: on this GPU the integer multiply-add
 // pipe retires 32x32->64-bit products many times faster than the FP64 pipe
-// retires FMAs, and a 64-bit integer add into shared memory is a native 32-bit
-// atomic plus a carry, where a double add is a compare-and-swap loop.
+// retires FMAs, and integer adds into shared memory are native, where a double
+// add is a compare-and-swap loop.
 //
-// Formats:
-// - a "value" x is an int64 in units of 2^-k for a scale k chosen per tile
-//   (fields) or per tile and component (current), split centred:
-//   x = hi 2^31 + lo with -2^30 <= lo < 2^30;
-// - a "weight" W is a non-negative int64 below 2^62 holding w 2^62 for
-//   0 <= w < 1 (shape factors, Esirkepov factors), split as
-//   W = hi 2^31 + lo with 0 <= lo < 2^31.
+// A number x is an int64 in units of 2^-k, split centred at 32 bits:
+// x = hi 2^32 + lo with -2^31 <= lo < 2^31.  The product of two,
+//   x y / 2^64 = xh yh + (xh yl + xl yh) / 2^32 + xl yl / 2^64,
+// takes three 32x32->64 multiply-adds into two accumulators; the cross
+// products' sum M is added through its high word, so that a product needs no
+// 64-bit shifts.  The last term is dropped: it
+// is below 1/4 unit and has zero mean, so that sums of thousands of products
+// add up no drift, and a sum of products of zeros is zero.
 //
-// x W / 2^62 = xh Wh + (xh Wl + xl Wh) / 2^31 + xl Wl / 2^62: three 32x32->64
-// multiply-adds into two accumulators (the two cross products share a scale).
-// The last term is dropped; its xl is centred, so that it is below half a unit
-// and has zero mean, and a sum of products of zeros is zero.  Range of the
-// second accumulator: a gather sums 16 products with |x| < 2^58 and weights
-// that sum to at most one, |sum xh Wl| < 16 x 2^27 x 2^31 = 2^62 and
-// |sum xl Wh| <= 2^30 x 2^31; a deposit product has |x| <= 2^62, |xh Wl| < 2^62
-// and |xl Wh| < 2^61; both stay within 2^63.
+// Scales and the range of M (|M| + 2^31 < 2^63):
+// - gather: fields |x| < 2^58 at 2^sF, weights at 2^63 (at most 2/3, products
+//   of two at most 4/9): a sum of 16 has |sum xh wl| < 16 x 2^26 x 2^31 and
+//   |sum xl wh| <= 2^31 x 2^31, since the weights sum to at most one;
+// - deposit factors: S and D = S1 - S of one axis at 2^62, |S| + |D| <= 6/5,
+//   times factors at 2^63 that are at most 2/3 and 1/3:
+//   |M| <= 2^62 (3/5 + 2/3 + 1/3);
+// - current: |P| < 2^63 times A < 1/2 at 2^63: |M| <= 2^62 (1 + 1/2).
 #pragma once
 
 #include <cuda_runtime.h>
 
 namespace pic {
 
-struct S31 {
+struct S32 {
   int hi, lo;
 };
 
-// a b + c, one 32x32->64 multiply-add.  Spelt out: from the C expression the
-// compiler widens operands that it knows to be non-negative and multiplies in
-// 64 bits (16 instructions per acc31 instead of 3).
+// a b + c, one 32x32->64 multiply-add: the pair of a low multiply-add with carry
+// and a high one is one instruction.  (mad.wide in inline assembly becomes a
+// multiply and an add; the C expression is reassociated and, where the compiler
+// knows an operand to be non-negative, widened to 64-bit multiplies.)
 __device__ __forceinline__ long long mad_wide(int a, int b, long long c) {
   long long d;
-  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
+  asm("{ .reg .u32 l, h, m, n; mov.b64 {l, h}, %3; mad.lo.cc.s32 m, %1, %2, l; madc.hi.s32 n, %1, %2, h;"
+      " mov.b64 %0, {m, n}; }"
+      : "=l"(d)
+      : "r"(a), "r"(b), "l"(c));
   return d;
 }
 
-// Centred split of a value; plain split of a weight (>= 0).
-__device__ __forceinline__ S31 split31(long long x) {
-  return {(int)((x + (1LL << 30)) >> 31), ((int)((unsigned)x << 1)) >> 1};
+__device__ __forceinline__ S32 split32(long long x) {
+  return {(int)((unsigned long long)(x + 0x80000000LL) >> 32), (int)x};
 }
-__device__ __forceinline__ S31 splitw(long long W) { return {(int)(W >> 31), (int)(W & 0x7FFFFFFFLL)}; }
 
-struct Acc31 {
+struct Acc32 {
   long long H, M;
 };
-__device__ __forceinline__ Acc31 acc31_init() { return {0LL, 1LL << 30}; }  // rounds the shift
-__device__ __forceinline__ void acc31(Acc31& a, S31 x, S31 w) {
+__device__ __forceinline__ Acc32 acc32_init() { return {0LL, 1LL << 31}; }  // rounds the high word of M
+__device__ __forceinline__ void acc32(Acc32& a, S32 x, S32 w) {
   a.H = mad_wide(x.hi, w.hi, a.H);
   a.M = mad_wide(x.hi, w.lo, a.M);
   a.M = mad_wide(x.lo, w.hi, a.M);
 }
-__device__ __forceinline__ long long acc31_result(const Acc31& a) { return a.H + (a.M >> 31); }
+__device__ __forceinline__ long long acc32_result(const Acc32& a) { return a.H + (a.M >> 32); }
+// Twice the result, with one more bit, for a sum that began at {0, kRound2}.
+constexpr long long kRound2 = 1LL << 30;
+__device__ __forceinline__ long long acc32_result2(const Acc32& a) { return 2 * a.H + (a.M >> 31); }
 
-// x W / 2^62 for one product.
-__device__ __forceinline__ long long mul62(S31 x, S31 w) {
-  Acc31 a = acc31_init();
-  acc31(a, x, w);
-  return acc31_result(a);
+// x w / 2^64 for one product; floor64 without the rounding, for factors whose
+// last unit does not add up.
+__device__ __forceinline__ long long mul64(S32 x, S32 w) {
+  Acc32 a = acc32_init();
+  acc32(a, x, w);
+  return acc32_result(a);
+}
+__device__ __forceinline__ long long floor64(S32 x, S32 w) {
+  Acc32 a = {0LL, 0LL};
+  acc32(a, x, w);
+  return acc32_result(a);
 }
 
-// round(v 2^k) for |v| 2^k < 2^62, from the bit pattern of v (integer
+// round(v 2^k) for |v| 2^k < 2^63, from the bit pattern of v (integer
 // instructions only; zero and subnormal v give 0).
 __device__ __forceinline__ long long to_fixed(double v, int k) {
   const long long b = __double_as_longlong(v);
   const int e = (int)((b >> 52) & 0x7FF);
   const long long m = (b & 0xFFFFFFFFFFFFFLL) | 0x10000000000000LL;
-  const int sh = e - 1075 + k;  // |v| 2^k = m 2^sh, sh <= 9 by the caller's bound
+  const int sh = e - 1075 + k;  // |v| 2^k = m 2^sh, sh <= 10 by the caller's bound
   const int l = max(sh, 0), r = min(max(-sh, 0), 62);
   long long X = ((m << l) + ((1LL << r) >> 1)) >> r;
   X = e == 0 ? 0 : X;
   return b < 0 ? -X : X;
+}
+
+// A staged field value v as round(v 2^k), k = 57 + 1023 - emax for the tile's
+// largest biased exponent emax (below 2047): |v| 2^k < 2^58.
+__device__ __forceinline__ long long field_fixed(long long b, int emax) {
+  const int e = (int)((b >> 52) & 0x7FF);
+  const unsigned long long m = (unsigned long long)(b & 0xFFFFFFFFFFFFFLL) | 0x10000000000000ull;
+  unsigned long long X = (m << 6) >> min(emax - e, 63);  // one bit below the unit
+  X = e == 0 ? 0ull : (X + 1) >> 1;
+  const long long n = b >> 63;
+  return ((long long)X ^ n) - n;
+}
+
+// o 2^63 for 0 <= o < 1 (what falls below 2^-63 is cut off).
+__device__ __forceinline__ long long offset63(double o) {
+  const long long b = __double_as_longlong(o);
+  const int e = (int)(b >> 52);
+  const unsigned long long m = (unsigned long long)(b & 0xFFFFFFFFFFFFFLL) | 0x10000000000000ull;
+  return (long long)((m << 10) >> min(1022 - e, 63));
 }
 
 // 2^k as a double, for -1022 <= k <= 1023.
@@ -94,66 +125,61 @@ __device__ __forceinline__ double fixed_to_double(long long x, int k) {
   return __longlong_as_double(x < 0 ? b | (long long)0x8000000000000000ull : b);
 }
 
-// Cubic B-spline weights at 2^62 of the nodes c-1, c, c+1, c+2 for an offset
-// T / 2^62 in [0, 1): w3 = t^3/6, w1 = 2/3 - t^2 + t^3/2, w2 = 1/6 + (t + t^2 -
-// t^3)/2 (= 2/3 - s^2 + s^3/2 with s = 1 - t), w0 = 1 - w1 - w2 - w3 (= s^3/6):
-// within a few units of 2^-62, and they sum to one.
-__device__ __forceinline__ void spline62(long long T, long long (&w)[4]) {
-  constexpr long long kOne = 1LL << 62, kTwo3 = 3074457345618258603LL, kSixth = 768614336404564651LL;
-  const S31 t = splitw(T);
-  const long long t2 = mad_wide(t.hi, t.hi, mad_wide(t.hi, t.lo, 1LL << 29) >> 30);
-  const long long t3 = mul62(splitw(t2), t);
-  w[3] = mul62(splitw(t3), splitw(kSixth));
-  w[1] = kTwo3 - t2 + (t3 >> 1);
-  w[2] = kSixth + ((T + t2 - t3) >> 1);
-  w[0] = max(kOne - w[1] - w[2] - w[3], 0LL);  // clamps a rounding below zero
+__device__ __forceinline__ S32 third64() { return {0x55555555, 0x55555555}; }  // 1/3 at 2^64
+
+// Cubic B-spline weights at 2^K (62 or 63) of the nodes c-1, c, c+1, c+2 for
+// u = t - 1/2 = U / 2^63, t in [0, 1) the offset in the cell:
+//   w0, w3 = (1/48 + u^2/4) -+ (u/8 + u^3/6), w1, w2 = (23/48 - u^2/4) -+ (5u/8 -
+// u^3/2), the cubic's pieces in even and odd parts.  Within a few units, and
+// they sum to one exactly.
+template <int K>
+__device__ __forceinline__ void spline_fixed(long long U, long long (&w)[4]) {
+  constexpr long long kOne48 = K == 63 ? 192153584101141163LL : 96076792050570581LL;  // 2^K / 48
+  constexpr long long k23_48 = (1LL << (K - 1)) - kOne48;
+  constexpr int sh = 63 - K;
+  const S32 u = split32(U);
+  const long long q = floor64(u, u);                       // u^2 at 2^62
+  const long long c = floor64(u, split32(q));              // u^3 at 2^61
+  const long long c3 = floor64(split32(c), third64());     // u^3 / 3 at 2^61
+  const long long e = q >> (sh + 1), u3 = U >> (3 + sh);   // u^2 / 4, u / 8 at 2^K
+  const long long e0 = kOne48 + e, e1 = k23_48 - e;
+  const long long o0 = u3 + (sh ? c3 : 2 * c3);
+  const long long o1 = u3 + (U >> (1 + sh)) - (sh ? c : 2 * c);
+  w[0] = e0 - o0;
+  w[1] = e1 - o1;
+  w[2] = e1 + o1;
+  w[3] = e0 + o0;
 }
-__device__ __forceinline__ void spline62(long long T, S31 (&w)[4]) {
+__device__ __forceinline__ void spline63(long long U, S32 (&w)[4]) {
   long long v[4];
-  spline62(T, v);
+  spline_fixed<63>(U, v);
 #pragma unroll
-  for (int k = 0; k < 4; ++k) w[k] = splitw(v[k]);
+  for (int k = 0; k < 4; ++k) w[k] = split32(v[k]);
 }
+constexpr long long kHalf63 = 1LL << 62;  // 1/2 at 2^63
 
-// S / 2 + D / 3 = ((3 S + 2 D) / 2) / 3 for weights S and S + D (the sum of up
-// to 3 x 2^62 is formed unsigned).
-__device__ __forceinline__ long long third62(long long S, long long D) {
-  constexpr long long kThird = 1537228672809129301LL;
-  const unsigned long long v = 3ull * (unsigned long long)S + 2ull * (unsigned long long)D;
-  return mul62(splitw((long long)(v >> 1)), splitw(kThird));
-}
-
-// Sum over 4x4x4 nodes of a staged component (split words), weights wde over
-// the first two axes and wf over the last.
-__device__ __forceinline__ long long gather64(const int2* __restrict__ s, int sd, int se, const S31 (&wde)[4][4],
-                                              const S31 (&wf)[4]) {
-  Acc31 sum = acc31_init();
+// Sum over 4x4x4 nodes of a staged component (split words at 2^sF), weights wde
+// over the first two axes and wf over the last, both at 2^63: at 2^sF.
+__device__ __forceinline__ long long gather64(const int2* __restrict__ s, int sd, int se, const S32 (&wde)[4][4],
+                                              const S32 (&wf)[4]) {
+  Acc32 sum = {0LL, kRound2};
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
-    Acc31 a = acc31_init();
+    // the two cross sums apart: three chains of multiply-adds instead of two
+    long long H = 0, M = kRound2, N = 0;
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const int2 v = s[i * sd + j * se + c];
-        acc31(a, {v.y, v.x}, wde[i][j]);
+        H = mad_wide(v.y, wde[i][j].hi, H);
+        M = mad_wide(v.y, wde[i][j].lo, M);
+        N = mad_wide(v.x, wde[i][j].hi, N);
       }
-    acc31(sum, split31(acc31_result(a)), wf[c]);
+    const Acc32 a = {H, M + N};
+    acc32(sum, split32(acc32_result2(a)), wf[c]);
   }
-  return acc31_result(sum);
-}
-
-__device__ __forceinline__ unsigned atom_add_u32_shared(unsigned* a, unsigned v) {
-  unsigned old;
-  asm volatile("atom.shared.add.u32 %0, [%1], %2;"
-               : "=r"(old)
-               : "r"((unsigned)__cvta_generic_to_shared(a)), "r"(v)
-               : "memory");
-  return old;
-}
-
-__device__ __forceinline__ void red_add_u32_shared(unsigned* a, unsigned v) {
-  asm volatile("red.shared.add.u32 [%0], %1;" ::"r"((unsigned)__cvta_generic_to_shared(a)), "r"(v) : "memory");
+  return acc32_result2(sum);
 }
 
 }  // namespace pic

@@ -27,12 +27,13 @@ constexpr unsigned kStray = 1u << 30;  // outside the tile: dropped, error bit s
 // [i_d][i_e][i_f] with (e, f) the axes after d in cyclic order, so that one
 // body serves the three rotations with the same offsets (three unrolled bodies
 // overflow the instruction cache): two field components per d, in T or 64-bit
-// words, and J as [d][hi, lo] in 32-bit words.  FIXED: tiles of up to 8 cells
-// per axis, strides known to the compiler; otherwise any tile.  The fixed
-// strides keep a warp on 4x8 neighbouring cells within two wavefronts per
-// 32-bit access, one for one of the three rotations (12 and 17 modulo 32 for
-// the fields, 13 and 12 modulo 32 for J), and within 4.3 of the 2 that a 64-bit
-// access needs when the lanes start at either half cell (12 and 9 modulo 16).
+// words, and J as [d][words of a sum] in 32-bit words (FP32 2, FP64 3).  FIXED:
+// tiles of up to 8 cells per axis, strides known to the compiler; otherwise any tile.  The fixed
+// strides are the best of a search over shapes of a warp's 32 cells and pitches:
+// 1x8x4 cells (slot order) read 32-bit fields and add to J in 1, 2 and 1 (fields)
+// or 2, 1 and 1 (J) wavefronts for the three rotations, and read 64-bit fields,
+// where each lane starts at its own half cell, in 1.72 per half warp (linear
+// cell order with one pitch: 5/3 and 2.13).
 template <typename T, bool FIXED>
 struct PushLayout {
   int t[3];
@@ -40,23 +41,31 @@ struct PushLayout {
   // pad = 4: staged fields, 5: J
   __host__ __device__ __forceinline__ int se(int d, int pad) const { return FIXED ? 8 + pad : t[(d + 2) % 3] + pad; }
   __host__ __device__ __forceinline__ int sd(int d, int pad) const {
-    return FIXED ? (pad == 4 ? (sizeof(T) == 8 ? 153 : 145) : 172) : (t[(d + 1) % 3] + pad) * se(d, pad);
+    if (!FIXED) return (t[(d + 1) % 3] + pad) * se(d, pad);
+    if (pad == 5) return d == 0 ? 169 : (d == 1 ? 172 : 184);
+    return d == 0 ? 144 : (sizeof(T) == 8 ? (d == 1 ? 149 : 148) : (d == 1 ? 145 : 152));
   }
   __host__ __device__ __forceinline__ int part(int d, int pad) const {
     return FIXED ? (8 + pad) * sd(d, pad) : (t[d] + pad) * sd(d, pad);
   }
-  __host__ __device__ __forceinline__ int start(int d, int pad) const { return FIXED ? 2 * d * part(0, pad) : 2 * d * part(d, pad); }
-  __host__ __device__ int region(int pad) const { return 6 * part(0, pad); }
-  // cell slots: a warp's 32 are 4x8 cells (fixed) or consecutive cells
+  static constexpr int kJWords = sizeof(T) == 8 ? 3 : 2;
+  __host__ __device__ __forceinline__ int start(int d, int pad) const {
+    const int n = pad == 4 ? 2 : kJWords;
+    return d == 0 ? 0 : n * (part(0, pad) + (d == 1 ? 0 : part(1, pad)));
+  }
+  __host__ __device__ int region(int pad) const {
+    return (pad == 4 ? 2 : kJWords) * (part(0, pad) + part(1, pad) + part(2, pad));
+  }
+  // cell slots: a warp's 32 are 1x8x4 cells (fixed) or consecutive cells
   __host__ __device__ int words() const { return FIXED ? 2 * t[0] : (t[0] * t[1] * t[2] + 31) / 32; }
   __device__ __forceinline__ int slot(int lx, int ly, int lz) const {
-    return FIXED ? lx * 64 + ly * 8 + lz : (lx * t[1] + ly) * t[2] + lz;
+    return FIXED ? (lx * 2 + (lz >> 2)) * 32 + ly * 4 + (lz & 3) : (lx * t[1] + ly) * t[2] + lz;
   }
   __device__ __forceinline__ void cell(int s, int (&l)[3]) const {
     if (FIXED) {
       l[0] = s >> 6;
-      l[1] = (s >> 3) & 7;
-      l[2] = s & 7;
+      l[1] = (s >> 2) & 7;
+      l[2] = ((s >> 3) & 4) | (s & 3);
     } else {
       l[0] = s / (t[1] * t[2]);
       const int r = s - l[0] * t[1] * t[2];
@@ -160,6 +169,37 @@ __device__ __forceinline__ void rank_clear(const PushTile& P, int W) {
 }
 
 constexpr int kPerThread = kChunk / kPushThreads;
+
+// Constants of a push that cost divisions, formed on the host.
+template <typename T>
+struct PushCoef {
+  T h;       // q dt / (2 m)
+  T q;
+  T dtd[3];  // dt / d
+  T jc[3];   // -1 / (dt d_e d_f)
+};
+
+__device__ __forceinline__ void prefetch_l1(const void* p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
+
+// The (x, y) rows of a halo of ny rows per slab that a half warp takes, 16 rows
+// apart: no division per row.
+struct RowWalk {
+  int lx, ly, ny, qx, qy;
+  __device__ __forceinline__ explicit RowWalk(int n) : ny(n), qx(16 / n), qy(16 % n) {
+    const int r = threadIdx.x >> 4;
+    lx = r / n;
+    ly = r % n;
+  }
+  __device__ __forceinline__ void next() {
+    lx += qx;
+    ly += qy;
+    if (ly >= ny) {
+      ly -= ny;
+      lx += 1;
+    }
+  }
+};
+static_assert(kPushThreads == 256, "RowWalk: 16 half warps");
 
 // Count the pass's particles [c0, c0 + nch) per cell: sr[] = slot and rank of
 // this thread's particles (-2: outside the tile).  A barrier must follow.

@@ -188,7 +188,7 @@ template <bool FIXED>
 __global__ void __launch_bounds__(kPushThreads, 2)
     k_push32(Geom<float> g, Tiles tl, Fields<float> f, Parts<float> p, Parts<float> pn,
              const int* __restrict__ tstart, int capacity, int* __restrict__ keys, int* __restrict__ cnt_next,
-             float h, float q, int origin_after, int xlo, int xhi, unsigned long long* pushed, int* err) {
+             PushCoef<float> pc, int origin_after, int xlo, int xhi, unsigned long long* pushed, int* err) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (g.dyn) origin_after = g.dyn->origin_after;
   const int t = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
@@ -209,7 +209,6 @@ __global__ void __launch_bounds__(kPushThreads, 2)
     if (ntile >= (1 << 20)) atomicOr(err, 16);
   }
   const int npass = (ntile + kChunk - 1) / kChunk, per_pass = (ntile + npass - 1) / npass;
-  const float dtd[3] = {g.dt / g.dx, g.dt / g.dy, g.dt / g.dz};
   int own = 0;
 
   for (int ch0 = 0; ch0 < ntile; ch0 += per_pass) {
@@ -219,9 +218,9 @@ __global__ void __launch_bounds__(kPushThreads, 2)
 
     // stage E, B: a half warp per (x, y) row, the lanes along z
     {
-      const int SY = tl.ty + 4, rows = (tl.tx + 4) * SY, SZ = tl.tz + 4;
-      for (int r = tid >> 4; r < rows; r += kPushThreads / 16) {
-        const int lx = r / SY, ly = r - lx * SY;
+      const int SX = tl.tx + 4, SZ = tl.tz + 4;
+      for (RowWalk r(tl.ty + 4); r.lx < SX; r.next()) {
+        const int lx = r.lx, ly = r.ly;
         const int gi0 = P.tabx[lx] + P.taby[ly];
         for (int lz = tid & 15; lz < SZ; lz += 16) {
           const int gi = gi0 + P.tabz[lz];
@@ -263,9 +262,8 @@ __global__ void __launch_bounds__(kPushThreads, 2)
     rank_masks(P, W);
     if (tid < 3) {
       // kp: |P| 2^kp < 2^31 for P <= 0.76 |q| max w jc, and B 2^(kp + 1) < 2^42
-      const float jcc = tid == 0 ? g.dt * g.dy * g.dz : (tid == 1 ? g.dt * g.dx * g.dz : g.dt * g.dx * g.dy);
-      const float Pm = 0.76f * fabsf(q) * __int_as_float(sc[3]) / jcc;
-      const float B = 1.001f * fabsf(q) * __int_as_float(sc[2]) / jcc;
+      const float jc = fabsf(pc.q * (tid == 0 ? pc.jc[0] : (tid == 1 ? pc.jc[1] : pc.jc[2])));
+      const float Pm = 0.76f * jc * __int_as_float(sc[3]), B = 1.001f * jc * __int_as_float(sc[2]);
       const int ep = ((__float_as_int(Pm) >> 23) & 255) - 127, eb = ((__float_as_int(B) >> 23) & 255) - 127;
       sc[4 + tid] = B > 0.0f ? max(min(min(30 - ep, 40 - eb), 120), -120) : 0;
     }
@@ -325,6 +323,11 @@ __global__ void __launch_bounds__(kPushThreads, 2)
         L.cell(s, l);
         const int idx[2] = {c0 + (int)(ent[0] & 4095), c0 + (int)(ent[1] & 4095)};
         float2 u[3], E[3], B[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {  // for after the gather
+          prefetch_l1(p.u[d] + idx[0]);
+          prefetch_l1(p.u[d] + idx[1]);
+        }
         {
           float2 wn[3][4], wh[3][5];
 #pragma unroll
@@ -355,7 +358,7 @@ __global__ void __launch_bounds__(kPushThreads, 2)
         }
 #pragma unroll
         for (int d = 0; d < 3; ++d) u[d] = make_float2(p.u[d][idx[0]], p.u[d][idx[1]]);
-        const float2 ig = boris32(h, E, B, u);
+        const float2 ig = boris32(pc.h, E, B, u);
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
           if (k == 1 && !have[1]) break;
@@ -372,7 +375,7 @@ __global__ void __launch_bounds__(kPushThreads, 2)
           for (int d = 0; d < 3; ++d) {
             const float o = p.o[d][idx[k]];
             float o1;
-            dc[d] = step32(good ? o + dtd[d] * uk[d] * igk : o, o1);
+            dc[d] = step32(good ? o + pc.dtd[d] * uk[d] * igk : o, o1);
             pn.o[d][dst] = o1;
             pn.u[d][dst] = uk[d];
           }
@@ -396,7 +399,6 @@ __global__ void __launch_bounds__(kPushThreads, 2)
     }
     __syncthreads();
     const float third = 1.0f / 3.0f;
-    const float jcc[3] = {g.dt * g.dy * g.dz, g.dt * g.dx * g.dz, g.dt * g.dx * g.dy};
     round = 0;
     for (int i = tid; i < nitem; i += kPushThreads) {
       int posA;
@@ -416,7 +418,7 @@ __global__ void __launch_bounds__(kPushThreads, 2)
       float2 S[3][4], D[3][4], qw;
       {
         const int i0 = c0 + (int)(ent[0] & 4095), i1 = c0 + (int)(ent[1] & 4095), d0 = c0 + pos[0], d1 = c0 + pos[1];
-        qw = make_float2(dep[0] ? q * p.w[i0] : 0.0f, dep[1] ? q * p.w[i1] : 0.0f);
+        qw = make_float2(dep[0] ? pc.q * p.w[i0] : 0.0f, dep[1] ? pc.q * p.w[i1] : 0.0f);
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
           const float2 a = make_float2(p.o[d][i0], p.o[d][i1]);
@@ -435,7 +437,7 @@ __global__ void __launch_bounds__(kPushThreads, 2)
         int Pi[2][3];
         {
           const float scale = __int_as_float((127 + sc[4 + d]) << 23);
-          const float jc = -1.0f / (d == 0 ? jcc[0] : (d == 1 ? jcc[1] : jcc[2]));
+          const float jc = d == 0 ? pc.jc[0] : (d == 1 ? pc.jc[1] : pc.jc[2]);
           const float2 c = mul2(mul2(dup2(jc), qw), dup2(scale));
           float2 run = make_float2(0.0f, 0.0f);
 #pragma unroll
@@ -481,7 +483,7 @@ __global__ void __launch_bounds__(kPushThreads, 2)
       int r[3], n[3];
       L.cell((e >> 12) & 4095, r);
       const int idx = c0 + (int)(e & 4095), dst = c0 + pos;
-      const float qw = q * p.w[idx];
+      const float qw = pc.q * p.w[idx];
       float S[3][5], D[3][5];
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
@@ -507,7 +509,7 @@ __global__ void __launch_bounds__(kPushThreads, 2)
         int Pi[4];
         {
           const float scale = __int_as_float((127 + sc[4 + d]) << 23);
-          const float c = -1.0f / (d == 0 ? jcc[0] : (d == 1 ? jcc[1] : jcc[2])) * qw * scale;
+          const float c = (d == 0 ? pc.jc[0] : (d == 1 ? pc.jc[1] : pc.jc[2])) * qw * scale;
           float run = 0.0f;
 #pragma unroll
           for (int m = 0; m < 4; ++m) {
@@ -548,9 +550,9 @@ __global__ void __launch_bounds__(kPushThreads, 2)
 
     // flush: a half warp per (x, y) row, the lanes along z
     {
-      const int NY = tl.ty + 5, rows = (tl.tx + 5) * NY, NZ = tl.tz + 5;
-      for (int r = tid >> 4; r < rows; r += kPushThreads / 16) {
-        const int lx = r / NY, ly = r - lx * NY;
+      const int NX = tl.tx + 5, NZ = tl.tz + 5;
+      for (RowWalk r(tl.ty + 5); r.lx < NX; r.next()) {
+        const int lx = r.lx, ly = r.ly;
         const int gi0 = P.tabx[lx] + P.taby[ly];
         for (int lz = tid & 15; lz < NZ; lz += 16) {
           const int i3[3] = {lx, ly, lz};

@@ -11,22 +11,25 @@
 // What bounded the one-pass kernel that this replaces: instructions, about
 // 20,000 per particle, issued 36 % of the time (16 warps per SM, waits for
 // instructions and for the shared-memory adds' returns).  What changed:
-// - one 32x32->64 multiply-add per product, spelt out (mad_wide), and values
-//   split at 31 bits, so that the two cross products share an accumulator;
+// - one instruction per 32x32->64 product (mad_wide: from the plain expression
+//   the compiler made 16 of 3) and centred splits at 32 bits, whose products
+//   need no 64-bit shifts;
 // - the weights of two axes are multiplied once for the two components that
 //   share them (E_d and B_e), and the gather then sums 16 products per node of
-//   the third axis: 96 products of weights and 408 of values, from 504;
-// - the shape factors are formed in fixed point: 130 FP64 instructions per
+//   the third axis: 48 products of weights and 408 of values, from 504;
+// - the shape factors are formed in fixed point: 90 FP64 instructions per
 //   particle, from 230;
 // - particles that stay in their cell (4-node windows) deposit apart from those
 //   that leave it (5-node windows), which made every warp run the wide loops;
-// - the lanes of a warp hold neighbouring cells, and the returns of a node
-//   column's adds are waited for together.
+// - a current word pair with a carry became three overlapping words added by
+//   reductions that return nothing.
 //
 // Measured (whole step, before -> after): 118 M particles, 1536x256x256 cells
-// 183 -> 113 ms; 7 M, 384x96x96 10.6 -> 6.4 ms; 126 k, 128x32x32 0.368 ->
-// 0.251 ms.  Issue is active 42 % of cycles, the integer ALU 43 %, the FP64 pipe
-// 25 %; the top stalls are fixed latencies and the adds' returns.
+// 183 -> 93 ms; 7 M, 384x96x96 10.6 -> 5.26 ms; 436 k at random places 0.97 ->
+// 0.62 ms.  About 9,000 instructions per particle, issued 43 % of the time; the
+// gather takes 42 % of the kernel, the ordered deposit 32 %, particles that left
+// their cell 6 %, the flush 4 %; no pipe is above a third (integer ALU, FMA,
+// FP64) and shared memory is at 45 %: fixed latencies at 16 warps per SM bound it.
 #pragma once
 
 #include "pic_push.cuh"
@@ -34,7 +37,8 @@
 namespace pic {
 
 constexpr int kField64Range = 58;  // staged fields: 16-term sums need |x| < 2^58
-constexpr int kJ64Range = 62;      // J sums of single products
+constexpr int kFieldExpMin = 80;   // smallest biased exponent that sets a scale (sF <= 1000)
+constexpr int kJ64Range = 62;      // J sums
 
 // Scale exponent of the J tile for component c: B 2^s < 2^62 with B = 1.001 |q|
 // S / (dt d_b d_c), S a bound on sum |w| |running sum|.  A particle moves at
@@ -42,37 +46,40 @@ constexpr int kJ64Range = 62;      // J sums of single products
 // rotation keeps |u|), and a running sum of the deposit changes by at most 3/4
 // of the move (the slope bound of the cubic spline's partial sums); 2^-20
 // covers the rounding.  su = sum |w| min(1, |u|), sw = sum |w|, kick >= 2 |h| |E|.
-__device__ __forceinline__ int j64_scale(const Geom<double>& g, double q, int c, float su, float sw, float kick) {
-  const float dtd = (float)(g.dt / (c == 0 ? g.dx : (c == 1 ? g.dy : g.dz)));
+__device__ __forceinline__ int j64_scale(const PushCoef<double>& pc, int c, float su, float sw, float kick) {
+  const float dtd = (float)(c == 0 ? pc.dtd[0] : (c == 1 ? pc.dtd[1] : pc.dtd[2]));
   const float S = 0.75f * (dtd * fminf(su + kick * sw, sw) + 0x1p-20f * sw);
-  const double jcc = c == 0 ? g.dt * g.dy * g.dz : (c == 1 ? g.dt * g.dx * g.dz : g.dt * g.dx * g.dy);
-  const float B = 1.001f * fabsf((float)q) * S / (float)jcc;
+  const float B = 1.001f * fabsf((float)pc.q) * S * fabsf((float)(c == 0 ? pc.jc[0] : (c == 1 ? pc.jc[1] : pc.jc[2])));
   const int eb = ((__float_as_int(B) >> 23) & 255) - 127;  // B in [2^eb, 2^(eb+1))
   return B > 0.0f ? kJ64Range - 1 - eb : 0;
 }
 
-// Exact 64-bit adds of X[0 .. N) into the shared word pairs at lo + m stride
-// (hi words hi_off further): the low words' adds return the old values, which
-// give the carries; the N returns are waited for together.
-template <int N>
-__device__ __forceinline__ void add_current64(unsigned* hi, int lo_off, int stride, const long long (&X)[N], int n) {
-  unsigned old[N];
-#pragma unroll
-  for (int m = 0; m < N; ++m)
-    if (m < n) old[m] = atom_add_u32_shared(hi + lo_off + m * stride, (unsigned)X[m]);
-#pragma unroll
-  for (int m = 0; m < N; ++m)
-    if (m < n) {
-      const unsigned l = (unsigned)X[m], h = (unsigned)((unsigned long long)X[m] >> 32);
-      red_add_u32_shared(hi + m * stride, h + (old[m] + l < l ? 1u : 0u));
-    }
+// Exact 64-bit add of X as three overlapping words, X mod 2^32, X >> 20 and
+// X >> 40 mod 2^32, by reductions that return nothing (an add of two words
+// waits for the low word's old value to form the carry).
+__device__ __forceinline__ void add_current64(unsigned* j, int part, long long X) {
+  const unsigned l = (unsigned)X, h = (unsigned)((unsigned long long)X >> 32);
+  red_u32(j, l);
+  red_u32(j + part, __funnelshift_r(l, h, 20));
+  red_u32(j + 2 * part, (unsigned)((int)h >> 8));
 }
+
+// The sum of X from the words' sums of up to 3072 adds: sum (X >> 40) is exact
+// (the sum itself is below 2^62); sum (X >> 20) lies within n 2^20 < 2^32 above
+// 2^20 times it, and sum X within n 2^20 above 2^20 times that.
+__device__ __forceinline__ long long sum_current64(unsigned w0, unsigned w1, unsigned w2) {
+  const long long a = (long long)(int)w2 << 20;
+  const long long b = a + (long long)(w1 - (unsigned)a);
+  const long long c = b << 20;
+  return c + (long long)(w0 - (unsigned)c);
+}
+static_assert(kChunk < 4096, "the words' overlap holds the carries of 2^12 adds");
 
 template <bool FIXED>
 __global__ void __launch_bounds__(kPushThreads, 2)
     k_push64(Geom<double> g, Tiles tl, Fields<double> f, Parts<double> p, Parts<double> pn,
              const int* __restrict__ tstart, int capacity, int* __restrict__ keys, int* __restrict__ cnt_next,
-             double h, double q, int origin_after, int xlo, int xhi, unsigned long long* pushed, int* err) {
+             PushCoef<double> pc, int origin_after, int xlo, int xhi, unsigned long long* pushed, int* err) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (g.dyn) origin_after = g.dyn->origin_after;
   const int t = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
@@ -98,11 +105,11 @@ __global__ void __launch_bounds__(kPushThreads, 2)
 
     // Stage E_d (part 0) and B_e, e the axis after d (part 1): a half warp per
     // (x, y) row, the lanes along z; take the largest exponent of each.
-    const int SY = tl.ty + 4, rows = (tl.tx + 4) * SY, SZ = tl.tz + 4;
+    const int SX = tl.tx + 4, SZ = tl.tz + 4;
     {
       int emax[6] = {0, 0, 0, 0, 0, 0};
-      for (int r = tid >> 4; r < rows; r += kPushThreads / 16) {
-        const int lx = r / SY, ly = r - lx * SY;
+      for (RowWalk r(tl.ty + 4); r.lx < SX; r.next()) {
+        const int lx = r.lx, ly = r.ly;
         const int gi0 = P.tabx[lx] + P.taby[ly];
         for (int lz = tid & 15; lz < SZ; lz += 16) {
           const int gi = gi0 + P.tabz[lz];
@@ -153,24 +160,24 @@ __global__ void __launch_bounds__(kPushThreads, 2)
     if (tid < 3) {
       // |E| <= sqrt 3 max_c |E_c| < sqrt 3 2^(emax - 1022)
       const int eE = max(max(sc[50], sc[52]), sc[54]);
-      const float kick = eE == 0 ? 0.0f : ldexpf(3.4642f * fabsf((float)h), eE - 1022);
-      sc[4 + tid] = j64_scale(g, q, tid, __int_as_float(sc[2]), __int_as_float(sc[3]), kick);
+      const float kick = eE == 0 ? 0.0f : ldexpf(3.4642f * fabsf((float)pc.h), eE - 1022);
+      sc[4 + tid] = j64_scale(pc, tid, __int_as_float(sc[2]), __int_as_float(sc[3]), kick);
     }
     if (tid < 6) {
-      // max|F| 2^sF < 2^58; an all-zero component takes sF = 1000; a non-finite value is reported
+      // max|F| 2^sF < 2^58; a non-finite value is reported
       const int e = sc[50 + tid];
       if (e == 0x7FF) atomicOr(err, 8);
-      sc[56 + tid] = e == 0 ? 1000 : min(kField64Range - 1 - (e - 1023), 1000);
+      sc[56 + tid] = kField64Range - 1 - (max(e, kFieldExpMin) - 1023);
     }
     __syncthreads();
     rank_order(P, W, nch, sr);
     {
       // the staged doubles become split fixed-point words in place
-      int k58[6];
+      int emax[6];
 #pragma unroll
-      for (int k = 0; k < 6; ++k) k58[k] = sc[56 + k];
-      for (int r = tid >> 4; r < rows; r += kPushThreads / 16) {
-        const int lx = r / SY, ly = r - lx * SY;
+      for (int k = 0; k < 6; ++k) emax[k] = max(sc[50 + k], kFieldExpMin);
+      for (RowWalk r(tl.ty + 4); r.lx < SX; r.next()) {
+        const int lx = r.lx, ly = r.ly;
         for (int lz = tid & 15; lz < SZ; lz += 16) {
           const int i3[3] = {lx, ly, lz};
 #pragma unroll
@@ -178,7 +185,7 @@ __global__ void __launch_bounds__(kPushThreads, 2)
             const int d = k >> 1;
             long long* w = sF + L.start(d, 4) + (k & 1) * L.part(d, 4) + i3[d] * L.sd(d, 4) +
                            i3[(d + 1) % 3] * L.se(d, 4) + i3[(d + 2) % 3];
-            const S31 x = split31(to_fixed(__longlong_as_double(*w), k58[k]));
+            const S32 x = split32(field_fixed(*w, emax[k]));
             *reinterpret_cast<int2*>(w) = make_int2(x.lo, x.hi);
           }
         }
@@ -187,7 +194,6 @@ __global__ void __launch_bounds__(kPushThreads, 2)
     __syncthreads();
 
     // ---- gather, push, move ----
-    const double dtd[3] = {g.dt / g.dx, g.dt / g.dy, g.dt / g.dz};
     for (int i0 = 0; i0 < nch; i0 += kPushThreads) {
       const int pos = i0 + tid;
       bool have = pos < nch;
@@ -203,48 +209,55 @@ __global__ void __launch_bounds__(kPushThreads, 2)
         L.cell((ent >> 12) & 4095, l);
         const int idx = c0 + (int)(ent & 4095), dst = c0 + pos;
         double E[3], B[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) prefetch_l1(p.u[d] + idx);  // for after the gather
         {
-          S31 wn[3][4], wh[3][4];
-          int r[3], hs[3];  // cell and half-node start (0: c-2, 1: c-1) per axis
+          long long T[3];  // offsets at 2^63
+          int r[3];
 #pragma unroll
           for (int d = 0; d < 3; ++d) {
-            const long long T = to_fixed(p.o[d][idx], 62);
-            const bool low = T < (1LL << 61);
-            spline62(T, wn[d]);
-            spline62(low ? T + (1LL << 61) : T - (1LL << 61), wh[d]);
+            T[d] = offset63(p.o[d][idx]);
             r[d] = l[d];
-            hs[d] = low ? 0 : 1;
           }
+          // Axes 0, 1, 2 of the arrays: d, e, f.  E_d sits on half nodes of d and
+          // nodes of e, f; B_e on half nodes of d and f and nodes of e: the two
+          // share the weights of (d, e).  The weights are formed again for every
+          // rotation: kept, they would fill the registers.
 #pragma unroll 1
-          for (int d = 0; d < 3; ++d) {  // axes 0, 1, 2 of the arrays: d, e, f
-            // E_d sits on half nodes of d and nodes of e, f; B_e on half nodes
-            // of d and f and nodes of e: the two share the weights of (d, e)
+          for (int d = 0; d < 3; ++d) {
             const int sd = L.sd(d, 4), se = L.se(d, 4);
-            const int2* b = reinterpret_cast<const int2*>(sF) + L.start(d, 4) + (r[0] + hs[0]) * sd + (r[1] + 1) * se + r[2];
-            S31 wde[4][4];
+            // half nodes see the offset t + 1/2 from c-2 (t < 1/2) or t - 1/2 from c-1: u = t or t - 1
+            const bool low0 = T[0] < kHalf63, low2 = T[2] < kHalf63;
+            const int2* b = reinterpret_cast<const int2*>(sF) + L.start(d, 4) + (r[0] + (low0 ? 0 : 1)) * sd +
+                            (r[1] + 1) * se + r[2];
+            S32 wde[4][4], wf[4];
+            {
+              S32 wd[4], we[4];
+              spline63(low0 ? T[0] : T[0] - kHalf63 - kHalf63, wd);
+              spline63(T[1] - kHalf63, we);
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+              for (int i = 0; i < 4; ++i)
 #pragma unroll
-              for (int j = 0; j < 4; ++j) wde[i][j] = splitw(mul62(wh[0][i], wn[1][j]));
-            const double e = fixed_to_double(gather64(b + 1, sd, se, wde, wn[2]), sc[56 + 2 * d]);
-            const double m = fixed_to_double(gather64(b + L.part(d, 4) + hs[2], sd, se, wde, wh[2]), sc[57 + 2 * d]);
-            E[0] = E[1], E[1] = E[2], E[2] = e;
-            B[1] = B[2], B[2] = B[0], B[0] = m;  // after three turns: B_y, B_z, B_x came in that order
-            const int r0 = r[0], h0 = hs[0];
-            r[0] = r[1], r[1] = r[2], r[2] = r0;
-            hs[0] = hs[1], hs[1] = hs[2], hs[2] = h0;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const S31 v = wn[0][k], w = wh[0][k];
-              wn[0][k] = wn[1][k], wn[1][k] = wn[2][k], wn[2][k] = v;
-              wh[0][k] = wh[1][k], wh[1][k] = wh[2][k], wh[2][k] = w;
+                for (int j = 0; j < 4; ++j) wde[i][j] = split32(2 * floor64(wd[i], we[j]));
             }
+            spline63(T[2] - kHalf63, wf);
+            const double e = fixed_to_double(gather64(b + 1, sd, se, wde, wf), sc[56 + 2 * d]);
+            spline63(low2 ? T[2] : T[2] - kHalf63 - kHalf63, wf);
+            const double m =
+                fixed_to_double(gather64(b + L.part(d, 4) + (low2 ? 0 : 1), sd, se, wde, wf), sc[57 + 2 * d]);
+            E[0] = E[1], E[1] = E[2], E[2] = e;
+            B[1] = B[2], B[2] = B[0], B[0] = m;  // B_y, B_z, B_x come in this order
+            const int r0 = r[0];
+            r[0] = r[1], r[1] = r[2], r[2] = r0;
+            const long long t0 = T[0];
+            T[0] = T[1], T[1] = T[2], T[2] = t0;
           }
         }
         double u[3];
 #pragma unroll
         for (int d = 0; d < 3; ++d) u[d] = p.u[d][idx];
         // relativistic Boris push
+        const double h = pc.h;
         double um[3], tv[3], sv[3];
 #pragma unroll
         for (int d = 0; d < 3; ++d) um[d] = u[d] + h * E[d];
@@ -270,7 +283,7 @@ __global__ void __launch_bounds__(kPushThreads, 2)
         int dc[3];
 #pragma unroll
         for (int d = 0; d < 3; ++d) {  // |move| < 1 cell per axis
-          double o = p.o[d][idx] + dtd[d] * u[d] * ig;
+          double o = p.o[d][idx] + pc.dtd[d] * u[d] * ig;
           int k = 0;
           if (lt_zero(o)) {
             o += 1.0;
@@ -303,21 +316,29 @@ __global__ void __launch_bounds__(kPushThreads, 2)
       for (int i = tid; i < n; i += kPushThreads) z[i] = make_int4(0, 0, 0, 0);
     }
     __syncthreads();
-    // P 2^s = q w jc run 2^s, below 2^62 by the choice of the scale; run at 2^62
-    const double jc[3] = {-1.0 / (g.dt * g.dy * g.dz), -1.0 / (g.dt * g.dx * g.dz), -1.0 / (g.dt * g.dx * g.dy)};
+    // 2 P 2^s = 2 q w jc run 2^s, below 2^63 by the choice of the scale; run at 2^62
     for (int pos = tid; pos < nch; pos += kPushThreads) {
       const unsigned ent = order[pos];
+      if (pos + kPushThreads < nch) {  // the next particle's records
+        const int ni = c0 + (int)(order[pos + kPushThreads] & 4095);
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          prefetch_l1(p.o[d] + ni);
+          prefetch_l1(pn.o[d] + c0 + pos + kPushThreads);
+        }
+        prefetch_l1(p.w + ni);
+      }
       if (ent & kCross) continue;
       int r[3];
       L.cell((ent >> 12) & 4095, r);
       const int idx = c0 + (int)(ent & 4095), dst = c0 + pos;
-      const double qw = q * p.w[idx];
+      const double qw = pc.q * p.w[idx];
       long long S[3][4], D[3][4];
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
         long long w1[4];
-        spline62(to_fixed(p.o[d][idx], 62), S[d]);
-        spline62(to_fixed(pn.o[d][dst], 62), w1);
+        spline_fixed<62>(offset63(p.o[d][idx]) - kHalf63, S[d]);
+        spline_fixed<62>(offset63(pn.o[d][dst]) - kHalf63, w1);
 #pragma unroll
         for (int k = 0; k < 4; ++k) D[d][k] = w1[k] - S[d][k];
       }
@@ -325,35 +346,35 @@ __global__ void __launch_bounds__(kPushThreads, 2)
       for (int d = 0; d < 3; ++d) {  // axes 0, 1, 2 of the arrays: d, e, f
         const int sd = L.sd(d, 5), se = L.se(d, 5), lo = L.part(d, 5);
         unsigned* j = sJ + L.start(d, 5) + (r[0] + 1) * sd + (r[1] + 1) * se + r[2] + 1;  // nodes c-1 .. c+2
-        S31 Pi[3];
+        S32 Pi[3];
         {
-          const double cfs = qw * (d == 0 ? jc[0] : (d == 1 ? jc[1] : jc[2])) * exp2i(sc[4 + d] - 62);
+          const double cfs = qw * ((d == 0 ? pc.jc[0] : (d == 1 ? pc.jc[1] : pc.jc[2])) * exp2i(sc[4 + d] - 61));
           long long run = 0;
 #pragma unroll
           for (int m = 0; m < 3; ++m) {
             run += D[0][m];
-            Pi[m] = split31(to_fixed(fixed_to_double(run, 0) * cfs, 0));
+            Pi[m] = split32(to_fixed(fixed_to_double(run, 0) * cfs, 0));
           }
         }
-        S31 ak[4], bk[4];
+        S32 ak[4], bk[4];
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-          ak[c] = splitw((2 * S[2][c] + D[2][c]) >> 1);       // S_f + D_f / 2
-          bk[c] = splitw(third62(S[2][c], D[2][c]));  // S_f / 2 + D_f / 3
+          // at 2^63: S_f + D_f / 2 and S_f / 2 + D_f / 3 (= S1 - D / 3 at 2^62)
+          const long long S1 = S[2][c] + D[2][c];
+          ak[c] = split32(S[2][c] + S1);
+          bk[c] = split32(S1 - floor64(split32(D[2][c]), third64()));
         }
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
-          const S31 sb = splitw(S[1][b]), db = split31(D[1][b]);
+          const S32 sb = split32(S[1][b]), db = split32(D[1][b]);
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
-            Acc31 a = acc31_init();
-            acc31(a, sb, ak[c]);
-            acc31(a, db, bk[c]);
-            const S31 A = splitw(max(acc31_result(a), 0LL));  // A >= 0; clamps a rounding below zero
-            long long X[3];
+            Acc32 a = {0LL, 0LL};
+            acc32(a, sb, ak[c]);
+            acc32(a, db, bk[c]);
+            const S32 A = split32(acc32_result(a) << 2);  // at 2^63
 #pragma unroll
-            for (int m = 0; m < 3; ++m) X[m] = mul62(Pi[m], A);
-            add_current64<3>(j + b * se + c, lo, sd, X, 3);
+            for (int m = 0; m < 3; ++m) add_current64(j + m * sd + b * se + c, lo, mul64(Pi[m], A));
           }
         }
         const int r0 = r[0];
@@ -374,14 +395,14 @@ __global__ void __launch_bounds__(kPushThreads, 2)
       int r[3], n[3];
       L.cell((ent >> 12) & 4095, r);
       const int idx = c0 + (int)(ent & 4095), dst = c0 + pos;
-      const double qw = q * p.w[idx];
+      const double qw = pc.q * p.w[idx];
       long long S[3][5], D[3][5];
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
         const int dc = (int)((ent >> (24 + 2 * d)) & 3u) - 1;
         long long w0[4], w1[4];
-        spline62(to_fixed(p.o[d][idx], 62), w0);
-        spline62(to_fixed(pn.o[d][dst], 62), w1);
+        spline_fixed<62>(offset63(p.o[d][idx]) - kHalf63, w0);
+        spline_fixed<62>(offset63(pn.o[d][dst]) - kHalf63, w1);
         const int p0 = dc < 0 ? 1 : 0, p1 = dc > 0 ? 1 : 0;
         r[d] += 1 - p0;
         n[d] = dc != 0 ? 5 : 4;
@@ -397,37 +418,37 @@ __global__ void __launch_bounds__(kPushThreads, 2)
       for (int d = 0; d < 3; ++d) {
         const int sd = L.sd(d, 5), se = L.se(d, 5), lo = L.part(d, 5);
         unsigned* j = sJ + L.start(d, 5) + r[0] * sd + r[1] * se + r[2];
-        S31 Pi[4];
+        S32 Pi[4];
         {
-          const double cfs = qw * (d == 0 ? jc[0] : (d == 1 ? jc[1] : jc[2])) * exp2i(sc[4 + d] - 62);
+          const double cfs = qw * ((d == 0 ? pc.jc[0] : (d == 1 ? pc.jc[1] : pc.jc[2])) * exp2i(sc[4 + d] - 61));
           long long run = 0;
 #pragma unroll
           for (int m = 0; m < 4; ++m) {
             run += D[0][m];
-            Pi[m] = split31(to_fixed(fixed_to_double(run, 0) * cfs, 0));
+            Pi[m] = split32(to_fixed(fixed_to_double(run, 0) * cfs, 0));
           }
         }
-        S31 ak[5], bk[5];
+        S32 ak[5], bk[5];
 #pragma unroll
         for (int c = 0; c < 5; ++c) {
-          ak[c] = splitw((2 * S[2][c] + D[2][c]) >> 1);
-          bk[c] = splitw(third62(S[2][c], D[2][c]));
+          const long long S1 = S[2][c] + D[2][c];
+          ak[c] = split32(S[2][c] + S1);
+          bk[c] = split32(S1 - floor64(split32(D[2][c]), third64()));
         }
 #pragma unroll
         for (int b = 0; b < 5; ++b)
           if (b < n[1]) {
-            const S31 sb = splitw(S[1][b]), db = split31(D[1][b]);
+            const S32 sb = split32(S[1][b]), db = split32(D[1][b]);
 #pragma unroll
             for (int c = 0; c < 5; ++c)
               if (c < n[2]) {
-                Acc31 a = acc31_init();
-                acc31(a, sb, ak[c]);
-                acc31(a, db, bk[c]);
-                const S31 A = splitw(max(acc31_result(a), 0LL));
-                long long X[4];
+                Acc32 a = {0LL, 0LL};
+                acc32(a, sb, ak[c]);
+                acc32(a, db, bk[c]);
+                const S32 A = split32(acc32_result(a) << 2);
 #pragma unroll
-                for (int m = 0; m < 4; ++m) X[m] = mul62(Pi[m], A);
-                add_current64<4>(j + b * se + c, lo, sd, X, n[0] - 1);
+                for (int m = 0; m < 4; ++m)
+                  if (m < n[0] - 1) add_current64(j + m * sd + b * se + c, lo, mul64(Pi[m], A));
               }
           }
         const int r0 = r[0], n0 = n[0];
@@ -445,16 +466,16 @@ __global__ void __launch_bounds__(kPushThreads, 2)
 
     // flush: a half warp per (x, y) row, the lanes along z
     {
-      const int NY = tl.ty + 5, nrow = (tl.tx + 5) * NY, NZ = tl.tz + 5;
-      for (int r = tid >> 4; r < nrow; r += kPushThreads / 16) {
-        const int lx = r / NY, ly = r - lx * NY;
+      const int NX = tl.tx + 5, NZ = tl.tz + 5;
+      for (RowWalk r(tl.ty + 5); r.lx < NX; r.next()) {
+        const int lx = r.lx, ly = r.ly;
         const int gi0 = P.tabx[lx] + P.taby[ly];
         for (int lz = tid & 15; lz < NZ; lz += 16) {
           const int i3[3] = {lx, ly, lz};
 #pragma unroll
           for (int d = 0; d < 3; ++d) {
             const unsigned* w = sJ + L.start(d, 5) + i3[d] * L.sd(d, 5) + i3[(d + 1) % 3] * L.se(d, 5) + i3[(d + 2) % 3];
-            const long long X = (long long)(((unsigned long long)w[0] << 32) | w[L.part(d, 5)]);
+            const long long X = sum_current64(w[0], w[L.part(d, 5)], w[2 * L.part(d, 5)]);
             if (X != 0) atomicAdd(f.c[JX + d] + gi0 + P.tabz[lz], fixed_to_double(X, sc[4 + d]));
           }
         }

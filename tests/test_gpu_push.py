@@ -1,10 +1,10 @@
-"""One FP32 step against the FP64 oracle at the sizes where the FP32 push can
-go wrong: tiles that do not divide the grid, strides known to the compiler and
+"""One step against the FP64 oracle at the sizes where the push can go wrong: tiles that do not divide the grid, strides known to the compiler and
 not, one particle, an odd number in a cell (half a pair), more particles in a
 tile than one pass takes (3072), more in a cell than are ranked (32), and
 momenta with which most particles leave their cell (the separate deposit).
 
-Tolerances (eps = 2^-24): momenta 32 eps of the largest |u| (a few dozen
+Tolerances: FP64 the 1e-10 parity bar, relative to the largest value and in
+cells.  FP32 (eps = 2^-24): momenta 32 eps of the largest |u| (a few dozen
 roundings of the Boris push and the gather), positions 32 eps of a cell, and
 for a current value 16 eps sum |q w jc| over the particles whose window can
 reach the node: a contribution q w jc run A has |run| <= 3/4, A <= 0.45, the
@@ -53,11 +53,12 @@ def _positions(kind, shape, n, rng):
     ((16, 16, 16), None, "cell", 65, 0.01), ((16, 16, 16), None, "cell", 4001, 0.5),
     ((16, 16, 16), None, "tile", 3072, 0.5), ((16, 16, 16), None, "tile", 3073, 0.5),
     ((16, 16, 16), None, "tile", 9999, 2.0), ((16, 16, 16), None, "corner", 500, 2.0)])
-def test_fp32_step_against_oracle(shape, tile, kind, n, umax, monkeypatch):
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_step_against_oracle(precision, shape, tile, kind, n, umax, monkeypatch):
     if tile:
         monkeypatch.setenv("PIC_TILE", tile)
     args = (*shape, LAM / 8, LAM / 3, LAM / 2, LAM)
-    g = pic.Sim(*args, periodic_x=True, precision="fp32", track_ids=True)
+    g = pic.Sim(*args, periodic_x=True, precision=precision, track_ids=True)
     o = O.Sim(*args, periodic_x=True)
     inf = o.info()
     rng = np.random.default_rng(n)
@@ -74,10 +75,11 @@ def test_fp32_step_against_oracle(shape, tile, kind, n, umax, monkeypatch):
     o.step(1)
     pg, po = by_id(g.particles()), by_id(o.particles())
     assert np.array_equal(pg["id"], po["id"])
-    assert np.abs(pg["u"] - po["u"]).max() <= 32 * EPS * max(1.0, np.abs(po["u"]).max())
+    fp32 = precision == "fp32"
+    assert np.abs(pg["u"] - po["u"]).max() <= (32 * EPS if fp32 else 1e-10) * max(1.0, np.abs(po["u"]).max())
     dx = np.abs(pg["xi"] - po["xi"])
     dx = np.minimum(dx, np.array(shape)[:, None] - dx)
-    assert dx.max() <= 32 * EPS
+    assert dx.max() <= (32 * EPS if fp32 else 1e-10)
     assert np.array_equal(pg["w"], po["w"])
     # sum of |w| over the cells within 3 of a node
     near = np.zeros(shape)
@@ -86,5 +88,7 @@ def test_fp32_step_against_oracle(shape, tile, kind, n, umax, monkeypatch):
         near = sum(np.roll(near, k, axis) for k in range(-3, 4))
     jc = [1 / (inf["dt"] * inf["d" + "xyz"[b]] * inf["d" + "xyz"[c]]) for b, c in ((1, 2), (0, 2), (0, 1))]
     for a in range(3):
-        assert np.all(np.abs(g.field(6 + a) - o.field(6 + a)) <= 16 * EPS * jc[a] * near), "J%s" % "xyz"[a]
+        ref = o.field(6 + a)
+        bar = 16 * EPS * jc[a] * near if fp32 else 1e-10 * np.abs(ref).max()
+        assert np.all(np.abs(g.field(6 + a) - ref) <= bar), "J%s" % "xyz"[a]
     g.close()
