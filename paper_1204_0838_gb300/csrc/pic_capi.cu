@@ -15,6 +15,7 @@
 #include <vector>
 
 #include "../../include/pic.h"
+#include "pic_field64.cuh"
 #include "pic_host.h"
 #include "pic_runtime.h"
 #include "pic_push32.cuh"
@@ -348,28 +349,66 @@ FieldCoef<T> field_coef(const pic_t* h) {
   return c;
 }
 
+// The half-step magnetic field kept between steps.
 template <typename T>
-Fields<T> curl_view(const pic_t* h) {
+Fields<T> half_b(const pic_t* h) {
   Fields<T> c;
   for (int i = 0; i < NCOMP; ++i) c.c[i] = nullptr;
-  for (int i = 0; i < 3; ++i) c.c[i] = (T*)h->curl + (size_t)i * h->ncell;
+  for (int i = 0; i < 3; ++i) c.c[i] = (T*)h->half + (size_t)i * h->ncell;
   return c;
 }
 
-// Launch of the tiled smoothed curl over window-relative slabs [i0, i0 + ni).
-template <typename T>
-void launch_curl(const pic_t* h, const Geom<T>& g, int mode, int i0, int ni, cudaStream_t s) {
-  const dim3 grid((ni + CB_X - 1) / CB_X, (h->ny + CB_Y - 1) / CB_Y, (h->nz + CB_Z - 1) / CB_Z);
-  k_curl_tiled<T><<<grid, 256, curl_tiled_smem_bytes<T>(), s>>>(g, smooth<T>(h), fields<T>(h), curl_view<T>(h),
-                                                               field_coef<T>(h), mode, i0, ni, pml_view<T>(h));
+// Constant weights of the FP64 field kernels as split integers.
+FieldConst64 field_const64(const pic_t* h) {
+  auto split = [](double v, int k) {
+    const long long x = std::llround(std::ldexp(v, k));
+    const long long lo = (long long)(int)(unsigned)x;
+    return S32{(int)((x - lo) >> 32), (int)lo};
+  };
+  FieldConst64 w;
+  const double d[3] = {h->dx, h->dy, h->dz};
+  for (int a = 0; a < 3; ++a) {
+    const double s[4] = {h->sm_a[a], h->sm_b1[a], h->sm_b2[a], h->sm_g[a]};
+    for (int k = 0; k < 4; ++k) w.s[a][k] = split(s[k], 62);
+    w.hd[a] = split(0.5 * h->dt / d[a], 63);
+    w.fd[a] = split(h->dt / d[a], 62);
+  }
+  w.idt = 1.0 / h->dt;
+  w.ihdt = 2.0 / h->dt;
+  return w;
 }
 
-// C = curl'(E) over window-relative slabs [i0, i0 + ni).
+dim3 field_blocks(const pic_t* h, int ni) {
+  return dim3((ni + CB_X - 1) / CB_X, (h->ny + CB_Y - 1) / CB_Y, (h->nz + CB_Z - 1) / CB_Z);
+}
+
+// Electric step.
+void launch_e_update(const pic_t* h, const Geom<float>& g, cudaStream_t s) {
+  k_e_update<float><<<e_update_grid(h), e_update_block(h), 0, s>>>(g, fields<float>(h), half_b<float>(h),
+                                                                    field_coef<float>(h), pml_view<float>(h));
+}
+void launch_e_update(const pic_t* h, const Geom<double>& g, cudaStream_t s) {
+  k_e_update64<<<field_blocks(h, h->nx), 256, 0, s>>>(g, fields<double>(h), half_b<double>(h), field_coef<double>(h),
+                                                      field_const64(h), pml_view<double>(h));
+}
+
+// Magnetic half steps over window-relative slabs [i0, i0 + ni) (see k_curl_tiled).
+void launch_curl(const pic_t* h, const Geom<float>& g, int mode, int i0, int ni, cudaStream_t s) {
+  k_curl_tiled<float><<<field_blocks(h, ni), 256, curl_tiled_smem_bytes<float>(), s>>>(
+      g, smooth<float>(h), fields<float>(h), half_b<float>(h), field_coef<float>(h), mode, i0, ni, pml_view<float>(h));
+}
+void launch_curl(const pic_t* h, const Geom<double>& g, int mode, int i0, int ni, cudaStream_t s) {
+  k_curl64<<<field_blocks(h, ni), 256, kCurl64Smem, s>>>(g, smooth<double>(h), fields<double>(h), half_b<double>(h),
+                                                        field_coef<double>(h), field_const64(h), mode, i0, ni,
+                                                        pml_view<double>(h));
+}
+
+// H = B - (dt/2) curl'(E) over window-relative slabs [i0, i0 + ni).
 template <typename T>
-int curl_only(pic_t* h, int i0, int ni) {
+int half_only(pic_t* h, int i0, int ni) {
   GroupTimer tm(h, G_FIELD);
   counted(h, G_FIELD);
-  launch_curl<T>(h, geom<T>(h), 0, i0, ni, h->stream);
+  launch_curl(h, geom<T>(h), 0, i0, ni, h->stream);
   CK(h, cudaGetLastError());
   return PIC_OK;
 }
@@ -455,15 +494,14 @@ int zero_front_slab(pic_t* h, int storage_slab) {
 
 template <typename T>
 int field_first_half(pic_t* h) {
-  if (!h->curl_valid) {
-    int rc = curl_only<T>(h, 0, h->nx);
+  if (!h->half_valid) {
+    int rc = half_only<T>(h, 0, h->nx);
     if (rc) return rc;
-    h->curl_valid = true;
+    h->half_valid = true;
   }
   GroupTimer tm(h, G_FIELD);
   counted(h, G_FIELD);
-  k_e_update<T><<<e_update_grid(h), e_update_block(h), 0, h->stream>>>(geom<T>(h), fields<T>(h), curl_view<T>(h),
-                                                         field_coef<T>(h), pml_view<T>(h));
+  launch_e_update(h, geom<T>(h), h->stream);
   CK(h, cudaGetLastError());
   return PIC_OK;
 }
@@ -472,20 +510,20 @@ template <typename T>
 int field_second_half(pic_t* h) {
   GroupTimer tm(h, G_FIELD);
   counted(h, G_FIELD);
-  launch_curl<T>(h, geom<T>(h), 1, 0, h->nx, h->stream);
+  launch_curl(h, geom<T>(h), 1, 0, h->nx, h->stream);
   CK(h, cudaGetLastError());
   return PIC_OK;
 }
 
 // After a shift the storage slab that left at the back is the new, zeroed
-// front slab; the cached curl is recomputed where the window edges moved.
+// front slab; the half-step magnetic field is formed anew where the window edges moved.
 template <typename T>
 int after_shift_fields(pic_t* h, int old_origin) {
   int rc = zero_front_slab<T>(h, old_origin);
   if (rc) return rc;
-  if (h->curl_valid) {
-    rc = curl_only<T>(h, 0, 1);
-    if (!rc) rc = curl_only<T>(h, h->nx - 1, 1);
+  if (h->half_valid) {
+    rc = half_only<T>(h, 0, 1);
+    if (!rc) rc = half_only<T>(h, h->nx - 1, 1);
   }
   return rc;
 }
@@ -864,13 +902,13 @@ int pic_create(const pic_grid* g, double dt, const pic_window* w, pic_t** out) {
   if (noalloc_attach(h) != cudaSuccess) cudaGetLastError();
   h->stream = h->own_stream;
   h->fields = dalloc(h, NCOMP * h->ncell * esize(h));
-  h->curl = dalloc(h, 3 * h->ncell * esize(h));
+  h->half = dalloc(h, 3 * h->ncell * esize(h));
   h->tstart[0] = (int*)dalloc(h, sizeof(int) * (h->tiles.n + 1));
   h->tstart[1] = (int*)dalloc(h, sizeof(int) * (h->tiles.n + 1));
   h->tcnt = (int*)dalloc(h, sizeof(int) * h->tiles.n);
   h->tfill = (int*)dalloc(h, sizeof(int) * h->tiles.n);
   h->tiles_alloc = h->tiles.n;
-  if (!h->curl || !h->tstart[0] || !h->tstart[1] || !h->tcnt || !h->tfill) {
+  if (!h->half || !h->tstart[0] || !h->tstart[1] || !h->tcnt || !h->tfill) {
     pic_destroy(h);
     return PIC_ERR_OOM;
   }
@@ -884,8 +922,8 @@ int pic_create(const pic_grid* g, double dt, const pic_window* w, pic_t** out) {
               ? cudaFuncSetAttribute(push_kernel<double>(fixed), cudaFuncAttributeMaxDynamicSharedMemorySize, sm)
               : cudaFuncSetAttribute(push_kernel<float>(fixed), cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
     if (e == cudaSuccess)
-      e = h->precision == PIC_FP64 ? cudaFuncSetAttribute(k_curl_tiled<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                          (int)curl_tiled_smem_bytes<double>())
+      e = h->precision == PIC_FP64 ? cudaFuncSetAttribute(k_curl64, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                          (int)kCurl64Smem)
                                    : cudaFuncSetAttribute(k_curl_tiled<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                           (int)curl_tiled_smem_bytes<float>());
     if (e != cudaSuccess) {
@@ -1009,7 +1047,7 @@ int pic_add_laser(pic_t* h, double a0, double waist, double duration_fwhm, doubl
   h->laser_mode = mode;
   int rc;
   const double t = (double)h->step * h->dt;
-  h->curl_valid = false;
+  h->half_valid = false;
   if (mode == PIC_LASER_HARD_SOURCE)
     rc = h->precision == PIC_FP64 ? hard_source<double>(h, t) : hard_source<float>(h, t);
   else
@@ -1085,7 +1123,7 @@ int pic_set_field(pic_t* h, int comp, const double* host_in) {
   CK(h, cudaMemcpyAsync((char*)h->fields + comp * h->ncell * es, buf.data(), h->ncell * es, cudaMemcpyHostToDevice,
                         h->stream));
   CK(h, cudaStreamSynchronize(h->stream));
-  if (comp <= EZ) h->curl_valid = false;
+  if (comp <= BZ) h->half_valid = false;
   return PIC_OK;
 }
 
@@ -1376,7 +1414,7 @@ int pic_load(pic_t* h, const char* path) {
   h->step = hd.step;
   h->shifts = hd.shifts;
   h->win_frac = hd.win_frac;
-  h->curl_valid = false;
+  h->half_valid = false;
   unsigned long long pushed = (unsigned long long)hd.pushed;
   CK(h, cudaMemcpyAsync(h->d_pushed, &pushed, sizeof(pushed), cudaMemcpyHostToDevice, h->stream));
   CK(h, cudaStreamSynchronize(h->stream));
@@ -1479,7 +1517,7 @@ int set_tiles(pic_t* h, int tx, int ty, int tz) {
 // Device copy of the state that a trial step changes.
 struct Snapshot {
   void* fields = nullptr;
-  void* curl = nullptr;
+  void* half = nullptr;
   void* psi = nullptr;  // absorbing-layer memory variables (none without layers)
   void* part = nullptr;
   int ctrl[6];
@@ -1487,7 +1525,7 @@ struct Snapshot {
   int64_t step = 0, shifts = 0;
   int origin = 0;
   double win_frac = 0;
-  bool curl_valid = false, need_sort = false;
+  bool half_valid = false, need_sort = false;
   int np = 0;
 };
 
@@ -1497,12 +1535,12 @@ int snapshot_take(pic_t* h, Snapshot* sn) {
   CK(h, cudaMemcpy(sn->ctrl, h->d_ctrl, sizeof(sn->ctrl), cudaMemcpyDeviceToHost));
   sn->np = sn->ctrl[h->cur];
   sn->fields = dalloc(h, NCOMP * h->ncell * es);
-  sn->curl = dalloc(h, 3 * h->ncell * es);
+  sn->half = dalloc(h, 3 * h->ncell * es);
   const size_t per = 4 + 7 * es + (h->pb[0].id ? 4 : 0);
   sn->part = dalloc(h, per * (size_t)std::max(sn->np, 1));
-  if (!sn->fields || !sn->curl || !sn->part) return fail(h, PIC_ERR_OOM, "autotune snapshot");
+  if (!sn->fields || !sn->half || !sn->part) return fail(h, PIC_ERR_OOM, "autotune snapshot");
   CK(h, cudaMemcpyAsync(sn->fields, h->fields, NCOMP * h->ncell * es, cudaMemcpyDeviceToDevice, h->stream));
-  CK(h, cudaMemcpyAsync(sn->curl, h->curl, 3 * h->ncell * es, cudaMemcpyDeviceToDevice, h->stream));
+  CK(h, cudaMemcpyAsync(sn->half, h->half, 3 * h->ncell * es, cudaMemcpyDeviceToDevice, h->stream));
   if (h->psi) {
     sn->psi = dalloc(h, psi_values(h) * es);
     if (!sn->psi) return fail(h, PIC_ERR_OOM, "autotune snapshot");
@@ -1523,7 +1561,7 @@ int snapshot_take(pic_t* h, Snapshot* sn) {
   sn->shifts = h->shifts;
   sn->origin = h->origin;
   sn->win_frac = h->win_frac;
-  sn->curl_valid = h->curl_valid;
+  sn->half_valid = h->half_valid;
   sn->need_sort = h->need_sort;
   CK(h, cudaStreamSynchronize(h->stream));
   return PIC_OK;
@@ -1534,7 +1572,7 @@ int snapshot_restore(pic_t* h, Snapshot* sn) {
   const size_t es = esize(h);
   CK(h, cudaStreamSynchronize(h->stream));
   CK(h, cudaMemcpyAsync(h->fields, sn->fields, NCOMP * h->ncell * es, cudaMemcpyDeviceToDevice, h->stream));
-  CK(h, cudaMemcpyAsync(h->curl, sn->curl, 3 * h->ncell * es, cudaMemcpyDeviceToDevice, h->stream));
+  CK(h, cudaMemcpyAsync(h->half, sn->half, 3 * h->ncell * es, cudaMemcpyDeviceToDevice, h->stream));
   if (sn->psi) CK(h, cudaMemcpyAsync(h->psi, sn->psi, psi_values(h) * es, cudaMemcpyDeviceToDevice, h->stream));
   const PartBuf& b = h->pb[0];
   const char* src = (const char*)sn->part;
@@ -1556,11 +1594,11 @@ int snapshot_restore(pic_t* h, Snapshot* sn) {
   h->shifts = sn->shifts;
   h->origin = sn->origin;
   h->win_frac = sn->win_frac;
-  h->curl_valid = sn->curl_valid;
+  h->half_valid = sn->half_valid;
   h->need_sort = true;
   CK(h, cudaStreamSynchronize(h->stream));
   dfree(h, sn->fields);
-  dfree(h, sn->curl);
+  dfree(h, sn->half);
   dfree(h, sn->psi);
   dfree(h, sn->part);
   return PIC_OK;
@@ -1747,19 +1785,16 @@ int enqueue_step_dyn(pic_t* h, cudaStream_t s, int tsi, long long* kernels) {
   Geom<T> gs = g;
   gs.gate = 1;
   Fields<T> f = fields<T>(h);
-  const FieldCoef<T> fc = field_coef<T>(h);
-  const Smooth<T> S = smooth<T>(h);
   CK(h, cudaMemsetAsync(f.c[JX], 0, 3 * n * sizeof(T), s));
   CK(h, cudaMemsetAsync(h->tcnt, 0, sizeof(int) * tl.n, s));
   k_step_begin<<<1, 32, 0, s>>>(h->d_dyn);
   launch_push<T>(h, g, tsi, 0, s);
-  k_e_update<T><<<e_update_grid(h), e_update_block(h), 0, s>>>(g, f, curl_view<T>(h), fc, pml_view<T>(h));
-  launch_curl<T>(h, g, 1, 0, h->nx, s);
+  launch_e_update(h, g, s);
+  launch_curl(h, g, 1, 0, h->nx, s);
   k_window_commit<<<1, 32, 0, s>>>(h->d_dyn);
   k_zero_front_slab<T><<<grid_for((long long)NCOMP * h->ny * h->nz), 256, 0, s>>>(gs, f, pml_view<T>(h));
-  launch_curl<T>(h, gs, 0, 0, 1, s);
-  launch_curl<T>(h, gs, 0, h->nx - 1, 1, s);
-  (void)S;
+  launch_curl(h, gs, 0, 0, 1, s);
+  launch_curl(h, gs, 0, h->nx - 1, 1, s);
   LoadSpec L;
   const bool inject = h->has_species;
   const long long nslot = (long long)h->ny * h->nz * std::max(h->ppc, 1);
@@ -1832,10 +1867,10 @@ int prepare_and_capture(pic_batch_t* b) {
       if (rc) return bfail(b, rc, h->err);
       h->need_sort = false;
     }
-    if (!h->curl_valid) {
-      int rc = curl_only<float>(h, 0, h->nx);
+    if (!h->half_valid) {
+      int rc = half_only<float>(h, 0, h->nx);
       if (rc) return bfail(b, rc, h->err);
-      h->curl_valid = true;
+      h->half_valid = true;
     }
     int rc = dyn_to_device(h);
     if (rc) return bfail(b, rc, h->err);
@@ -1916,7 +1951,7 @@ int pic_batch_step(pic_batch_t* b, int n) {
   for (pic_t* s : b->sims) {
     int rc = grow_if_needed(s);
     if (rc) return bfail(b, rc, s->err);
-    if (s->need_sort) b->stale = true;
+    if (s->need_sort || !s->half_valid) b->stale = true;
   }
   if (b->stale) {
     int rc = prepare_and_capture(b);

@@ -99,13 +99,14 @@ __global__ void __launch_bounds__(256) k_curl_e(Geom<T> g, Smooth<T> S, const T*
 }
 
 // ---------------------------------------------------------------------------
-// Field update with a cached smoothed curl.  The two magnetic half steps of
-// consecutive steps use the same curl'(E^{n+1}), so it is computed once per
-// step and kept in C:
-//   k_e_update:     B^{n+1/2} = B^n - (dt/2) C^n (formed on the fly),
-//                   E^{n+1} = E^n + dt (curl B^{n+1/2} - J)
-//   k_curl_tiled:   C^{n+1} = curl'(E^{n+1}),
-//                   B^{n+1} = (B^n - (dt/2) C^n) - (dt/2) C^{n+1}
+// Field update with the half-step magnetic field kept.  The two magnetic half
+// steps of consecutive steps use the same curl'(E^{n+1}), so it is formed once
+// per step and never stored; H holds B^{n+1/2}:
+//   k_e_update:     E^{n+1} = E^n + dt (curl H - J)
+//   k_curl_tiled:   B^{n+1} = H - (dt/2) curl'(E^{n+1}),
+//                   H <- B^{n+1} - (dt/2) curl'(E^{n+1})
+// (12 values per cell and kernel; keeping the curl instead took 15, and formed H
+// anew at every neighbour: FP32 step on 101 M cells 28.1 -> 27.6 ms.)
 // Reciprocal spacings are precomputed (no divisions in the loops).
 // ---------------------------------------------------------------------------
 template <typename T>
@@ -114,66 +115,144 @@ struct FieldCoef {
   T idx, idy, idz;       // 1/dx, 1/dy, 1/dz
 };
 
+// H at a cell one below the grid at most (periodic, or zero beyond the grid).
 template <typename T>
-__device__ __forceinline__ T bhalf(const T* __restrict__ B, const T* __restrict__ C, const Geom<T>& g, int s,
-                                   int j, int k, T hdt) {
+__device__ __forceinline__ T below(const T* __restrict__ H, const Geom<T>& g, int s, int j, int k) {
   if (s < 0) return T(0);
   if (g.pml && (j < 0 || k < 0)) return T(0);
   j = (j < 0) ? j + g.ny : j;
   k = (k < 0) ? k + g.nz : k;
+  return H[(size_t)s * g.nyz + (size_t)j * g.nz + k];
+}
+
+template <typename T>
+__device__ __forceinline__ void e_update_cell(const Geom<T>& g, const Fields<T>& f, const Fields<T>& hb,
+                                              const FieldCoef<T>& fc, const Pml<T>& pm, int i, int j, int k) {
+  const T *Hx = hb.c[0], *Hy = hb.c[1], *Hz = hb.c[2];
+  const int s = slab_of(g, i), sm = slab_of(g, i - 1);
   const size_t id = (size_t)s * g.nyz + (size_t)j * g.nz + k;
-  return B[id] - hdt * C[id];
+  const T bx = Hx[id], by = Hy[id], bz = Hz[id];
+  T dyBz = (bz - below(Hz, g, s, j - 1, k)) * fc.idy;
+  T dzBy = (by - below(Hy, g, s, j, k - 1)) * fc.idz;
+  T dzBx = (bx - below(Hx, g, s, j, k - 1)) * fc.idz;
+  const T dxBz = (bz - below(Hz, g, sm, j, k)) * fc.idx;
+  const T dxBy = (by - below(Hy, g, sm, j, k)) * fc.idx;
+  T dyBx = (bx - below(Hx, g, s, j - 1, k)) * fc.idy;
+  if (pm.L) {  // Ex (i+1/2, j, k), Ey (i, j+1/2, k), Ez (i, j, k+1/2): y and z at nodes
+    const int jr = pml_row(j, g.ny, pm.L);
+    if (jr >= 0) {
+      const T a = pm.cy[j], b = pm.cy[g.ny + j];
+      const size_t pi = ((size_t)s * pm.rows + jr) * g.nz + k;
+      const T p0 = b * pm.py[0][pi] + a * dyBz, p1 = b * pm.py[1][pi] + a * dyBx;
+      pm.py[0][pi] = p0;
+      pm.py[1][pi] = p1;
+      dyBz += p0;
+      dyBx += p1;
+    }
+    const int kr = pml_row(k, g.nz, pm.L);
+    if (kr >= 0) {
+      const T a = pm.cz[k], b = pm.cz[g.nz + k];
+      const size_t pi = ((size_t)s * g.ny + j) * pm.rows + kr;
+      const T p0 = b * pm.pz[0][pi] + a * dzBy, p1 = b * pm.pz[1][pi] + a * dzBx;
+      pm.pz[0][pi] = p0;
+      pm.pz[1][pi] = p1;
+      dzBy += p0;
+      dzBx += p1;
+    }
+  }
+  f.c[EX][id] += fc.dt * ((dyBz - dzBy) - f.c[JX][id]);
+  f.c[EY][id] += fc.dt * ((dzBx - dxBz) - f.c[JY][id]);
+  f.c[EZ][id] += fc.dt * ((dxBy - dyBx) - f.c[JZ][id]);
 }
 
 // Launch: grid (ceil(nz / blockDim.x), ny, nx), one thread per cell; k from
 // the thread, j and the window-relative slab i from the block (no division).
 template <typename T>
-__global__ void __launch_bounds__(256) k_e_update(Geom<T> g, Fields<T> f, Fields<T> cc, FieldCoef<T> fc, Pml<T> pm) {
+__global__ void __launch_bounds__(256) k_e_update(Geom<T> g, Fields<T> f, Fields<T> hb, FieldCoef<T> fc, Pml<T> pm) {
   if (!dyn_prologue(g)) return;
-  const int nyz = g.nyz;
-  const T *Bx = f.c[BX], *By = f.c[BY], *Bz = f.c[BZ];
-  const T *Cx = cc.c[0], *Cy = cc.c[1], *Cz = cc.c[2];
-  {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y, i = blockIdx.z;
-    if (k >= g.nz) return;
-    const int r = j * g.nz + k;
-    const int s = slab_of(g, i), sm = slab_of(g, i - 1);
-    const size_t id = (size_t)s * nyz + r;
-    const T bx = Bx[id] - fc.hdt * Cx[id];
-    const T by = By[id] - fc.hdt * Cy[id];
-    const T bz = Bz[id] - fc.hdt * Cz[id];
-    T dyBz = (bz - bhalf(Bz, Cz, g, s, j - 1, k, fc.hdt)) * fc.idy;
-    T dzBy = (by - bhalf(By, Cy, g, s, j, k - 1, fc.hdt)) * fc.idz;
-    T dzBx = (bx - bhalf(Bx, Cx, g, s, j, k - 1, fc.hdt)) * fc.idz;
-    const T dxBz = (bz - bhalf(Bz, Cz, g, sm, j, k, fc.hdt)) * fc.idx;
-    const T dxBy = (by - bhalf(By, Cy, g, sm, j, k, fc.hdt)) * fc.idx;
-    T dyBx = (bx - bhalf(Bx, Cx, g, s, j - 1, k, fc.hdt)) * fc.idy;
-    if (pm.L) {  // Ex (i+1/2, j, k), Ey (i, j+1/2, k), Ez (i, j, k+1/2): y and z at nodes
-      const int jr = pml_row(j, g.ny, pm.L);
-      if (jr >= 0) {
-        const T a = pm.cy[j], b = pm.cy[g.ny + j];
-        const size_t pi = ((size_t)s * pm.rows + jr) * g.nz + k;
-        const T p0 = b * pm.py[0][pi] + a * dyBz, p1 = b * pm.py[1][pi] + a * dyBx;
-        pm.py[0][pi] = p0;
-        pm.py[1][pi] = p1;
-        dyBz += p0;
-        dyBx += p1;
-      }
-      const int kr = pml_row(k, g.nz, pm.L);
-      if (kr >= 0) {
-        const T a = pm.cz[k], b = pm.cz[g.nz + k];
-        const size_t pi = ((size_t)s * g.ny + j) * pm.rows + kr;
-        const T p0 = b * pm.pz[0][pi] + a * dzBy, p1 = b * pm.pz[1][pi] + a * dzBx;
-        pm.pz[0][pi] = p0;
-        pm.pz[1][pi] = p1;
-        dzBy += p0;
-        dzBx += p1;
-      }
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k < g.nz) e_update_cell(g, f, hb, fc, pm, (int)blockIdx.z, (int)blockIdx.y, k);
+}
+
+// The six derivatives of curl'(E) at a cell.
+template <typename T>
+struct CurlD {
+  T dyEz, dzEy, dzEx, dxEz, dxEy, dyEx;
+};
+
+// Absorbing layers in curl'(E): Bx (i, j+1/2, k+1/2), By (i+1/2, j, k+1/2), Bz
+// (i+1/2, j+1/2, k) at half nodes.  Mode 1 advances the memory variables with
+// E^{n+1}; mode 0 uses them as stored.
+template <typename T>
+__device__ __forceinline__ void curl_layers(const Geom<T>& g, const Pml<T>& pm, int mode, int slab, int j, int k,
+                                            CurlD<T>& d) {
+  const int jr = pml_row(j, g.ny, pm.L);
+  if (jr >= 0) {
+    const size_t pi = ((size_t)slab * pm.rows + jr) * g.nz + k;
+    T p2 = pm.py[2][pi], p3 = pm.py[3][pi];
+    if (mode == 1) {
+      const T a = pm.cy[2 * g.ny + j], b = pm.cy[3 * g.ny + j];
+      p2 = b * p2 + a * d.dyEz;
+      p3 = b * p3 + a * d.dyEx;
+      pm.py[2][pi] = p2;
+      pm.py[3][pi] = p3;
     }
-    f.c[EX][id] += fc.dt * ((dyBz - dzBy) - f.c[JX][id]);
-    f.c[EY][id] += fc.dt * ((dzBx - dxBz) - f.c[JY][id]);
-    f.c[EZ][id] += fc.dt * ((dxBy - dyBx) - f.c[JZ][id]);
+    d.dyEz += p2;
+    d.dyEx += p3;
   }
+  const int kr = pml_row(k, g.nz, pm.L);
+  if (kr >= 0) {
+    const size_t pi = ((size_t)slab * g.ny + j) * pm.rows + kr;
+    T p2 = pm.pz[2][pi], p3 = pm.pz[3][pi];
+    if (mode == 1) {
+      const T a = pm.cz[2 * g.nz + k], b = pm.cz[3 * g.nz + k];
+      p2 = b * p2 + a * d.dzEy;
+      p3 = b * p3 + a * d.dzEx;
+      pm.pz[2][pi] = p2;
+      pm.pz[3][pi] = p3;
+    }
+    d.dzEy += p2;
+    d.dzEx += p3;
+  }
+}
+
+// The magnetic updates of a cell from curl'(E); mode 0: H = B - (dt/2) curl'
+// only.  b: B (mode 0) or H (mode 1) as stored.
+template <typename T>
+__device__ __forceinline__ void curl_store(const Geom<T>& g, const Fields<T>& f, const Fields<T>& hb,
+                                           const FieldCoef<T>& fc, const Pml<T>& pm, int mode, int slab, int j, int k,
+                                           CurlD<T> d, const T (&b)[3]) {
+  if (pm.L) curl_layers(g, pm, mode, slab, j, k, d);
+  const T c[3] = {d.dyEz - d.dzEy, d.dzEx - d.dxEz, d.dxEy - d.dyEx};
+  const size_t id = (size_t)slab * g.nyz + (size_t)j * g.nz + k;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    T v = b[a];
+    if (mode == 1) {
+      v -= fc.hdt * c[a];
+      f.c[BX + a][id] = v;
+    }
+    hb.c[a][id] = v - fc.hdt * c[a];
+  }
+}
+
+// One cell of k_curl_tiled from global memory.
+template <typename T>
+__device__ __forceinline__ void curl_cell(const Geom<T>& g, const Smooth<T>& S, const Fields<T>& f, const Fields<T>& hb,
+                                          const FieldCoef<T>& fc, const Pml<T>& pm, int mode, int i, int j, int k) {
+  const int s = slab_of(g, i), sm = slab_of(g, i - 1), sp = slab_of(g, i + 1);
+  const T *Ex = f.c[EX], *Ey = f.c[EY], *Ez = f.c[EZ];
+  CurlD<T> d;
+  d.dyEz = (smooth_y(Ez, g, S, sm, s, sp, j + 1, k) - smooth_y(Ez, g, S, sm, s, sp, j, k)) * fc.idy;
+  d.dzEy = (smooth_z(Ey, g, S, sm, s, sp, j, k + 1) - smooth_z(Ey, g, S, sm, s, sp, j, k)) * fc.idz;
+  d.dzEx = (smooth_z(Ex, g, S, sm, s, sp, j, k + 1) - smooth_z(Ex, g, S, sm, s, sp, j, k)) * fc.idz;
+  d.dxEz = (smooth_x(Ez, g, S, sp, j, k) - smooth_x(Ez, g, S, s, j, k)) * fc.idx;
+  d.dxEy = (smooth_x(Ey, g, S, sp, j, k) - smooth_x(Ey, g, S, s, j, k)) * fc.idx;
+  d.dyEx = (smooth_y(Ex, g, S, sm, s, sp, j + 1, k) - smooth_y(Ex, g, S, sm, s, sp, j, k)) * fc.idy;
+  const size_t id = (size_t)s * g.nyz + (size_t)j * g.nz + k;
+  const T* const* src = mode == 1 ? hb.c : f.c + BX;
+  const T b[3] = {src[0][id], src[1][id], src[2][id]};
+  curl_store(g, f, hb, fc, pm, mode, s, j, k, d, b);
 }
 
 // ---------------------------------------------------------------------------
@@ -183,10 +262,11 @@ __global__ void __launch_bounds__(256) k_e_update(Geom<T> g, Fields<T> f, Fields
 // smoothed fields (S_x Ey, S_x Ez over x = i .. i+CB_X; S_y Ez, S_y Ex over
 // y = j .. j+CB_Y; S_z Ex, S_z Ey over z = k .. k+CB_Z) once per point, and
 // forms curl'(E) from their differences.
-// mode 0: C = curl'(E) only (start, after E changed outside a step, or the
-//         slabs next to a moved window edge), over window-relative slabs
-//         [i0, i0 + ni);
-// mode 1: C^{n+1} = curl'(E^{n+1}) and the two B half steps.
+// mode 0: H = B - (dt/2) curl'(E) only (start, after E or B changed outside a
+//         step, or the slabs next to a moved window edge), over window-relative
+//         slabs [i0, i0 + ni);
+// mode 1: the two magnetic half steps around t^{n+1}.
+// FP64 runs k_curl64 (pic_field64.cuh).
 // ---------------------------------------------------------------------------
 constexpr int CB_X = 4, CB_Y = 8, CB_Z = 32;
 constexpr int CE_X = CB_X + 2, CE_Y = CB_Y + 2, CE_Z = CB_Z + 2;  // staged E extents
@@ -202,7 +282,7 @@ size_t curl_tiled_smem_bytes() {
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) k_curl_tiled(Geom<T> g, Smooth<T> S, Fields<T> f, Fields<T> cc,
+__global__ void __launch_bounds__(256) k_curl_tiled(Geom<T> g, Smooth<T> S, Fields<T> f, Fields<T> hb,
                                                    FieldCoef<T> fc, int mode, int i0, int ni, Pml<T> pm) {
   if (!dyn_prologue(g)) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -236,12 +316,12 @@ __global__ void __launch_bounds__(256) k_curl_tiled(Geom<T> g, Smooth<T> S, Fiel
 #pragma unroll
     for (int c = 0; c < 3; ++c) sE[c * CE_N + q] = s < 0 ? T(0) : f.c[EX + c][gi];
   }
-  // Read what the output step needs from global memory (C, and B in mode 1)
+  // Read what the output step needs from global memory (H, or B in mode 0)
   // now, so that these loads overlap the shared-memory smoothing below.
   // blockDim.x is 256: each thread owns kPer cells of the block.
   constexpr int kPer = CB_X * CB_Y * CB_Z / 256;
   static_assert(CB_X * CB_Y * CB_Z % 256 == 0, "whole cells per thread");
-  T pb[kPer][3], pc[kPer][3];
+  T pb[kPer][3];
 #pragma unroll
   for (int t = 0; t < kPer; ++t) {
     const int q = tid + 256 * t;
@@ -251,10 +331,7 @@ __global__ void __launch_bounds__(256) k_curl_tiled(Geom<T> g, Smooth<T> S, Fiel
     const bool in = i < i0 + ni && j < g.ny && k < g.nz;
     const size_t id = in ? (size_t)slab_of(g, i) * g.nyz + (size_t)j * g.nz + k : 0;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      pc[t][c] = in && mode == 1 ? cc.c[c][id] : T(0);
-      pb[t][c] = in && mode == 1 ? f.c[BX + c][id] : T(0);
-    }
+    for (int c = 0; c < 3; ++c) pb[t][c] = in ? (mode == 1 ? hb.c[c][id] : f.c[BX + c][id]) : T(0);
   }
   __syncthreads();
 
@@ -313,52 +390,14 @@ __global__ void __launch_bounds__(256) k_curl_tiled(Geom<T> g, Smooth<T> S, Fiel
     const int y0 = (lx * (CB_Y + 1) + ly) * CB_Z + lz, y1 = (lx * (CB_Y + 1) + ly + 1) * CB_Z + lz;
     const int z0 = (lx * CB_Y + ly) * (CB_Z + 1) + lz;
     // Bx: D_y S_y Ez - D_z S_z Ey; By: D_z S_z Ex - D_x S_x Ez; Bz: D_x S_x Ey - D_y S_y Ex
-    T dyEz = (sSyEz[y1] - sSyEz[y0]) * fc.idy, dzEy = (sSzEy[z0 + 1] - sSzEy[z0]) * fc.idz;
-    T dzEx = (sSzEx[z0 + 1] - sSzEx[z0]) * fc.idz;
-    const T dxEz = (sSxEz[x1] - sSxEz[x0]) * fc.idx, dxEy = (sSxEy[x1] - sSxEy[x0]) * fc.idx;
-    T dyEx = (sSyEx[y1] - sSyEx[y0]) * fc.idy;
-    const int slab = slab_of(g, i);
-    if (pm.L) {  // Bx (i, j+1/2, k+1/2), By (i+1/2, j, k+1/2), Bz (i+1/2, j+1/2, k): half nodes
-      // mode 1 advances the memory variables with E^{n+1}; mode 0 uses them as stored
-      const int jr = pml_row(j, g.ny, pm.L);
-      if (jr >= 0) {
-        const size_t pi = ((size_t)slab * pm.rows + jr) * g.nz + k;
-        T p2 = pm.py[2][pi], p3 = pm.py[3][pi];
-        if (mode == 1) {
-          const T a = pm.cy[2 * g.ny + j], b = pm.cy[3 * g.ny + j];
-          p2 = b * p2 + a * dyEz;
-          p3 = b * p3 + a * dyEx;
-          pm.py[2][pi] = p2;
-          pm.py[3][pi] = p3;
-        }
-        dyEz += p2;
-        dyEx += p3;
-      }
-      const int kr = pml_row(k, g.nz, pm.L);
-      if (kr >= 0) {
-        const size_t pi = ((size_t)slab * g.ny + j) * pm.rows + kr;
-        T p2 = pm.pz[2][pi], p3 = pm.pz[3][pi];
-        if (mode == 1) {
-          const T a = pm.cz[2 * g.nz + k], b = pm.cz[3 * g.nz + k];
-          p2 = b * p2 + a * dzEy;
-          p3 = b * p3 + a * dzEx;
-          pm.pz[2][pi] = p2;
-          pm.pz[3][pi] = p3;
-        }
-        dzEy += p2;
-        dzEx += p3;
-      }
-    }
-    const T cx = dyEz - dzEy, cy = dzEx - dxEz, cz = dxEy - dyEx;
-    const size_t id = (size_t)slab * g.nyz + (size_t)j * g.nz + k;
-    if (mode == 1) {
-      f.c[BX][id] = (pb[t][0] - fc.hdt * pc[t][0]) - fc.hdt * cx;
-      f.c[BY][id] = (pb[t][1] - fc.hdt * pc[t][1]) - fc.hdt * cy;
-      f.c[BZ][id] = (pb[t][2] - fc.hdt * pc[t][2]) - fc.hdt * cz;
-    }
-    cc.c[0][id] = cx;
-    cc.c[1][id] = cy;
-    cc.c[2][id] = cz;
+    CurlD<T> d;
+    d.dyEz = (sSyEz[y1] - sSyEz[y0]) * fc.idy;
+    d.dzEy = (sSzEy[z0 + 1] - sSzEy[z0]) * fc.idz;
+    d.dzEx = (sSzEx[z0 + 1] - sSzEx[z0]) * fc.idz;
+    d.dxEz = (sSxEz[x1] - sSxEz[x0]) * fc.idx;
+    d.dxEy = (sSxEy[x1] - sSxEy[x0]) * fc.idx;
+    d.dyEx = (sSyEx[y1] - sSyEx[y0]) * fc.idy;
+    curl_store(g, f, hb, fc, pm, mode, slab_of(g, i), j, k, d, pb[t]);
   }
 }
 
