@@ -378,9 +378,11 @@ FieldConst64 field_const64(const pic_t* h) {
   return w;
 }
 
-dim3 field_blocks(const pic_t* h, int ni) {
-  return dim3((ni + CB_X - 1) / CB_X, (h->ny + CB_Y - 1) / CB_Y, (h->nz + CB_Z - 1) / CB_Z);
+// Blocks of the field kernels over all slabs, or over the two edge slabs.
+dim3 field_blocks(const pic_t* h, bool edges = false) {
+  return dim3(edges ? 2 : (h->nx + CB_X - 1) / CB_X, (h->ny + CB_Y - 1) / CB_Y, (h->nz + CB_Z - 1) / CB_Z);
 }
+FieldSpan field_span(const pic_t* h, bool edges) { return edges ? FieldSpan{h->nx - 1, 1} : FieldSpan{CB_X, CB_X}; }
 
 // Electric step.
 void launch_e_update(const pic_t* h, const Geom<float>& g, cudaStream_t s) {
@@ -388,27 +390,28 @@ void launch_e_update(const pic_t* h, const Geom<float>& g, cudaStream_t s) {
                                                                     field_coef<float>(h), pml_view<float>(h));
 }
 void launch_e_update(const pic_t* h, const Geom<double>& g, cudaStream_t s) {
-  k_e_update64<<<field_blocks(h, h->nx), 256, 0, s>>>(g, fields<double>(h), half_b<double>(h), field_coef<double>(h),
+  k_e_update64<<<field_blocks(h), 256, 0, s>>>(g, fields<double>(h), half_b<double>(h), field_coef<double>(h),
                                                       field_const64(h), pml_view<double>(h));
 }
 
-// Magnetic half steps over window-relative slabs [i0, i0 + ni) (see k_curl_tiled).
-void launch_curl(const pic_t* h, const Geom<float>& g, int mode, int i0, int ni, cudaStream_t s) {
-  k_curl_tiled<float><<<field_blocks(h, ni), 256, curl_tiled_smem_bytes<float>(), s>>>(
-      g, smooth<float>(h), fields<float>(h), half_b<float>(h), field_coef<float>(h), mode, i0, ni, pml_view<float>(h));
+// Magnetic half steps over all slabs or the two edge slabs (see k_curl_tiled).
+void launch_curl(const pic_t* h, const Geom<float>& g, int mode, bool edges, cudaStream_t s) {
+  k_curl_tiled<float><<<field_blocks(h, edges), 256, curl_tiled_smem_bytes<float>(), s>>>(
+      g, smooth<float>(h), fields<float>(h), half_b<float>(h), field_coef<float>(h), mode, field_span(h, edges),
+      pml_view<float>(h));
 }
-void launch_curl(const pic_t* h, const Geom<double>& g, int mode, int i0, int ni, cudaStream_t s) {
-  k_curl64<<<field_blocks(h, ni), 256, kCurl64Smem, s>>>(g, smooth<double>(h), fields<double>(h), half_b<double>(h),
-                                                        field_coef<double>(h), field_const64(h), mode, i0, ni,
-                                                        pml_view<double>(h));
+void launch_curl(const pic_t* h, const Geom<double>& g, int mode, bool edges, cudaStream_t s) {
+  k_curl64<<<field_blocks(h, edges), 256, kCurl64Smem, s>>>(g, smooth<double>(h), fields<double>(h), half_b<double>(h),
+                                                        field_coef<double>(h), field_const64(h), mode,
+                                                        field_span(h, edges), pml_view<double>(h));
 }
 
-// H = B - (dt/2) curl'(E) over window-relative slabs [i0, i0 + ni).
+// H = B - (dt/2) curl'(E) over all slabs or the two edge slabs.
 template <typename T>
-int half_only(pic_t* h, int i0, int ni) {
+int half_only(pic_t* h, bool edges) {
   GroupTimer tm(h, G_FIELD);
   counted(h, G_FIELD);
-  launch_curl(h, geom<T>(h), 0, i0, ni, h->stream);
+  launch_curl(h, geom<T>(h), 0, edges, h->stream);
   CK(h, cudaGetLastError());
   return PIC_OK;
 }
@@ -446,6 +449,28 @@ void launch_push(pic_t* h, const Geom<T>& g, int tsi, int origin_after, cudaStre
       h->tcnt, pc, origin_after, x_lo(h), x_hi(h), h->d_pushed, h->d_ctrl + 2);
 }
 
+// The tile arrays: counts, fill counters behind them (cleared together), and the
+// scan's partial sums.
+size_t tile_count_bytes(int tiles) {
+  return sizeof(int) * 2 * (((size_t)tiles + 3) / 4 * 4) + sizeof(long long) * ((size_t)tiles / kScanTiles + 1);
+}
+void set_tile_counts(pic_t* h, int* base, int tiles) {
+  h->tcnt = base;
+  h->tfill = base + ((size_t)tiles + 3) / 4 * 4;
+  h->tsum = (long long*)(h->tfill + ((size_t)tiles + 3) / 4 * 4);
+}
+cudaError_t clear_tile_counts(pic_t* h, cudaStream_t s) {
+  return cudaMemsetAsync(h->tcnt, 0, (char*)(h->tfill + h->tiles.n) - (char*)h->tcnt, s);
+}
+
+// Tile starts [ts] from the counts; returns the kernels launched.
+int scan_tiles(pic_t* h, int ts, int* np_out, cudaStream_t s) {
+  const int n = h->tiles.n, blocks = (n + kScanTiles - 1) / kScanTiles;
+  if (blocks > 1) k_tile_sums<<<blocks, 1024, 0, s>>>(h->tcnt, n, h->tsum);
+  k_scan_tiles<<<blocks, 1024, 0, s>>>(h->tcnt, h->tstart[ts], n, h->tsum, np_out, (int)h->capacity, h->d_ctrl + 2);
+  return blocks > 1 ? 2 : 1;
+}
+
 // Counting sort of the current buffer by tile into the other buffer.
 template <typename T>
 int resort_all(pic_t* h) {
@@ -453,12 +478,10 @@ int resort_all(pic_t* h) {
   const int nb = 1 - h->cur, ns = 1 - h->tsi;
   const Tiles tl = h->tiles;
   GroupTimer tm(h, G_PART);
-  CK(h, cudaMemsetAsync(h->tcnt, 0, sizeof(int) * tl.n, h->stream));
-  CK(h, cudaMemsetAsync(h->tfill, 0, sizeof(int) * tl.n, h->stream));
+  CK(h, clear_tile_counts(h, h->stream));
   k_keys<T><<<grid_for(h->capacity, 256, 152 * 16), 256, 0, h->stream>>>(geom<T>(h), tl, parts<T>(h, h->cur),
                                                                          h->d_ctrl + h->cur, h->keys, h->tcnt);
-  k_scan_tiles<<<1, 1024, 0, h->stream>>>(h->tcnt, h->tstart[ns], tl.n, h->d_ctrl + nb, (int)h->capacity,
-                                          h->d_ctrl + 2);
+  scan_tiles(h, ns, h->d_ctrl + nb, h->stream);
   k_scatter<T><<<grid_for(h->capacity, 256, 152 * 16), 256, 0, h->stream>>>(
       parts<T>(h, h->cur), h->keys, h->d_ctrl + h->cur, parts<T>(h, nb), h->tstart[ns], h->tfill, h->d_ctrl + 2);
   counted(h, G_PART, 3);
@@ -478,24 +501,9 @@ int window_due(pic_t* h, double t_old, double t_new, double* frac_new) {
 }
 
 template <typename T>
-int zero_front_slab(pic_t* h, int storage_slab) {
-  Fields<T> f = fields<T>(h);
-  const size_t slab = (size_t)h->ny * h->nz;
-  for (int c = 0; c < NCOMP; ++c)
-    CK(h, cudaMemsetAsync(f.c[c] + (size_t)storage_slab * slab, 0, slab * sizeof(T), h->stream));
-  const Pml<T> pm = pml_view<T>(h);
-  for (int c = 0; c < 4 && pm.L; ++c) {
-    const size_t ny_ = (size_t)pm.rows * h->nz, nz_ = (size_t)h->ny * pm.rows;
-    CK(h, cudaMemsetAsync(pm.py[c] + (size_t)storage_slab * ny_, 0, ny_ * sizeof(T), h->stream));
-    CK(h, cudaMemsetAsync(pm.pz[c] + (size_t)storage_slab * nz_, 0, nz_ * sizeof(T), h->stream));
-  }
-  return PIC_OK;
-}
-
-template <typename T>
 int field_first_half(pic_t* h) {
   if (!h->half_valid) {
-    int rc = half_only<T>(h, 0, h->nx);
+    int rc = half_only<T>(h, false);
     if (rc) return rc;
     h->half_valid = true;
   }
@@ -510,7 +518,7 @@ template <typename T>
 int field_second_half(pic_t* h) {
   GroupTimer tm(h, G_FIELD);
   counted(h, G_FIELD);
-  launch_curl(h, geom<T>(h), 1, 0, h->nx, h->stream);
+  launch_curl(h, geom<T>(h), 1, false, h->stream);
   CK(h, cudaGetLastError());
   return PIC_OK;
 }
@@ -518,12 +526,17 @@ int field_second_half(pic_t* h) {
 // After a shift the storage slab that left at the back is the new, zeroed
 // front slab; the half-step magnetic field is formed anew where the window edges moved.
 template <typename T>
-int after_shift_fields(pic_t* h, int old_origin) {
-  int rc = zero_front_slab<T>(h, old_origin);
-  if (rc) return rc;
+int after_shift_fields(pic_t* h) {
+  {
+    GroupTimer tm(h, G_PART);
+    counted(h, G_PART);
+    k_zero_front_slab<T><<<grid_for((long long)NCOMP * h->ny * h->nz), 256, 0, h->stream>>>(geom<T>(h), fields<T>(h),
+                                                                                            pml_view<T>(h));
+    CK(h, cudaGetLastError());
+  }
+  int rc = PIC_OK;
   if (h->half_valid) {
-    rc = half_only<T>(h, 0, 1);
-    if (!rc) rc = half_only<T>(h, h->nx - 1, 1);
+    rc = half_only<T>(h, true);
   }
   return rc;
 }
@@ -541,7 +554,7 @@ int step_tiled(pic_t* h) {
   const int cur = h->cur, moved = 1 - cur, ns = 1 - h->tsi;  // re-binning brings the moved particles back
   CK(h, cudaMemsetAsync(f.c[JX], 0, 3 * n * sizeof(T), h->stream));
   if (h->capacity > 0) {
-    CK(h, cudaMemsetAsync(h->tcnt, 0, sizeof(int) * tl.n, h->stream));
+    CK(h, clear_tile_counts(h, h->stream));
     GroupTimer tm(h, G_PUSH);
     counted(h, G_PUSH);
     launch_push<T>(h, geom<T>(h), h->tsi, origin_after, h->stream);
@@ -561,10 +574,9 @@ int step_tiled(pic_t* h) {
   LoadSpec L;
   if (shift) {
     h->win_frac -= 1.0;
-    const int old_origin = h->origin;
     h->origin = origin_after;
     h->shifts += 1;
-    rc = after_shift_fields<T>(h, old_origin);
+    rc = after_shift_fields<T>(h);
     if (rc) return rc;
   }
   if (h->capacity == 0) return PIC_OK;
@@ -577,13 +589,11 @@ int step_tiled(pic_t* h) {
         geom<T>(h), tl, parts<T>(h, cur), L, 0, h->tcnt, h->tstart[ns], h->tfill, h->d_ctrl + 2);
     counted(h, G_PART);
   }
-  k_scan_tiles<<<1, 1024, 0, h->stream>>>(h->tcnt, h->tstart[ns], tl.n, h->d_ctrl + cur, (int)h->capacity,
-                                          h->d_ctrl + 2);
-  CK(h, cudaMemsetAsync(h->tfill, 0, sizeof(int) * tl.n, h->stream));
+  counted(h, G_PART, scan_tiles(h, ns, h->d_ctrl + cur, h->stream));
   k_scatter<T><<<grid_for(h->capacity, 256, 152 * 16), 256, 0, h->stream>>>(
       parts<T>(h, moved), h->keys, h->tstart[h->tsi] + tl.n, parts<T>(h, cur), h->tstart[ns], h->tfill,
       h->d_ctrl + 2);
-  counted(h, G_PART, 2);
+  counted(h, G_PART);
   if (inject) {
     const long long nslot = (long long)h->ny * h->nz * h->ppc;
     k_inject_tiled<T><<<grid_for(nslot, 256, 152 * 16), 256, 0, h->stream>>>(
@@ -905,10 +915,9 @@ int pic_create(const pic_grid* g, double dt, const pic_window* w, pic_t** out) {
   h->half = dalloc(h, 3 * h->ncell * esize(h));
   h->tstart[0] = (int*)dalloc(h, sizeof(int) * (h->tiles.n + 1));
   h->tstart[1] = (int*)dalloc(h, sizeof(int) * (h->tiles.n + 1));
-  h->tcnt = (int*)dalloc(h, sizeof(int) * h->tiles.n);
-  h->tfill = (int*)dalloc(h, sizeof(int) * h->tiles.n);
+  if (int* base = (int*)dalloc(h, tile_count_bytes(h->tiles.n))) set_tile_counts(h, base, h->tiles.n);
   h->tiles_alloc = h->tiles.n;
-  if (!h->half || !h->tstart[0] || !h->tstart[1] || !h->tcnt || !h->tfill) {
+  if (!h->half || !h->tstart[0] || !h->tstart[1] || !h->tcnt) {
     pic_destroy(h);
     return PIC_ERR_OOM;
   }
@@ -1496,17 +1505,14 @@ int set_tiles(pic_t* h, int tx, int ty, int tz) {
   if (tl.n > h->tiles_alloc) {
     int* a0 = (int*)dalloc(h, sizeof(int) * (tl.n + 1));
     int* a1 = (int*)dalloc(h, sizeof(int) * (tl.n + 1));
-    int* c = (int*)dalloc(h, sizeof(int) * tl.n);
-    int* f = (int*)dalloc(h, sizeof(int) * tl.n);
-    if (!a0 || !a1 || !c || !f) return fail(h, PIC_ERR_OOM, "tile arrays");
+    int* c = (int*)dalloc(h, tile_count_bytes(tl.n));
+    if (!a0 || !a1 || !c) return fail(h, PIC_ERR_OOM, "tile arrays");
     dfree(h, h->tstart[0]);
     dfree(h, h->tstart[1]);
     dfree(h, h->tcnt);
-    dfree(h, h->tfill);
     h->tstart[0] = a0;
     h->tstart[1] = a1;
-    h->tcnt = c;
-    h->tfill = f;
+    set_tile_counts(h, c, tl.n);
     h->tiles_alloc = tl.n;
   }
   h->tiles = tl;
@@ -1786,15 +1792,14 @@ int enqueue_step_dyn(pic_t* h, cudaStream_t s, int tsi, long long* kernels) {
   gs.gate = 1;
   Fields<T> f = fields<T>(h);
   CK(h, cudaMemsetAsync(f.c[JX], 0, 3 * n * sizeof(T), s));
-  CK(h, cudaMemsetAsync(h->tcnt, 0, sizeof(int) * tl.n, s));
+  CK(h, clear_tile_counts(h, s));
   k_step_begin<<<1, 32, 0, s>>>(h->d_dyn);
   launch_push<T>(h, g, tsi, 0, s);
   launch_e_update(h, g, s);
-  launch_curl(h, g, 1, 0, h->nx, s);
+  launch_curl(h, g, 1, false, s);
   k_window_commit<<<1, 32, 0, s>>>(h->d_dyn);
   k_zero_front_slab<T><<<grid_for((long long)NCOMP * h->ny * h->nz), 256, 0, s>>>(gs, f, pml_view<T>(h));
-  launch_curl(h, gs, 0, 0, 1, s);
-  launch_curl(h, gs, 0, h->nx - 1, 1, s);
+  launch_curl(h, gs, 0, true, s);
   LoadSpec L;
   const bool inject = h->has_species;
   const long long nslot = (long long)h->ny * h->nz * std::max(h->ppc, 1);
@@ -1803,15 +1808,14 @@ int enqueue_step_dyn(pic_t* h, cudaStream_t s, int tsi, long long* kernels) {
     k_inject_tiled<T><<<grid_for(nslot, 256, 152 * 16), 256, 0, s>>>(gs, tl, parts<T>(h, cur), L, 0, h->tcnt,
                                                                      h->tstart[ns], h->tfill, h->d_ctrl + 2);
   }
-  k_scan_tiles<<<1, 1024, 0, s>>>(h->tcnt, h->tstart[ns], tl.n, h->d_ctrl + cur, (int)h->capacity, h->d_ctrl + 2);
-  CK(h, cudaMemsetAsync(h->tfill, 0, sizeof(int) * tl.n, s));
+  const int scans = scan_tiles(h, ns, h->d_ctrl + cur, s);
   k_scatter<T><<<grid_for(h->capacity, 256, 152 * 16), 256, 0, s>>>(parts<T>(h, moved), h->keys, h->tstart[tsi] + tl.n,
                                                                      parts<T>(h, cur), h->tstart[ns], h->tfill,
                                                                      h->d_ctrl + 2);
   if (inject)
     k_inject_tiled<T><<<grid_for(nslot, 256, 152 * 16), 256, 0, s>>>(gs, tl, parts<T>(h, cur), L, 1, h->tcnt,
                                                                      h->tstart[ns], h->tfill, h->d_ctrl + 2);
-  *kernels += 11 + (inject ? 2 : 0);
+  *kernels += 8 + scans + (inject ? 2 : 0);
   CK(h, cudaGetLastError());
   return PIC_OK;
 }
@@ -1868,7 +1872,7 @@ int prepare_and_capture(pic_batch_t* b) {
       h->need_sort = false;
     }
     if (!h->half_valid) {
-      int rc = half_only<float>(h, 0, h->nx);
+      int rc = half_only<float>(h, false);
       if (rc) return bfail(b, rc, h->err);
       h->half_valid = true;
     }

@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(256, 2)
 constexpr size_t kCurl64Smem = 8 * (3 * (size_t)CE_N + 2 * (size_t)(SXN + SYN + SZN));
 __global__ void __launch_bounds__(256, 2)
     k_curl64(Geom<double> g, Smooth<double> S, Fields<double> f, Fields<double> hb, FieldCoef<double> fc,
-             FieldConst64 k64, int mode, int i0, int ni, Pml<double> pm) {
+             FieldConst64 k64, int mode, FieldSpan sp, Pml<double> pm) {
   if (!dyn_prologue(g)) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int sh[3];
@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(256, 2)
   long long* sSyEx = sSyEz + SYN;
   long long* sSzEx = sSyEx + SYN;                          // [CB_X][CB_Y][CB_Z+1]
   long long* sSzEy = sSzEx + SZN;
-  const int bx = i0 + blockIdx.x * CB_X, by = blockIdx.y * CB_Y, bz = blockIdx.z * CB_Z;
+  const int bx = blockIdx.x * sp.step, bx1 = min(bx + sp.width, g.nx), by = blockIdx.y * CB_Y, bz = blockIdx.z * CB_Z;
   const int tid = threadIdx.x;
   constexpr int kPer = CB_X * CB_Y * CB_Z / 256;
   int e[3];
@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(256, 2)
       const int q = tid + 256 * t;
       const int lz = q % CB_Z, r = q / CB_Z;
       const int i = bx + r / CB_Y, j = by + r % CB_Y, k = bz + lz;
-      const bool in = i < i0 + ni && j < g.ny && k < g.nz;
+      const bool in = i < bx1 && j < g.ny && k < g.nz;
       const size_t id = in ? (size_t)slab_of(g, i) * g.nyz + (size_t)j * g.nz + k : 0;
 #pragma unroll
       for (int c = 0; c < 3; ++c) pb[t][c] = mode == 1 ? hb.c[c][id] : f.c[BX + c][id];
@@ -275,7 +275,7 @@ __global__ void __launch_bounds__(256, 2)
       const int q = tid + 256 * t;
       const int lz = q % CB_Z, r = q / CB_Z;
       const int i = bx + r / CB_Y, j = by + r % CB_Y, k = bz + lz;
-      if (i < i0 + ni && j < g.ny && k < g.nz) curl_cell(g, S, f, hb, fc, pm, mode, i, j, k);
+      if (i < bx1 && j < g.ny && k < g.nz) curl_cell(g, S, f, hb, fc, pm, mode, i, j, k);
     }
     return;
   }
@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(256, 2)
     const int q = tid + 256 * t;
     const int lz = q % CB_Z, r = q / CB_Z, ly = r % CB_Y, lx = r / CB_Y;
     const int i = bx + lx, j = by + ly, k = bz + lz;
-    if (i >= i0 + ni || j >= g.ny || k >= g.nz) continue;
+    if (i >= bx1 || j >= g.ny || k >= g.nz) continue;
     const int x0 = (lx * CB_Y + ly) * CB_Z + lz, x1 = x0 + CB_Y * CB_Z;
     const int y0 = (lx * (CB_Y + 1) + ly) * CB_Z + lz, y1 = y0 + CB_Z;
     const int z0 = (lx * CB_Y + ly) * (CB_Z + 1) + lz;

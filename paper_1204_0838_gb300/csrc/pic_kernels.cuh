@@ -263,12 +263,17 @@ __device__ __forceinline__ void curl_cell(const Geom<T>& g, const Smooth<T>& S, 
 // y = j .. j+CB_Y; S_z Ex, S_z Ey over z = k .. k+CB_Z) once per point, and
 // forms curl'(E) from their differences.
 // mode 0: H = B - (dt/2) curl'(E) only (start, after E or B changed outside a
-//         step, or the slabs next to a moved window edge), over window-relative
-//         slabs [i0, i0 + ni);
+//         step, or the slabs next to a moved window edge);
 // mode 1: the two magnetic half steps around t^{n+1}.
 // FP64 runs k_curl64 (pic_field64.cuh).
 // ---------------------------------------------------------------------------
 constexpr int CB_X = 4, CB_Y = 8, CB_Z = 32;
+// Window-relative slabs of a launch: block b covers [b step, b step + width).
+// All slabs: step = width = CB_X; the two at the window's edges: step = nx - 1,
+// width 1.
+struct FieldSpan {
+  int step, width;
+};
 constexpr int CE_X = CB_X + 2, CE_Y = CB_Y + 2, CE_Z = CB_Z + 2;  // staged E extents
 constexpr int CE_N = CE_X * CE_Y * CE_Z;
 // smoothed-field extents
@@ -283,7 +288,7 @@ size_t curl_tiled_smem_bytes() {
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_curl_tiled(Geom<T> g, Smooth<T> S, Fields<T> f, Fields<T> hb,
-                                                   FieldCoef<T> fc, int mode, int i0, int ni, Pml<T> pm) {
+                                                   FieldCoef<T> fc, int mode, FieldSpan sp, Pml<T> pm) {
   if (!dyn_prologue(g)) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* sE = reinterpret_cast<T*>(smem_raw);  // [3][CE_X][CE_Y][CE_Z], origin (bx-1, by-1, bz-1)
@@ -293,7 +298,7 @@ __global__ void __launch_bounds__(256) k_curl_tiled(Geom<T> g, Smooth<T> S, Fiel
   T* sSyEx = sSyEz + SYN;
   T* sSzEx = sSyEx + SYN;                  // [CB_X][CB_Y][CB_Z+1]
   T* sSzEy = sSzEx + SZN;
-  const int bx = i0 + blockIdx.x * CB_X, by = blockIdx.y * CB_Y, bz = blockIdx.z * CB_Z;
+  const int bx = blockIdx.x * sp.step, bx1 = bx + sp.width, by = blockIdx.y * CB_Y, bz = blockIdx.z * CB_Z;
   const int tid = threadIdx.x;
 
   // stage E with a one-cell halo (zero outside an open window)
@@ -328,7 +333,7 @@ __global__ void __launch_bounds__(256) k_curl_tiled(Geom<T> g, Smooth<T> S, Fiel
     const int lz = q % CB_Z, r = q / CB_Z;
     const int ly = r % CB_Y, lx = r / CB_Y;
     const int i = bx + lx, j = by + ly, k = bz + lz;
-    const bool in = i < i0 + ni && j < g.ny && k < g.nz;
+    const bool in = i < min(bx1, g.nx) && j < g.ny && k < g.nz;
     const size_t id = in ? (size_t)slab_of(g, i) * g.nyz + (size_t)j * g.nz + k : 0;
 #pragma unroll
     for (int c = 0; c < 3; ++c) pb[t][c] = in ? (mode == 1 ? hb.c[c][id] : f.c[BX + c][id]) : T(0);
@@ -385,7 +390,7 @@ __global__ void __launch_bounds__(256) k_curl_tiled(Geom<T> g, Smooth<T> S, Fiel
     const int lz = q % CB_Z, r = q / CB_Z;
     const int ly = r % CB_Y, lx = r / CB_Y;
     const int i = bx + lx, j = by + ly, k = bz + lz;
-    if (i >= i0 + ni || j >= g.ny || k >= g.nz) continue;
+    if (i >= min(bx1, g.nx) || j >= g.ny || k >= g.nz) continue;
     const int x0 = (lx * CB_Y + ly) * CB_Z + lz, x1 = ((lx + 1) * CB_Y + ly) * CB_Z + lz;
     const int y0 = (lx * (CB_Y + 1) + ly) * CB_Z + lz, y1 = (lx * (CB_Y + 1) + ly + 1) * CB_Z + lz;
     const int z0 = (lx * CB_Y + ly) * (CB_Z + 1) + lz;

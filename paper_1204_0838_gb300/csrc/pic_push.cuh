@@ -15,8 +15,8 @@
 
 namespace pic {
 
-constexpr int kPushThreads = 256;  // two CTAs per SM at 128 registers
-constexpr int kChunk = 3072;       // particles per pass over a tile
+constexpr int kPushThreads = 256;  // per SM: FP32 three CTAs at 80 registers, FP64 two at 128
+constexpr int kChunk = 2304;       // particles per pass over a tile (FP32: the lists that fit three CTAs)
 constexpr int kRanks = 32;         // ranks per cell that are ordered; later ones follow in any order
 // entry of the order list: particle of the pass (12 bits), cell slot (12
 // bits), cell steps + 1 per axis (6 bits) and two flags

@@ -28,12 +28,18 @@
 // - The components run in a loop over rotated axes: unrolled, the two phases
 //   were 130 KB of code and a quarter of all stalls waited for instructions.
 //
-// Measured (whole step, before -> after): 118 M particles, 1536x256x256 cells,
-// 2 per cell 41.3 -> 29.5 ms; 14 M particles, 4 per cell, absorbing layers
-// 4.85 -> 2.84 ms; 3.1 M at random places, a quarter leaving their cell each
-// step, 1.01 -> 0.78 ms.  With the bodies unrolled the first took 38.6 ms.
-// Now issue is active 53 % of cycles; shared memory (loads 1.7 wavefronts
-// each) and the latency of the particle loads share the rest.
+// - Three CTAs of 256 threads per SM at 80 registers: the weights are formed
+//   again for every rotation instead of kept; two particles' arithmetic goes in
+//   packed FP32 instructions.
+//
+// Measured (whole step, before -> after the two kernels' steps): 118 M particles,
+// 1536x256x256 cells, 2 per cell 41.3 -> 26.2 ms; 14 M particles, 4 per cell,
+// absorbing layers 4.85 -> 2.53 ms; 3.1 M at random places, a quarter leaving
+// their cell each step, 1.01 -> 0.72 ms.  With the bodies unrolled the first took
+// 38.6 ms, with two CTAs at 128 registers 27.6.  Now about 2,600 instructions per
+// 32 particles (4 per cell), issued 54 % of the time; shared-memory wavefronts
+// take 65 % of the cycles; barriers and the latency of the particle loads share
+// the rest.
 //
 // Exact current: every contribution is an integer product P A, P = round(q w
 // jc run 2^kp) below 2^31 with kp per chunk and component, A at 2^30; a node's
@@ -76,31 +82,40 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b) {
   return r;
 }
 __device__ __forceinline__ float2 dup2(float a) { return make_float2(a, a); }
-__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
 __device__ __forceinline__ float2 rsqrt2(float2 a) { return make_float2(rsqrtf(a.x), rsqrtf(a.y)); }
 
-// Cubic weights of both particles (see bspline3).
-__device__ __forceinline__ void bspline3_2(float2 t, float2 (&w)[4]) {
-  const float2 s = add2(dup2(1.0f), neg2(t)), t2 = mul2(t, t), s2 = mul2(s, s), t3 = mul2(t2, t), s3 = mul2(s2, s);
-  const float2 sixth = dup2(1.0f / 6.0f), two3 = dup2(2.0f / 3.0f), half = dup2(0.5f);
-  w[0] = mul2(s3, sixth);
-  w[1] = fma2(t3, half, add2(two3, neg2(t2)));
-  w[2] = fma2(s3, half, add2(two3, neg2(s2)));
-  w[3] = mul2(t3, sixth);
+// Cubic B-spline weights of the nodes c-1 .. c+2 for an offset t (see bspline3).
+// 2/3 is carried as a value and its remainder: rounded up alone, the weights of an
+// axis would sum to 4e-8 above one, and the current to twice that.
+__device__ __forceinline__ void spline32(float2 t, float2 (&w)[4]) {
+  constexpr float hi = 2.0f / 3.0f, lo = (float)(2.0 / 3.0 - (double)hi), sixth = 1.0f / 6.0f;
+  const float2 s = fma2(t, dup2(-1.0f), dup2(1.0f)), t2 = mul2(t, t), s2 = mul2(s, s), t3 = mul2(t2, t), s3 = mul2(s2, s);
+  w[0] = mul2(s3, dup2(sixth));
+  w[1] = add2(fma2(t2, dup2(-1.0f), dup2(hi)), fma2(t3, dup2(0.5f), dup2(lo)));
+  w[2] = add2(fma2(s2, dup2(-1.0f), dup2(hi)), fma2(s3, dup2(0.5f), dup2(lo)));
+  w[3] = mul2(t3, dup2(sixth));
 }
 
-// Node weights (nodes c-1 .. c+2) and half-node weights over c-2 .. c+2 (one
-// end zero: the particle's half cell picks the other four).
-__device__ __forceinline__ void weights32(float2 o, float2 (&wn)[4], float2 (&wh)[5]) {
+// Half-node weights over c-2 .. c+2 (one end zero: the particle's half cell
+// picks the other four).
+__device__ __forceinline__ void half_weights32(float2 o, float2 (&wh)[5]) {
   float2 h[4];
-  bspline3_2(o, wn);
   const bool lx = o.x < 0.5f, ly = o.y < 0.5f;
-  bspline3_2(make_float2(lx ? o.x + 0.5f : o.x - 0.5f, ly ? o.y + 0.5f : o.y - 0.5f), h);
+  spline32(make_float2(lx ? o.x + 0.5f : o.x - 0.5f, ly ? o.y + 0.5f : o.y - 0.5f), h);
   wh[0] = make_float2(lx ? h[0].x : 0.0f, ly ? h[0].y : 0.0f);
   wh[1] = make_float2(lx ? h[1].x : h[0].x, ly ? h[1].y : h[0].y);
   wh[2] = make_float2(lx ? h[2].x : h[1].x, ly ? h[2].y : h[1].y);
   wh[3] = make_float2(lx ? h[3].x : h[2].x, ly ? h[3].y : h[2].y);
   wh[4] = make_float2(lx ? 0.0f : h[3].x, ly ? 0.0f : h[3].y);
+}
+
+// Shape factors of both particles at an axis's old offsets, and their change.
+__device__ __forceinline__ void shapes32(float2 o0, float2 o1, float2 (&S)[4], float2 (&D)[4]) {
+  float2 w1[4];
+  spline32(o0, S);
+  spline32(o1, w1);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) D[k] = fma2(S[k], dup2(-1.0f), w1[k]);
 }
 
 // One component for both particles: NA x NB x NC nodes read once, contracted
@@ -115,14 +130,9 @@ __device__ __forceinline__ float2 gather_pair(const float* __restrict__ s, int s
 #pragma unroll
     for (int b = 0; b < NB; ++b) {
       const float* row = s + a * sd + b * se;
-      float f = row[0];
-      float2 rc = make_float2(f * wc[0].x, f * wc[0].y);
+      float2 rc = mul2(dup2(row[0]), wc[0]);  // a value for both halves costs no move
 #pragma unroll
-      for (int c = 1; c < NC; ++c) {
-        f = row[c];
-        rc.x = fmaf(f, wc[c].x, rc.x);
-        rc.y = fmaf(f, wc[c].y, rc.y);
-      }
+      for (int c = 1; c < NC; ++c) rc = fma2(dup2(row[c]), wc[c], rc);
       rb = b == 0 ? mul2(rc, wb[0]) : fma2(rc, wb[b], rb);
     }
     ra = a == 0 ? mul2(rb, wa[0]) : fma2(rb, wa[a], ra);
@@ -133,25 +143,26 @@ __device__ __forceinline__ float2 gather_pair(const float* __restrict__ s, int s
 // Boris push of both particles in fields E, B: new momenta and 1 / gamma.
 __device__ __forceinline__ float2 boris32(float h, const float2 (&E)[3], const float2 (&B)[3], float2 (&u)[3]) {
   const float2 one = dup2(1.0f), hh = dup2(h);
-  float2 um[3], tv[3], sv[3], pv[3];
+  float2 um[3], tv[3], tn[3], pv[3];
 #pragma unroll
   for (int d = 0; d < 3; ++d) um[d] = fma2(hh, E[d], u[d]);
   const float2 hg = mul2(hh, rsqrt2(fma2(um[2], um[2], fma2(um[1], um[1], fma2(um[0], um[0], one)))));  // h / gamma-
 #pragma unroll
-  for (int d = 0; d < 3; ++d) tv[d] = mul2(hg, B[d]);
+  for (int d = 0; d < 3; ++d) {
+    tv[d] = mul2(hg, B[d]);
+    tn[d] = mul2(tv[d], dup2(-1.0f));
+  }
   const float2 den = fma2(tv[2], tv[2], fma2(tv[1], tv[1], fma2(tv[0], tv[0], one)));
   const float2 s2 = make_float2(2.0f / den.x, 2.0f / den.y);
 #pragma unroll
-  for (int d = 0; d < 3; ++d) sv[d] = mul2(s2, tv[d]);
-#pragma unroll
   for (int d = 0; d < 3; ++d) {
     const int e = (d + 1) % 3, f = (d + 2) % 3;
-    pv[d] = add2(um[d], fma2(um[e], tv[f], neg2(mul2(um[f], tv[e]))));
+    pv[d] = add2(um[d], fma2(um[e], tv[f], mul2(um[f], tn[e])));
   }
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     const int e = (d + 1) % 3, f = (d + 2) % 3;
-    u[d] = fma2(hh, E[d], add2(um[d], fma2(pv[e], sv[f], neg2(mul2(pv[f], sv[e])))));
+    u[d] = fma2(hh, E[d], fma2(s2, fma2(pv[e], tv[f], mul2(pv[f], tn[e])), um[d]));
   }
   return rsqrt2(fma2(u[2], u[2], fma2(u[1], u[1], fma2(u[0], u[0], one))));
 }
@@ -185,7 +196,7 @@ constexpr float kA30 = 1073741824.0f;  // 2^30
 constexpr long long kHalf28 = 1LL << 28;
 
 template <bool FIXED>
-__global__ void __launch_bounds__(kPushThreads, 2)
+__global__ void __launch_bounds__(kPushThreads, 3)
     k_push32(Geom<float> g, Tiles tl, Fields<float> f, Parts<float> p, Parts<float> pn,
              const int* __restrict__ tstart, int capacity, int* __restrict__ keys, int* __restrict__ cnt_next,
              PushCoef<float> pc, int origin_after, int xlo, int xhi, unsigned long long* pushed, int* err) {
@@ -329,31 +340,37 @@ __global__ void __launch_bounds__(kPushThreads, 2)
           prefetch_l1(p.u[d] + idx[1]);
         }
         {
-          float2 wn[3][4], wh[3][5];
+          float2 o[3];
 #pragma unroll
-          for (int d = 0; d < 3; ++d) weights32(make_float2(p.o[d][idx[0]], p.o[d][idx[1]]), wn[d], wh[d]);
+          for (int d = 0; d < 3; ++d) o[d] = make_float2(p.o[d][idx[0]], p.o[d][idx[1]]);
           int r[3] = {l[0], l[1], l[2]};
+          // axes 0, 1, 2 of the arrays: d, e, f; the weights are formed again for
+          // every rotation and component (kept, they would cost the third CTA)
 #pragma unroll 1
-          for (int d = 0; d < 3; ++d) {  // axes 0, 1, 2 of the arrays: d, e, f
+          for (int d = 0; d < 3; ++d) {
             const int sd = L.sd(d, 4), se = L.se(d, 4);
             // node-centred axes start at c-1, half-staggered ones at c-2
             const float* b = sF + L.start(d, 4) + r[0] * sd + r[1] * se + r[2];
-            const float2 e = gather_pair<5, 4, 4>(b + se + 1, sd, se, wh[0], wn[1], wn[2]);
-            const float2 m = gather_pair<4, 5, 5>(b + L.part(d, 4) + sd, sd, se, wn[0], wh[1], wh[2]);
-            E[0] = E[1], E[1] = E[2], E[2] = e;
-            B[0] = B[1], B[1] = B[2], B[2] = m;
+            E[0] = E[1], E[1] = E[2];
+            B[0] = B[1], B[1] = B[2];
+            {
+              float2 wd[5], we[4], wf[4];
+              half_weights32(o[0], wd);
+              spline32(o[1], we);
+              spline32(o[2], wf);
+              E[2] = gather_pair<5, 4, 4>(b + se + 1, sd, se, wd, we, wf);
+            }
+            {
+              float2 wd[4], we[5], wf[5];
+              spline32(o[0], wd);
+              half_weights32(o[1], we);
+              half_weights32(o[2], wf);
+              B[2] = gather_pair<4, 5, 5>(b + L.part(d, 4) + sd, sd, se, wd, we, wf);
+            }
             const int r0 = r[0];
             r[0] = r[1], r[1] = r[2], r[2] = r0;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const float2 v = wn[0][k];
-              wn[0][k] = wn[1][k], wn[1][k] = wn[2][k], wn[2][k] = v;
-            }
-#pragma unroll
-            for (int k = 0; k < 5; ++k) {
-              const float2 v = wh[0][k];
-              wh[0][k] = wh[1][k], wh[1][k] = wh[2][k], wh[2][k] = v;
-            }
+            const float2 t = o[0];
+            o[0] = o[1], o[1] = o[2], o[2] = t;
           }
         }
 #pragma unroll
@@ -415,19 +432,14 @@ __global__ void __launch_bounds__(kPushThreads, 2)
       if (!(dep[0] || dep[1])) continue;
       int r[3];
       L.cell((ent[0] >> 12) & 4095, r);
-      float2 S[3][4], D[3][4], qw;
+      float2 oa[3], ob[3], qw;  // old and new offsets
       {
         const int i0 = c0 + (int)(ent[0] & 4095), i1 = c0 + (int)(ent[1] & 4095), d0 = c0 + pos[0], d1 = c0 + pos[1];
         qw = make_float2(dep[0] ? pc.q * p.w[i0] : 0.0f, dep[1] ? pc.q * p.w[i1] : 0.0f);
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-          const float2 a = make_float2(p.o[d][i0], p.o[d][i1]);
-          const float2 b = make_float2(dep[0] ? pn.o[d][d0] : a.x, dep[1] ? pn.o[d][d1] : a.y);
-          float2 w1[4];
-          bspline3_2(a, S[d]);
-          bspline3_2(b, w1);
-#pragma unroll
-          for (int k = 0; k < 4; ++k) D[d][k] = add2(w1[k], neg2(S[d][k]));
+          oa[d] = make_float2(p.o[d][i0], p.o[d][i1]);
+          ob[d] = make_float2(dep[0] ? pn.o[d][d0] : oa[d].x, dep[1] ? pn.o[d][d1] : oa[d].y);
         }
       }
 #pragma unroll 1
@@ -436,13 +448,15 @@ __global__ void __launch_bounds__(kPushThreads, 2)
         unsigned* j = sJ + L.start(d, 5) + (r[0] + 1) * sd + (r[1] + 1) * se + r[2] + 1;  // nodes c-1 .. c+2
         int Pi[2][3];
         {
+          float2 S[4], D[4];
+          shapes32(oa[0], ob[0], S, D);
           const float scale = __int_as_float((127 + sc[4 + d]) << 23);
           const float jc = d == 0 ? pc.jc[0] : (d == 1 ? pc.jc[1] : pc.jc[2]);
           const float2 c = mul2(mul2(dup2(jc), qw), dup2(scale));
           float2 run = make_float2(0.0f, 0.0f);
 #pragma unroll
           for (int m = 0; m < 3; ++m) {
-            run = add2(run, D[0][m]);
+            run = add2(run, D[m]);
             const float2 v = mul2(c, run);
             Pi[0][m] = __float2int_rn(v.x);
             Pi[1][m] = __float2int_rn(v.y);
@@ -450,16 +464,22 @@ __global__ void __launch_bounds__(kPushThreads, 2)
         }
         // A(b, c) = S_e (S_f + D_f / 2) + D_e (S_f / 2 + D_f / 3)
         float2 ak[4], bk[4];
+        {
+          float2 S[4], D[4];
+          shapes32(oa[2], ob[2], S, D);
 #pragma unroll
-        for (int m = 0; m < 4; ++m) {
-          ak[m] = mul2(dup2(kA30), fma2(dup2(0.5f), D[2][m], S[2][m]));
-          bk[m] = mul2(dup2(kA30), fma2(dup2(third), D[2][m], mul2(dup2(0.5f), S[2][m])));
+          for (int m = 0; m < 4; ++m) {
+            ak[m] = mul2(dup2(kA30), fma2(dup2(0.5f), D[m], S[m]));
+            bk[m] = mul2(dup2(kA30), fma2(dup2(third), D[m], mul2(dup2(0.5f), S[m])));
+          }
         }
+        float2 S[4], D[4];
+        shapes32(oa[1], ob[1], S, D);
 #pragma unroll
         for (int b = 0; b < 4; ++b)
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
-            const float2 A = fma2(D[1][b], bk[c], mul2(S[1][b], ak[c]));
+            const float2 A = fma2(D[b], bk[c], mul2(S[b], ak[c]));
             const int A0 = __float2int_rn(A.x), A1 = __float2int_rn(A.y);
 #pragma unroll
             for (int m = 0; m < 3; ++m)
@@ -467,12 +487,9 @@ __global__ void __launch_bounds__(kPushThreads, 2)
           }
         const int r0 = r[0];
         r[0] = r[1], r[1] = r[2], r[2] = r0;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const float2 v = S[0][k], w = D[0][k];
-          S[0][k] = S[1][k], S[1][k] = S[2][k], S[2][k] = v;
-          D[0][k] = D[1][k], D[1][k] = D[2][k], D[2][k] = w;
-        }
+        const float2 t = oa[0], v = ob[0];
+        oa[0] = oa[1], oa[1] = oa[2], oa[2] = t;
+        ob[0] = ob[1], ob[1] = ob[2], ob[2] = v;
       }
     }
     // particles that left their cell: 5-node windows where they moved
@@ -488,16 +505,15 @@ __global__ void __launch_bounds__(kPushThreads, 2)
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
         const int dc = (int)((e >> (24 + 2 * d)) & 3u) - 1;
-        float wn[4], w1[4];
-        bspline3(p.o[d][idx], wn);
-        bspline3(pn.o[d][dst], w1);
+        float2 w[4];  // at the old and the new offset
+        spline32(make_float2(p.o[d][idx], pn.o[d][dst]), w);
         const int p0 = dc < 0 ? 1 : 0, p1 = dc > 0 ? 1 : 0;
         r[d] += 1 - p0;
         n[d] = dc != 0 ? 5 : 4;
 #pragma unroll
         for (int m = 0; m < 5; ++m) {
-          const float a0 = p0 ? (m > 0 ? wn[m > 0 ? m - 1 : 0] : 0.0f) : (m < 4 ? wn[m < 4 ? m : 3] : 0.0f);
-          const float a1 = p1 ? (m > 0 ? w1[m > 0 ? m - 1 : 0] : 0.0f) : (m < 4 ? w1[m < 4 ? m : 3] : 0.0f);
+          const float a0 = p0 ? (m > 0 ? w[m > 0 ? m - 1 : 0].x : 0.0f) : (m < 4 ? w[m < 4 ? m : 3].x : 0.0f);
+          const float a1 = p1 ? (m > 0 ? w[m > 0 ? m - 1 : 0].y : 0.0f) : (m < 4 ? w[m < 4 ? m : 3].y : 0.0f);
           S[d][m] = a0;
           D[d][m] = a1 - a0;
         }

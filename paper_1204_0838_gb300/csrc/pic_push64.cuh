@@ -64,7 +64,7 @@ __device__ __forceinline__ void add_current64(unsigned* j, int part, long long X
   red_u32(j + 2 * part, (unsigned)((int)h >> 8));
 }
 
-// The sum of X from the words' sums of up to 3072 adds: sum (X >> 40) is exact
+// The sum of X from the words' sums of up to kChunk adds: sum (X >> 40) is exact
 // (the sum itself is below 2^62); sum (X >> 20) lies within n 2^20 < 2^32 above
 // 2^20 times it, and sum X within n 2^20 above 2^20 times that.
 __device__ __forceinline__ long long sum_current64(unsigned w0, unsigned w1, unsigned w2) {

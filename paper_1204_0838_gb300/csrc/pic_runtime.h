@@ -54,7 +54,8 @@ struct pic_t {
   int* tstart[2] = {nullptr, nullptr};  // tile starts, [tsi] those of the current buffer
   int tsi = 0;
   int* tcnt = nullptr;      // per-tile counts of the next buffer
-  int* tfill = nullptr;     // per-tile fill counters of the scatter
+  int* tfill = nullptr;     // per-tile fill counters of the scatter (behind tcnt)
+  long long* tsum = nullptr;  // partial sums of the tile scan (behind tfill)
   bool need_sort = false;   // particles not grouped by tile (after load/set)
   int tiles_alloc = 0;      // tile entries the tile arrays were sized for
   pic::DynState* d_dyn = nullptr;  // device-side step state (batched stepping)

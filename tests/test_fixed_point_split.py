@@ -93,7 +93,7 @@ def test_products_of_current_and_factors_round_without_bias():
 
 def test_current_words_give_back_the_exact_sum():
     rng = random.Random(4)
-    for n, top in ((1, 1 << 61), (3072, (1 << 62) // 3072), (3072, 1 << 40), (5, 3)):
+    for n, top in ((1, 1 << 61), (2304, (1 << 62) // 2304), (2304, 1 << 40), (5, 3)):
         for sign in (-1, 1, 0):
             xs = [rng.randrange(-top, top + 1) if not sign else sign * rng.randrange(top + 1) for _ in range(n)]
             w = [sum(x >> s for x in xs) % (1 << 32) for s in (0, 20, 40)]
