@@ -304,8 +304,10 @@ int hard_source(pic_t* h, double t) {
   const double xplane = h->x0 + (double)h->shifts * h->dx;
   GroupTimer tm(h, G_OTHER);
   counted(h, G_OTHER);
-  k_hard_source<T><<<grid_for(h->ny * h->nz), 256, 0, h->stream>>>(geom<T>(h), fields<T>(h).c[EY], L, xplane, t,
-                                                                    h->dy, h->dz);
+  // one warp per CTA: a few hundred FP64 instructions per node on a pipe of two
+  // lanes per SM (1024 nodes took 17 us in CTAs of 256)
+  k_hard_source<T><<<grid_for(h->ny * h->nz, 32), 32, 0, h->stream>>>(geom<T>(h), fields<T>(h).c[EY], L, xplane, t,
+                                                                      h->dy, h->dz);
   CK(h, cudaGetLastError());
   return PIC_OK;
 }
