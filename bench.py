@@ -36,23 +36,23 @@ UNIT = "particle-steps/s"
 # 4-node support per axis (a particle that crosses a cell face needs more):
 # weights 138, gather 882, Boris 54, position 17, deposit 522 (FMA = 2 flop).
 FLOP_PER_PARTICLE = 1613
-# Algorithmic DRAM bytes of k_push_tiled per particle: the SoA record read
-# and written once (FP64 112 B, FP32 60 B), plus per cell the E, B read by the
-# gather and the J written (FP64 72 B, FP32 36 B) shared by the ppc particles
-# of the cell.
+# Algorithmic DRAM bytes of the push (k_push64, k_push32) per particle: the SoA
+# record read and written once (FP64 112 B, FP32 60 B), plus per cell the E, B
+# read by the gather and the J written (FP64 72 B, FP32 36 B) shared by the ppc
+# particles of the cell.
 ALG_BYTES_PER_PARTICLE = {"fp64": lambda ppc: 112 + 72 / ppc, "fp32": lambda ppc: 60 + 36 / ppc}
-# DRAM bytes (read + write) per particle of k_push_tiled, from one ncu capture
-# of the current kernel on a 256x128x128 window in a run's own state (run for
-# 256 steps past a load at rest), 8x8x16 tiles; traffic per launch scales
-# with the particles processed.  None where the kernel has changed since its
-# capture (FP32: the float-to-fixed conversion of the deposit and the order
-# of the tile set-up; its last capture read 83.2 B per particle).
-NCU_TRAFFIC_PER_PARTICLE = {"fp64": (860.888576e6 + 1019.139e6) / 8336282, "fp32": None}
+# DRAM bytes (read + write) per particle of the push, from one ncu capture per
+# precision on a 256x128x128 window in a run's own state (run for 256 steps past
+# a load at rest), 8x8x8 tiles; traffic per launch scales with the particles
+# processed.
+NCU_TRAFFIC_PER_PARTICLE = {"fp64": (822.058752e6 + 625.361664e6) / 8336282,
+                            "fp32": (419.947264e6 + 309.271552e6) / 8336282}
 TRAFFIC_SOURCE = ("ncu dram__bytes_read.sum + dram__bytes_write.sum per particle (c1 spacings, 256x128x128 "
                   "window in a run's state) x particles per launch")
-LIMITER = {"fp64": ("issue latency and instruction fetch (ncu: issue active 36 %, FP64 pipe 30 %, integer ALU "
-                    "27 %, 16 warps per SM, top stalls no_instruction 22 % and wait 19 % of samples; DRAM 2 %)"),
-           "fp32": "shared-memory pipe (ncu: L1tex ~80 %; DRAM ~3 %)"}
+LIMITER = {"fp64": ("latency at 16 warps per SM (ncu: issue active 39 %, shared-memory pipe 54 %, integer ALU 30 %, "
+                    "FMA 26 %, FP64 pipe 25 %; DRAM 4 %)"),
+           "fp32": ("shared-memory pipe (ncu: L1tex 76 %, issue active 48 %, FMA 37 %, 24 warps per SM; "
+                    "DRAM 7 %)")}
 
 
 def _args():
@@ -312,13 +312,13 @@ def run_reference(args):
 
 
 def _roofline(precision, pushes_per_launch, avg_launch_s, ppc, peaks, src, group_ms, steps):
-    """Roofline record of the dominant kernel, k_push_tiled."""
+    """Roofline record of the dominant kernel, the push."""
     achieved = FLOP_PER_PARTICLE * pushes_per_launch / avg_launch_s / 1e12 if avg_launch_s > 0 else 0.0
     peak = _fp_peak_tflops(precision, peaks.get("sm_max_mhz", 2070.0))
     alg = ALG_BYTES_PER_PARTICLE[precision](ppc)
     hbm = alg * pushes_per_launch / avg_launch_s / 1e9 if avg_launch_s > 0 else None
     per = NCU_TRAFFIC_PER_PARTICLE.get(precision)
-    return {"kernel": "k_push_tiled (gather + Boris + Esirkepov deposit)",
+    return {"kernel": "%s (gather + Boris + Esirkepov deposit)" % ("k_push64" if precision == "fp64" else "k_push32"),
             "bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
             "frac": achieved / peak if peak else None,
             "traffic": per * pushes_per_launch if per else None,
@@ -488,7 +488,7 @@ def batch_leg(args, rank, local, ws):
     peaks, src = _peaks()
     ppc_mean = sum(c["ppc"] for c in cfgs) / len(cfgs)
     roof = _roofline("fp32", pushed_k2, k2_ms / 1e3, ppc_mean, peaks, src, {}, 1)
-    roof["kernel"] = "k_push_tiled (FP32), one host-driven step per member, summed over members"
+    roof["kernel"] = "k_push32, one host-driven step per member, summed over members"
     roof["traffic"] = None  # no capture of these member shapes (1-2 ppc, dx = lambda0/16)
     roof["traffic_source"] = "no capture of the batch members' shapes"
     out = {"value": value, "unit": UNIT, "steps": args.steps, "warmup": args.warmup,

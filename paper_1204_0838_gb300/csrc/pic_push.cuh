@@ -30,8 +30,8 @@ constexpr unsigned kStray = 1u << 30;  // outside the tile: dropped, error bit s
 // words, and J as [d][words of a sum] in 32-bit words (FP32 2, FP64 3).  FIXED:
 // tiles of up to 8 cells per axis, strides known to the compiler; otherwise any tile, with
 // odd pitches of rows and planes (a warp's cells along z lie a plane apart in one of the
-// rotations, and an even pitch put them on few banks: FP32 window step on 4x8x16 tiles
-// 10.5 -> 5.9 ms, on 16x8x8 7.8 -> 6.8; on 8x8x8 fixed 5.0).  The fixed
+// rotations, and an even pitch put them on few banks: two FP32 steps of 14 M
+// particles on 4x8x16 tiles 10.5 -> 5.9 ms, on 16x8x8 7.8 -> 6.8; on 8x8x8 fixed 5.0).  The fixed
 // strides are the best of a search over shapes of a warp's 32 cells and pitches:
 // 1x8x4 cells (slot order) read 32-bit fields and add to J in 1, 2 and 1 (fields)
 // or 2, 1 and 1 (J) wavefronts for the three rotations, and read 64-bit fields,
