@@ -201,9 +201,11 @@ def _peaks():
 
 def _fp_peak_tflops(precision, sm_mhz):
     """ALU peak from unit counts and clock: 152 SMs x FMA lanes per SM x 2 flop.
-    FP32: 128 lanes/SM.  FP64: 1.25 TFLOP/s nominal for the part at 2.07 GHz,
-    i.e. 2 FMA lanes per SM."""
-    lanes = 128 if precision == "fp32" else 2
+    FP32: 128 lanes/SM.  FP64: the push's products run in 64-bit fixed point,
+    three 32x32->64-bit integer multiply-adds each at 64 per SM and clock (18.9 T/s
+    of 32-bit ones measured, 60 per SM and clock), i.e. 64 / 3 lanes; the FP64
+    pipe itself has 2."""
+    lanes = 128 if precision == "fp32" else 64 / 3
     return 152 * lanes * 2 * sm_mhz * 1e6 / 1e12
 
 
@@ -323,11 +325,10 @@ def _roofline(precision, pushes_per_launch, avg_launch_s, ppc, peaks, src, group
             "frac": achieved / peak if peak else None,
             "traffic": per * pushes_per_launch if per else None,
             "traffic_source": TRAFFIC_SOURCE if per else "no capture of the current kernel",
-            "peak_source": "derived: 152 SMs x %s FMA lanes x 2 flop x %.0f MHz max clock%s" % (
-                "128 FP32" if precision == "fp32" else "2 FP64", peaks.get("sm_max_mhz", 2070.0),
-                "" if precision == "fp32" else
-                " (the FP64 pipe's rate for the push's FP64 arithmetic; the push runs the gather and the "
-                "deposit in 64-bit fixed point on the integer pipes instead)"),
+            "peak_source": "derived: 152 SMs x %s x 2 flop x %.0f MHz max clock" % (
+                "128 FP32 FMA lanes" if precision == "fp32" else
+                "64 integer multiply-add lanes / 3 multiply-adds per fixed-point product",
+                peaks.get("sm_max_mhz", 2070.0)),
             "limiter": LIMITER[precision],
             "hbm_algorithmic_bytes_per_particle": alg,
             "hbm_achieved_gbs": hbm, "hbm_peak_gbs": peaks.get("hbm_gbs"), "hbm_peak_source": src,
