@@ -485,7 +485,8 @@ int resort_all(pic_t* h) {
                                                                          h->d_ctrl + h->cur, h->keys, h->tcnt);
   scan_tiles(h, ns, h->d_ctrl + nb, h->stream);
   k_scatter<T><<<grid_for(h->capacity, 256, 152 * 16), 256, 0, h->stream>>>(
-      parts<T>(h, h->cur), h->keys, h->d_ctrl + h->cur, parts<T>(h, nb), h->tstart[ns], h->tfill, h->d_ctrl + 2);
+      parts<T>(h, h->cur), h->keys, h->d_ctrl + h->cur, (int)h->capacity, parts<T>(h, nb), h->tstart[ns], h->tfill,
+      h->d_ctrl + 2);
   counted(h, G_PART, 3);
   CK(h, cudaGetLastError());
   h->cur = nb;
@@ -593,8 +594,8 @@ int step_tiled(pic_t* h) {
   }
   counted(h, G_PART, scan_tiles(h, ns, h->d_ctrl + cur, h->stream));
   k_scatter<T><<<grid_for(h->capacity, 256, 152 * 16), 256, 0, h->stream>>>(
-      parts<T>(h, moved), h->keys, h->tstart[h->tsi] + tl.n, parts<T>(h, cur), h->tstart[ns], h->tfill,
-      h->d_ctrl + 2);
+      parts<T>(h, moved), h->keys, h->tstart[h->tsi] + tl.n, (int)h->capacity, parts<T>(h, cur), h->tstart[ns],
+      h->tfill, h->d_ctrl + 2);
   counted(h, G_PART);
   if (inject) {
     const long long nslot = (long long)h->ny * h->nz * h->ppc;
@@ -1516,6 +1517,8 @@ int set_tiles(pic_t* h, int tx, int ty, int tz) {
     h->tstart[1] = a1;
     set_tile_counts(h, c, tl.n);
     h->tiles_alloc = tl.n;
+    // as pic_create leaves them: without particles nothing else writes the starts
+    for (int b = 0; b < 2; ++b) CK(h, cudaMemsetAsync(h->tstart[b], 0, sizeof(int) * (tl.n + 1), h->stream));
   }
   h->tiles = tl;
   h->need_sort = true;
@@ -1794,14 +1797,19 @@ int enqueue_step_dyn(pic_t* h, cudaStream_t s, int tsi, long long* kernels) {
   gs.gate = 1;
   Fields<T> f = fields<T>(h);
   CK(h, cudaMemsetAsync(f.c[JX], 0, 3 * n * sizeof(T), s));
-  CK(h, clear_tile_counts(h, s));
   k_step_begin<<<1, 32, 0, s>>>(h->d_dyn);
-  launch_push<T>(h, g, tsi, 0, s);
+  if (h->capacity > 0) {
+    CK(h, clear_tile_counts(h, s));
+    launch_push<T>(h, g, tsi, 0, s);
+  }
   launch_e_update(h, g, s);
   launch_curl(h, g, 1, false, s);
   k_window_commit<<<1, 32, 0, s>>>(h->d_dyn);
   k_zero_front_slab<T><<<grid_for((long long)NCOMP * h->ny * h->nz), 256, 0, s>>>(gs, f, pml_view<T>(h));
   launch_curl(h, gs, 0, true, s);
+  *kernels += 6;
+  CK(h, cudaGetLastError());
+  if (h->capacity == 0) return PIC_OK;  // fields only: there are no particle buffers to read
   LoadSpec L;
   const bool inject = h->has_species;
   const long long nslot = (long long)h->ny * h->nz * std::max(h->ppc, 1);
@@ -1812,12 +1820,12 @@ int enqueue_step_dyn(pic_t* h, cudaStream_t s, int tsi, long long* kernels) {
   }
   const int scans = scan_tiles(h, ns, h->d_ctrl + cur, s);
   k_scatter<T><<<grid_for(h->capacity, 256, 152 * 16), 256, 0, s>>>(parts<T>(h, moved), h->keys, h->tstart[tsi] + tl.n,
-                                                                     parts<T>(h, cur), h->tstart[ns], h->tfill,
-                                                                     h->d_ctrl + 2);
+                                                                     (int)h->capacity, parts<T>(h, cur), h->tstart[ns],
+                                                                     h->tfill, h->d_ctrl + 2);
   if (inject)
     k_inject_tiled<T><<<grid_for(nslot, 256, 152 * 16), 256, 0, s>>>(gs, tl, parts<T>(h, cur), L, 1, h->tcnt,
                                                                      h->tstart[ns], h->tfill, h->d_ctrl + 2);
-  *kernels += 8 + scans + (inject ? 2 : 0);
+  *kernels += 2 + scans + (inject ? 2 : 0);
   CK(h, cudaGetLastError());
   return PIC_OK;
 }

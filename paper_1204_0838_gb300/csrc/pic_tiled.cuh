@@ -147,9 +147,9 @@ static __global__ void __launch_bounds__(1024) k_scan_tiles(const int* __restric
 
 // Scatter the kept particles into their tiles of the other buffer.
 template <typename T>
-__global__ void k_scatter(Parts<T> src, const int* __restrict__ keys, const int* __restrict__ d_np_src,
+__global__ void k_scatter(Parts<T> src, const int* __restrict__ keys, const int* __restrict__ d_np_src, int capacity,
                           Parts<T> dst, const int* __restrict__ tstart, int* fill, int* err) {
-  const int n = *d_np_src;
+  const int n = min(*d_np_src, capacity);
   for (int base = blockIdx.x * blockDim.x; base < n; base += gridDim.x * blockDim.x) {
     const int pi = base + threadIdx.x;
     const int key = pi < n ? keys[pi] : -2;
