@@ -20,7 +20,7 @@ constexpr int kChunk = 2304;       // particles per pass over a tile (FP32: the 
 constexpr int kRanks = 32;         // ranks per cell that are ordered; later ones follow in any order
 // entry of the order list: particle of the pass (12 bits), cell slot (12
 // bits), cell steps + 1 per axis (6 bits) and two flags
-constexpr unsigned kCross = 1u << 31;  // does not deposit with the ordered particles
+constexpr unsigned kCross = 1u << 31;  // not with the ordered particles: alone (listed) or not at all
 constexpr unsigned kStray = 1u << 30;  // outside the tile: dropped, error bit set
 
 // The shared-memory region.  Components are stored with their axes rotated,
@@ -79,8 +79,8 @@ struct PushLayout {
 };
 
 // Shared memory: the region (staged fields and the ranking's scratch, then J),
-// the order list (32-bit entries), the FP32 pair list, the list of crossing
-// particles, the wrapped grid offsets per axis, and 64 ints of scalars.
+// the order list (32-bit entries), the FP32 pair list, the list of particles
+// that deposit alone, the wrapped grid offsets per axis, and 64 ints of scalars.
 struct PushSmem {
   size_t hist, mask, base, order, pair, cross, tab, scal, total;
   template <typename T, bool FIXED>
@@ -112,10 +112,11 @@ struct PushSmem {
 };
 
 // Pointers into the shared memory of a CTA, and the scalars: [0] particles
-// without an ordered rank, [1] particles that left their cell, [2, 4) sums or
+// without an ordered rank, [1] particles that deposit alone, [2, 4) sums or
 // maxima over the pass, [4, 7) J scale per component, [8, 16) scan partials,
 // [16, 33) first pair of each pair of ranks, [33] ordered particles, [34, 50)
-// first position of each pair of ranks, [50, 62) field scales (FP64).
+// first position of each pair of ranks, [50, 62) field scales (FP64), [50, 53)
+// scale of P per component and [53] the weight below which a particle is light (FP32).
 struct PushTile {
   int* hist;
   unsigned* mask;         // [rank][word]: cells that hold more than `rank` particles
@@ -298,14 +299,14 @@ __device__ __forceinline__ void rank_order(const PushTile& P, int W, int nch, co
 // Store a moved particle's cell and key.  l: its cell in the tile, dc: its
 // steps (at most one cell per axis, periodic in the storage frame).  Returns
 // the destination tile or -1 (absorbed), and lists a particle that left its
-// cell at position pos.
+// cell, or that deposits alone for another reason, at position pos.
 template <typename T>
 __device__ __forceinline__ int place_moved(const PushTile& P, const Geom<T>& g, const Tiles& tl, int t,
-                                           const int (&l)[3], const int (&dc)[3], bool good, int origin_after,
+                                           const int (&l)[3], const int (&dc)[3], bool good, bool alone, int origin_after,
                                            int xlo, int xhi, int pos, unsigned ent, int* cell_out, int* key_out) {
   int n0 = P.x0 + l[0] + dc[0], n1 = P.y0 + l[1] + dc[1], n2 = P.z0 + l[2] + dc[2];
   int key = t;
-  if (dc[0] | dc[1] | dc[2]) {
+  if ((dc[0] | dc[1] | dc[2]) || alone) {
     n0 = wrapi(n0, g.nx), n1 = wrapi(n1, g.ny), n2 = wrapi(n2, g.nz);
     if ((unsigned)(n0 - P.x0) >= (unsigned)tl.tx || (unsigned)(n1 - P.y0) >= (unsigned)tl.ty ||
         (unsigned)(n2 - P.z0) >= (unsigned)tl.tz)

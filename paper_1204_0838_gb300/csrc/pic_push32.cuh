@@ -41,15 +41,22 @@
 // take 65 % of the cycles; barriers and the latency of the particle loads share
 // the rest.
 //
-// Exact current: every contribution is an integer product P A, P = round(q w
-// jc run 2^kp) below 2^31 with kp per chunk and component, A at 2^30; a node's
-// sum over the pair, T = (sum P A + 2^28) >> 29, is added as two 32-bit words,
-// hi = T >> 12 and lo = T mod 2^32.  The words give back the exact sum of T:
-// it is congruent to lo modulo 2^32 and lies in [2^12 hi, 2^12 (hi + n)) for n
-// adds, n < 2^20.  The sum bound B 2^(kp + 1) < 2^42 (B = |q jc| sum |w|)
-// keeps hi below 2^30.  The tile sum does not depend on the order of the adds;
-// the rounding of P is 2^-32 of the largest |q w jc|, below the 2^-26 or so
-// that the FP32 shape factors leave in P itself.
+// Current: sums of integers at 2^s per pass and component, with s the largest
+// for which B 2^s < 2^42, B = |q jc| sum |w|.  A contribution is a product of
+// two rounded integers, P = q w jc run at 2^kp, below 2^31, and A at 2^31; a
+// pair's P A are added exactly and rounded once, T = sum P A >> (kp + 31 - s),
+// and T is added as two 32-bit words, hi = T >> 12 and lo = T mod 2^32.  The
+// words give back the exact sum of T: it is congruent to lo modulo 2^32 and
+// lies in [2^12 hi, 2^12 (hi + n)) for n adds, n < 2^20; hi stays below 2^31.
+// So the sum does not depend on the order of the adds.  A contribution is
+// rounded by 2^-42 of B, and P, if less than that, by
+// - 2^-31 of the pass's largest |q w jc| for particles within 8 of the largest
+//   weight, which share kp: at most 2^-28 of their own |q w jc|, below the 2^-26
+//   or so that the FP32 shape factors leave in P itself;
+// - 2^-31 of its own |q w jc| for a lighter particle or one that left its cell:
+//   these deposit one per lane, with a kp of their own.  (With one kp for all, the
+//   current of particles at 1e-4 of the largest weight was off by 1e-4 of itself,
+//   of those at 1e-6 by 1e-2.)
 #pragma once
 
 #include "pic_push.cuh"
@@ -185,15 +192,16 @@ __device__ __forceinline__ int step32(float o, float& o1) {
   return k;
 }
 
-__device__ __forceinline__ void add_current(unsigned* hi, int lo_off, long long X) {
+// Add T = X >> sh, 20 <= sh <= 31 (X holds the rounding half already).
+__device__ __forceinline__ void add_current(unsigned* hi, int lo_off, long long X, int sh) {
   const int xh = (int)(X >> 32);
   const unsigned xl = (unsigned)X;
-  red_u32(hi, (unsigned)(xh >> 9));                           // T >> 12
-  red_u32(hi + lo_off, __funnelshift_r(xl, (unsigned)xh, 29));  // T mod 2^32
+  red_u32(hi, (unsigned)(xh >> (sh - 20)));                   // T >> 12
+  red_u32(hi + lo_off, __funnelshift_r(xl, (unsigned)xh, sh));  // T mod 2^32
 }
 
-constexpr float kA30 = 1073741824.0f;  // 2^30
-constexpr long long kHalf28 = 1LL << 28;
+constexpr float kA31 = 2147483648.0f;  // 2^31; A is at most 4/9
+constexpr float kLight = 0.125f;       // of the largest weight: below it a particle has its own kp
 
 template <bool FIXED>
 __global__ void __launch_bounds__(kPushThreads, 3)
@@ -272,11 +280,17 @@ __global__ void __launch_bounds__(kPushThreads, 3)
     __syncthreads();
     rank_masks(P, W);
     if (tid < 3) {
-      // kp: |P| 2^kp < 2^31 for P <= 0.76 |q| max w jc, and B 2^(kp + 1) < 2^42
+      // s: B 2^s < 2^42; kp: |P| 2^kp < 2^31 for P <= 0.76 |q| max w jc, no finer
+      // than s.  B > Pm, so that 20 <= kp + 31 - s <= 31.
       const float jc = fabsf(pc.q * (tid == 0 ? pc.jc[0] : (tid == 1 ? pc.jc[1] : pc.jc[2])));
-      const float Pm = 0.76f * jc * __int_as_float(sc[3]), B = 1.001f * jc * __int_as_float(sc[2]);
+      const float wm = __int_as_float(sc[3]);
+      const float Pm = 0.76f * jc * wm, B = 1.001f * jc * __int_as_float(sc[2]);
       const int ep = ((__float_as_int(Pm) >> 23) & 255) - 127, eb = ((__float_as_int(B) >> 23) & 255) - 127;
-      sc[4 + tid] = B > 0.0f ? max(min(min(30 - ep, 40 - eb), 120), -120) : 0;
+      const int s = B > 0.0f ? min(41 - eb, 120) : 0;
+      const int kp = B > 0.0f ? max(min(30 - ep, s), s - 11) : 0;
+      sc[4 + tid] = s;
+      sc[50 + tid] = kp;
+      if (kp < s) atomicMax(sc + 53, __float_as_int(kLight * wm));
     }
     __syncthreads();
     rank_order(P, W, nch, sr);
@@ -396,10 +410,11 @@ __global__ void __launch_bounds__(kPushThreads, 3)
             pn.o[d][dst] = o1;
             pn.u[d][dst] = uk[d];
           }
-          pn.w[dst] = p.w[idx[k]];
+          const float w = p.w[idx[k]];
+          pn.w[dst] = w;
           if (pn.id) pn.id[dst] = p.id[idx[k]];
-          key[k] = place_moved(P, g, tl, t, l, dc, good, origin_after, xlo, xhi, pos[k], ent[k], pn.cell + dst,
-                               keys + dst);
+          key[k] = place_moved(P, g, tl, t, l, dc, good, good && fabsf(w) < __int_as_float(sc[53]), origin_after, xlo, xhi, pos[k],
+                               ent[k], pn.cell + dst, keys + dst);
           if (key[k] == t) own += 1;
         }
       }
@@ -446,11 +461,13 @@ __global__ void __launch_bounds__(kPushThreads, 3)
       for (int d = 0; d < 3; ++d) {  // axes 0, 1, 2 of the arrays: d, e, f
         const int sd = L.sd(d, 5), se = L.se(d, 5), lo = L.part(d, 5);
         unsigned* j = sJ + L.start(d, 5) + (r[0] + 1) * sd + (r[1] + 1) * se + r[2] + 1;  // nodes c-1 .. c+2
+        const int sh = sc[50 + d] + 31 - sc[4 + d];
+        const long long half = (long long)(1u << (sh - 1));
         int Pi[2][3];
         {
           float2 S[4], D[4];
           shapes32(oa[0], ob[0], S, D);
-          const float scale = __int_as_float((127 + sc[4 + d]) << 23);
+          const float scale = __int_as_float((127 + sc[50 + d]) << 23);
           const float jc = d == 0 ? pc.jc[0] : (d == 1 ? pc.jc[1] : pc.jc[2]);
           const float2 c = mul2(mul2(dup2(jc), qw), dup2(scale));
           float2 run = make_float2(0.0f, 0.0f);
@@ -469,8 +486,8 @@ __global__ void __launch_bounds__(kPushThreads, 3)
           shapes32(oa[2], ob[2], S, D);
 #pragma unroll
           for (int m = 0; m < 4; ++m) {
-            ak[m] = mul2(dup2(kA30), fma2(dup2(0.5f), D[m], S[m]));
-            bk[m] = mul2(dup2(kA30), fma2(dup2(third), D[m], mul2(dup2(0.5f), S[m])));
+            ak[m] = mul2(dup2(kA31), fma2(dup2(0.5f), D[m], S[m]));
+            bk[m] = mul2(dup2(kA31), fma2(dup2(third), D[m], mul2(dup2(0.5f), S[m])));
           }
         }
         float2 S[4], D[4];
@@ -483,7 +500,7 @@ __global__ void __launch_bounds__(kPushThreads, 3)
             const int A0 = __float2int_rn(A.x), A1 = __float2int_rn(A.y);
 #pragma unroll
             for (int m = 0; m < 3; ++m)
-              add_current(j + m * sd + b * se + c, lo, mad_wide(Pi[1][m], A1, mad_wide(Pi[0][m], A0, kHalf28)));
+              add_current(j + m * sd + b * se + c, lo, mad_wide(Pi[1][m], A1, mad_wide(Pi[0][m], A0, half)), sh);
           }
         const int r0 = r[0];
         r[0] = r[1], r[1] = r[2], r[2] = r0;
@@ -492,7 +509,7 @@ __global__ void __launch_bounds__(kPushThreads, 3)
         ob[0] = ob[1], ob[1] = ob[2], ob[2] = v;
       }
     }
-    // particles that left their cell: 5-node windows where they moved
+    // particles that left their cell, on 5-node windows where they moved, and light ones
     const int ncross = sc[1];
     for (int i = tid; i < ncross; i += kPushThreads) {
       const int pos = P.cross[i];
@@ -522,10 +539,13 @@ __global__ void __launch_bounds__(kPushThreads, 3)
       for (int d = 0; d < 3; ++d) {
         const int sd = L.sd(d, 5), se = L.se(d, 5), lo = L.part(d, 5);
         unsigned* j = sJ + L.start(d, 5) + r[0] * sd + r[1] * se + r[2];
-        int Pi[4];
+        int Pi[4], sh;
         {
-          const float scale = __int_as_float((127 + sc[4 + d]) << 23);
-          const float c = (d == 0 ? pc.jc[0] : (d == 1 ? pc.jc[1] : pc.jc[2])) * qw * scale;
+          const float jq = (d == 0 ? pc.jc[0] : (d == 1 ? pc.jc[1] : pc.jc[2])) * qw;
+          const int ep = ((__float_as_int(0.76f * jq) >> 23) & 255) - 127, s = sc[4 + d];
+          const int kp = max(min(30 - ep, s), sc[50 + d]);
+          sh = kp + 31 - s;
+          const float c = jq * __int_as_float((127 + kp) << 23);
           float run = 0.0f;
 #pragma unroll
           for (int m = 0; m < 4; ++m) {
@@ -536,8 +556,8 @@ __global__ void __launch_bounds__(kPushThreads, 3)
         float ak[5], bk[5];
 #pragma unroll
         for (int m = 0; m < 5; ++m) {
-          ak[m] = kA30 * (S[2][m] + 0.5f * D[2][m]);
-          bk[m] = kA30 * (0.5f * S[2][m] + third * D[2][m]);
+          ak[m] = kA31 * (S[2][m] + 0.5f * D[2][m]);
+          bk[m] = kA31 * (0.5f * S[2][m] + third * D[2][m]);
         }
 #pragma unroll
         for (int b = 0; b < 5; ++b)
@@ -548,7 +568,8 @@ __global__ void __launch_bounds__(kPushThreads, 3)
                 const int A = __float2int_rn(S[1][b] * ak[c] + D[1][b] * bk[c]);
 #pragma unroll
                 for (int m = 0; m < 4; ++m)
-                  if (m < n[0] - 1) add_current(j + m * sd + b * se + c, lo, mad_wide(Pi[m], A, kHalf28));
+                  if (m < n[0] - 1)
+                    add_current(j + m * sd + b * se + c, lo, mad_wide(Pi[m], A, (long long)(1u << (sh - 1))), sh);
               }
           }
         const int r0 = r[0], n0 = n[0];
@@ -580,7 +601,7 @@ __global__ void __launch_bounds__(kPushThreads, 3)
               // T = top 2^21 + low, both exact as floats: one rounding
               const long long T = (long long)(int)hi * 4096 + (long long)(lo - (hi << 12));
               const float v = fmaf((float)(int)(T >> 21), 2097152.0f, (float)(int)(T & 0x1fffff));
-              atomicAdd(f.c[JX + d] + gi0 + P.tabz[lz], v * __int_as_float((126 - sc[4 + d]) << 23));  // 2^-(kp + 1)
+              atomicAdd(f.c[JX + d] + gi0 + P.tabz[lz], v * __int_as_float((127 - sc[4 + d]) << 23));  // 2^-s
             }
           }
         }

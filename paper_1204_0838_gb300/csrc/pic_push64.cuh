@@ -302,7 +302,7 @@ __global__ void __launch_bounds__(kPushThreads, 2)
         }
         pn.w[dst] = p.w[idx];
         if (pn.id) pn.id[dst] = p.id[idx];
-        key = place_moved(P, g, tl, t, l, dc, good, origin_after, xlo, xhi, pos, ent, pn.cell + dst, keys + dst);
+        key = place_moved(P, g, tl, t, l, dc, good, false, origin_after, xlo, xhi, pos, ent, pn.cell + dst, keys + dst);
         if (key == t) own += 1;
       }
       count_leaving(cnt_next, key, t);
