@@ -1,11 +1,15 @@
 // pic_push.cuh -- what the FP32 and FP64 particle pushes share: the layout of
 // a tile's fields and current in shared memory, and the ranking of a tile's
-// particles per cell.  One CTA takes one tile, in passes of up to kChunk
-// particles:
-//   stage E, B; rank the particles per cell and list them in (rank, cell)
-//   order; gather, push, move, writing the moved particles in that order to the
-//   second buffer; turn the staged fields' memory into the J tile; deposit the
-//   particles that stayed in their cell, then the others; add the tile to J.
+// particles per cell.  One CTA takes one tile, its particles in passes of up to
+// kChunk:
+//   stage E, B; in passes: rank the particles per cell and list them in (rank,
+//   cell) order; gather, push, move, writing the moved particles in that order to
+//   the second buffer; then turn the staged fields' memory into the J tile; in
+//   passes: deposit the particles that stayed in their cell, then the others; add
+//   the tile to J, once, whatever the number of passes: each add rounds.
+// A tile of more than one pass keeps the passes' lists in global memory between
+// the two phases, in the cells and momenta of the first buffer, which nothing
+// reads any more in the step.
 // In (rank, cell) order the lanes of a warp hold distinct neighbouring cells,
 // so that their reads and adds at one offset from their own cells collide
 // little, and the writes are coalesced and nearly sorted for the next step.
@@ -113,10 +117,12 @@ struct PushSmem {
 
 // Pointers into the shared memory of a CTA, and the scalars: [0] particles
 // without an ordered rank, [1] particles that deposit alone, [2, 4) sums or
-// maxima over the pass, [4, 7) J scale per component, [8, 16) scan partials,
+// maxima over the tile, [4, 7) J scale per component, [8, 16) scan partials,
 // [16, 33) first pair of each pair of ranks, [33] ordered particles, [34, 50)
 // first position of each pair of ranks, [50, 62) field scales (FP64), [50, 53)
 // scale of P per component and [53] the weight below which a particle is light (FP32).
+// All but [2, 8) and [50, 64) belong to a pass.
+constexpr int kPassScalars = 50;
 struct PushTile {
   int* hist;
   unsigned* mask;         // [rank][word]: cells that hold more than `rank` particles
@@ -148,6 +154,7 @@ __device__ __forceinline__ PushTile push_tile(unsigned char* smem, const Geom<T>
   P.tabz = P.taby + tl.ty + 5;
   P.sc = reinterpret_cast<int*>(smem + so.scal);
   const int rest = t / tl.ntz;
+  if (threadIdx.x < 64) P.sc[threadIdx.x] = 0;
   P.x0 = (rest / tl.nty) * tl.tx;
   P.y0 = (rest % tl.nty) * tl.ty;
   P.z0 = (t % tl.ntz) * tl.tz;
@@ -165,11 +172,51 @@ __device__ __forceinline__ PushTile push_tile(unsigned char* smem, const Geom<T>
   return P;
 }
 
-// Clear the ranking's scratch for a pass (a barrier must follow).
+// Clear the ranking's scratch for a pass (a barrier must follow; the tile's
+// scalars are cleared once).
 __device__ __forceinline__ void rank_clear(const PushTile& P, int W) {
   for (int i = threadIdx.x; i < 32 * W; i += kPushThreads) P.hist[i] = 0;
   for (int i = threadIdx.x; i < kRanks * W; i += kPushThreads) P.mask[i] = 0u;
-  if (threadIdx.x < 64) P.sc[threadIdx.x] = 0;
+  if (threadIdx.x < 2) P.sc[threadIdx.x] = 0;
+}
+
+// Particles [begin, begin + n) of pass ps of npass over a tile of ntile: sizes
+// within one of each other, so that none of several passes is below kChunk / 2.
+struct Pass {
+  int begin, n;
+  __device__ __forceinline__ Pass(int ps, int npass, int ntile) {
+    const int per = ntile / npass, more = ntile - per * npass;
+    begin = ps * per + min(ps, more);
+    n = per + (ps < more ? 1 : 0);
+  }
+};
+
+// Keep a pass's lists: the order list in its cells, the pairs (nitem entries, or
+// none), the particles that deposit alone and the scalars in its momenta.  Barriers
+// before and after.
+template <typename T>
+__device__ __forceinline__ void keep_lists(const PushTile& P, const Parts<T>& p, int c0, int nch, int nitem,
+                                           const unsigned short* pair) {
+  unsigned *c = reinterpret_cast<unsigned*>(p.cell + c0), *u0 = reinterpret_cast<unsigned*>(p.u[0] + c0),
+           *u1 = reinterpret_cast<unsigned*>(p.u[1] + c0), *u2 = reinterpret_cast<unsigned*>(p.u[2] + c0);
+  for (int i = threadIdx.x; i < nch; i += kPushThreads) c[i] = P.order[i];
+  for (int i = threadIdx.x; i < nitem; i += kPushThreads) u0[i] = pair[i];
+  for (int i = threadIdx.x; i < P.sc[1]; i += kPushThreads) u1[i] = P.cross[i];
+  if (threadIdx.x < kPassScalars) u2[threadIdx.x] = (unsigned)P.sc[threadIdx.x];
+}
+// Bring them back (from L2: the cells were read through other paths before).
+template <typename T>
+__device__ __forceinline__ void fetch_lists(const PushTile& P, const Parts<T>& p, int c0, int nch,
+                                            unsigned short* pair) {
+  const unsigned *c = reinterpret_cast<unsigned*>(p.cell + c0), *u0 = reinterpret_cast<unsigned*>(p.u[0] + c0),
+                 *u1 = reinterpret_cast<unsigned*>(p.u[1] + c0), *u2 = reinterpret_cast<unsigned*>(p.u[2] + c0);
+  const int n1 = (int)__ldcg(u2 + 1);
+  for (int i = threadIdx.x; i < nch; i += kPushThreads) {
+    P.order[i] = __ldcg(c + i);
+    if (pair) pair[i] = (unsigned short)__ldcg(u0 + i);
+    if (i < n1) P.cross[i] = (unsigned short)__ldcg(u1 + i);
+  }
+  if (threadIdx.x < kPassScalars && !(threadIdx.x >= 2 && threadIdx.x < 8)) P.sc[threadIdx.x] = (int)__ldcg(u2 + threadIdx.x);
 }
 
 constexpr int kPerThread = kChunk / kPushThreads;

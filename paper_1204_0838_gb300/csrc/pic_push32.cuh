@@ -41,7 +41,7 @@
 // take 65 % of the cycles; barriers and the latency of the particle loads share
 // the rest.
 //
-// Current: sums of integers at 2^s per pass and component, with s the largest
+// Current: sums of integers at 2^s per tile and component, with s the largest
 // for which B 2^s < 2^42, B = |q jc| sum |w|.  A contribution is a product of
 // two rounded integers, P = q w jc run at 2^kp, below 2^31, and A at 2^31; a
 // pair's P A are added exactly and rounded once, T = sum P A >> (kp + 31 - s),
@@ -50,7 +50,7 @@
 // lies in [2^12 hi, 2^12 (hi + n)) for n adds, n < 2^20; hi stays below 2^31.
 // So the sum does not depend on the order of the adds.  A contribution is
 // rounded by 2^-42 of B, and P, if less than that, by
-// - 2^-31 of the pass's largest |q w jc| for particles within 8 of the largest
+// - 2^-31 of the tile's largest |q w jc| for particles within 8 of the largest
 //   weight, which share kp: at most 2^-28 of their own |q w jc|, below the 2^-26
 //   or so that the FP32 shape factors leave in P itself;
 // - 2^-31 of its own |q w jc| for a lighter particle or one that left its cell:
@@ -227,16 +227,17 @@ __global__ void __launch_bounds__(kPushThreads, 3)
     atomicAdd(pushed, (unsigned long long)ntile);
     if (ntile >= (1 << 20)) atomicOr(err, 16);
   }
-  const int npass = (ntile + kChunk - 1) / kChunk, per_pass = (ntile + npass - 1) / npass;
+  const int npass = (ntile + kChunk - 1) / kChunk;
   int own = 0;
 
-  for (int ch0 = 0; ch0 < ntile; ch0 += per_pass) {
-    const int nch = min(per_pass, ntile - ch0), c0 = pbeg + ch0;
+  for (int ps = 0; ps < npass; ++ps) {
+    const Pass pass(ps, npass, ntile);
+    const int nch = pass.n, c0 = pbeg + pass.begin;
     rank_clear(P, W);
     __syncthreads();
 
     // stage E, B: a half warp per (x, y) row, the lanes along z
-    {
+    if (ps == 0) {
       const int SX = tl.tx + 4, SZ = tl.tz + 4;
       for (RowWalk r(tl.ty + 4); r.lx < SX; r.next()) {
         const int lx = r.lx, ly = r.ly;
@@ -257,13 +258,13 @@ __global__ void __launch_bounds__(kPushThreads, 3)
       asm volatile("cp.async.commit_group;" ::: "memory");
     }
 
-    // rank the pass's particles per cell; sum and maximum of |w|
+    // rank the pass's particles per cell; sum and maximum of |w| over the tile
     int sr[kPerThread];
     rank_count(P, L, g, tl, p.cell, c0, nch, sr, err);
-    {
+    if (ps == 0) {
       float ws = 0.0f, wm = 0.0f;
-      for (int k = tid; k < nch; k += kPushThreads) {
-        const float wa = fabsf(p.w[c0 + k]);
+      for (int k = tid; k < ntile; k += kPushThreads) {
+        const float wa = fabsf(p.w[pbeg + k]);
         ws += wa;
         wm = fmaxf(wm, wa);
       }
@@ -279,7 +280,7 @@ __global__ void __launch_bounds__(kPushThreads, 3)
     }
     __syncthreads();
     rank_masks(P, W);
-    if (tid < 3) {
+    if (ps == 0 && tid < 3) {
       // s: B 2^s < 2^42; kp: |P| 2^kp < 2^31 for P <= 0.76 |q| max w jc, no finer
       // than s.  B > Pm, so that 20 <= kp + 31 - s <= 31.
       const float jc = fabsf(pc.q * (tid == 0 ? pc.jc[0] : (tid == 1 ? pc.jc[1] : pc.jc[2])));
@@ -422,16 +423,31 @@ __global__ void __launch_bounds__(kPushThreads, 3)
       for (int k = 0; k < 2; ++k) count_leaving(cnt_next, key[k], t);
     }
     __syncthreads();
+    if (npass > 1) {
+      keep_lists(P, p, c0, nch, nitem, pairB);
+      __syncthreads();
+    }
+  }
 
-    // ---- the region becomes the J tile ----
-    {
-      int4* z = reinterpret_cast<int4*>(smem_raw);
-      const int n = (int)(so.order / 16);
-      for (int i = tid; i < n; i += kPushThreads) z[i] = make_int4(0, 0, 0, 0);
+  // ---- the region becomes the J tile ----
+  {
+    int4* z = reinterpret_cast<int4*>(smem_raw);
+    const int n = (int)(so.order / 16);
+    for (int i = tid; i < n; i += kPushThreads) z[i] = make_int4(0, 0, 0, 0);
+  }
+  for (int ps = 0; ps < npass; ++ps) {
+    const Pass pass(ps, npass, ntile);
+    const int nch = pass.n, c0 = pbeg + pass.begin;
+    if (npass > 1) {
+      __syncthreads();
+      fetch_lists(P, p, c0, nch, pairB);
     }
     __syncthreads();
+    const int ranked = sc[33];
+    const int nround = sc[16 + kRanks / 2];
+    const int nitem = nround + (nch - ranked);
     const float third = 1.0f / 3.0f;
-    round = 0;
+    int round = 0;
     for (int i = tid; i < nitem; i += kPushThreads) {
       int posA;
       if (i < nround) {
@@ -583,31 +599,30 @@ __global__ void __launch_bounds__(kPushThreads, 3)
         }
       }
     }
-    __syncthreads();
+  }
+  __syncthreads();
 
-    // flush: a half warp per (x, y) row, the lanes along z
-    {
-      const int NX = tl.tx + 5, NZ = tl.tz + 5;
-      for (RowWalk r(tl.ty + 5); r.lx < NX; r.next()) {
-        const int lx = r.lx, ly = r.ly;
-        const int gi0 = P.tabx[lx] + P.taby[ly];
-        for (int lz = tid & 15; lz < NZ; lz += 16) {
-          const int i3[3] = {lx, ly, lz};
+  // flush: a half warp per (x, y) row, the lanes along z
+  {
+    const int NX = tl.tx + 5, NZ = tl.tz + 5;
+    for (RowWalk r(tl.ty + 5); r.lx < NX; r.next()) {
+      const int lx = r.lx, ly = r.ly;
+      const int gi0 = P.tabx[lx] + P.taby[ly];
+      for (int lz = tid & 15; lz < NZ; lz += 16) {
+        const int i3[3] = {lx, ly, lz};
 #pragma unroll
-          for (int d = 0; d < 3; ++d) {
-            const unsigned* w = sJ + L.start(d, 5) + i3[d] * L.sd(d, 5) + i3[(d + 1) % 3] * L.se(d, 5) + i3[(d + 2) % 3];
-            const unsigned hi = w[0], lo = w[L.part(d, 5)];
-            if (hi | lo) {
-              // T = top 2^21 + low, both exact as floats: one rounding
-              const long long T = (long long)(int)hi * 4096 + (long long)(lo - (hi << 12));
-              const float v = fmaf((float)(int)(T >> 21), 2097152.0f, (float)(int)(T & 0x1fffff));
-              atomicAdd(f.c[JX + d] + gi0 + P.tabz[lz], v * __int_as_float((127 - sc[4 + d]) << 23));  // 2^-s
-            }
+        for (int d = 0; d < 3; ++d) {
+          const unsigned* w = sJ + L.start(d, 5) + i3[d] * L.sd(d, 5) + i3[(d + 1) % 3] * L.se(d, 5) + i3[(d + 2) % 3];
+          const unsigned hi = w[0], lo = w[L.part(d, 5)];
+          if (hi | lo) {
+            // T = top 2^21 + low, both exact as floats: one rounding
+            const long long T = (long long)(int)hi * 4096 + (long long)(lo - (hi << 12));
+            const float v = fmaf((float)(int)(T >> 21), 2097152.0f, (float)(int)(T & 0x1fffff));
+            atomicAdd(f.c[JX + d] + gi0 + P.tabz[lz], v * __int_as_float((127 - sc[4 + d]) << 23));  // 2^-s
           }
         }
       }
     }
-    __syncthreads();
   }
   own = __reduce_add_sync(0xffffffffu, own);
   if (lane == 0 && own) atomicAdd(cnt_next + t, own);

@@ -4,7 +4,7 @@
 //
 // The staged E and B become int64 at a power of two 2^sF per tile and
 // component with max|F| 2^sF < 2^58, and the J tile holds exact 64-bit sums as
-// two 32-bit words at 2^s per pass and component with B 2^s < 2^62, B a bound on
+// three 32-bit words at 2^s per tile and component with B 2^s < 2^62, B a bound on
 // every node's sum taken from the particles' speeds before the push: a cold or
 // slow tile gets a fine scale, not one sized for moves of a whole cell.
 //
@@ -64,7 +64,7 @@ __device__ __forceinline__ void add_current64(unsigned* j, int part, long long X
   red_u32(j + 2 * part, (unsigned)((int)h >> 8));
 }
 
-// The sum of X from the words' sums of up to kChunk adds: sum (X >> 40) is exact
+// The sum of X from the words' sums of up to kChunk + 1 adds: sum (X >> 40) is exact
 // (the sum itself is below 2^62); sum (X >> 20) lies within n 2^20 < 2^32 above
 // 2^20 times it, and sum X within n 2^20 above 2^20 times that.
 __device__ __forceinline__ long long sum_current64(unsigned w0, unsigned w1, unsigned w2) {
@@ -73,7 +73,7 @@ __device__ __forceinline__ long long sum_current64(unsigned w0, unsigned w1, uns
   const long long c = b << 20;
   return c + (long long)(w0 - (unsigned)c);
 }
-static_assert(kChunk < 4096, "the words' overlap holds the carries of 2^12 adds");
+static_assert(kChunk + 1 < 4096, "the words' overlap holds the carries of 2^12 adds");
 
 template <bool FIXED>
 __global__ void __launch_bounds__(kPushThreads, 2)
@@ -95,18 +95,19 @@ __global__ void __launch_bounds__(kPushThreads, 2)
   const int W = L.words();
   const int ntile = pend - pbeg;
   if (tid == 0) atomicAdd(pushed, (unsigned long long)ntile);
-  const int npass = (ntile + kChunk - 1) / kChunk, per_pass = (ntile + npass - 1) / npass;
+  const int npass = (ntile + kChunk - 1) / kChunk;
   int own = 0;
 
-  for (int ch0 = 0; ch0 < ntile; ch0 += per_pass) {
-    const int nch = min(per_pass, ntile - ch0), c0 = pbeg + ch0;
+  for (int ps = 0; ps < npass; ++ps) {
+    const Pass pass(ps, npass, ntile);
+    const int nch = pass.n, c0 = pbeg + pass.begin;
     rank_clear(P, W);
     __syncthreads();
 
     // Stage E_d (part 0) and B_e, e the axis after d (part 1): a half warp per
     // (x, y) row, the lanes along z; take the largest exponent of each.
     const int SX = tl.tx + 4, SZ = tl.tz + 4;
-    {
+    if (ps == 0) {
       int emax[6] = {0, 0, 0, 0, 0, 0};
       for (RowWalk r(tl.ty + 4); r.lx < SX; r.next()) {
         const int lx = r.lx, ly = r.ly;
@@ -137,11 +138,11 @@ __global__ void __launch_bounds__(kPushThreads, 2)
     }
     int sr[kPerThread];
     rank_count(P, L, g, tl, p.cell, c0, nch, sr, err);
-    {
+    if (ps == 0) {  // over the tile
       float su = 0.0f, sw = 0.0f;
-      for (int k = tid; k < nch; k += kPushThreads) {
-        const float wa = fabsf((float)p.w[c0 + k]);
-        const float ux = (float)p.u[0][c0 + k], uy = (float)p.u[1][c0 + k], uz = (float)p.u[2][c0 + k];
+      for (int k = tid; k < ntile; k += kPushThreads) {
+        const float wa = fabsf((float)p.w[pbeg + k]);
+        const float ux = (float)p.u[0][pbeg + k], uy = (float)p.u[1][pbeg + k], uz = (float)p.u[2][pbeg + k];
         su += wa * fminf(1.0f, sqrtf(ux * ux + uy * uy + uz * uz));
         sw += wa;
       }
@@ -157,13 +158,13 @@ __global__ void __launch_bounds__(kPushThreads, 2)
     }
     __syncthreads();
     rank_masks(P, W);
-    if (tid < 3) {
+    if (ps == 0 && tid < 3) {
       // |E| <= sqrt 3 max_c |E_c| < sqrt 3 2^(emax - 1022)
       const int eE = max(max(sc[50], sc[52]), sc[54]);
       const float kick = eE == 0 ? 0.0f : ldexpf(3.4642f * fabsf((float)pc.h), eE - 1022);
       sc[4 + tid] = j64_scale(pc, tid, __int_as_float(sc[2]), __int_as_float(sc[3]), kick);
     }
-    if (tid < 6) {
+    if (ps == 0 && tid < 6) {
       // max|F| 2^sF < 2^58; a non-finite value is reported
       const int e = sc[50 + tid];
       if (e == 0x7FF) atomicOr(err, 8);
@@ -171,7 +172,7 @@ __global__ void __launch_bounds__(kPushThreads, 2)
     }
     __syncthreads();
     rank_order(P, W, nch, sr);
-    {
+    if (ps == 0) {
       // the staged doubles become split fixed-point words in place
       int emax[6];
 #pragma unroll
@@ -308,12 +309,37 @@ __global__ void __launch_bounds__(kPushThreads, 2)
       count_leaving(cnt_next, key, t);
     }
     __syncthreads();
+    if (npass > 1) {
+      keep_lists(P, p, c0, nch, 0, nullptr);
+      __syncthreads();
+    }
+  }
 
-    // ---- the region becomes the J tile ----
-    {
-      int4* z = reinterpret_cast<int4*>(smem_raw);
-      const int n = (int)(so.order / 16);
-      for (int i = tid; i < n; i += kPushThreads) z[i] = make_int4(0, 0, 0, 0);
+  // ---- the region becomes the J tile ----
+  {
+    int4* z = reinterpret_cast<int4*>(smem_raw);
+    const int n = (int)(so.order / 16);
+    for (int i = tid; i < n; i += kPushThreads) z[i] = make_int4(0, 0, 0, 0);
+  }
+  for (int ps = 0; ps < npass; ++ps) {
+    const Pass pass(ps, npass, ntile);
+    const int nch = pass.n, c0 = pbeg + pass.begin;
+    if (npass > 1) {
+      __syncthreads();
+      if (ps > 0) {  // the sums so far as the words of one add (see sum_current64)
+#pragma unroll 1
+        for (int d = 0; d < 3; ++d) {
+          const int n = L.part(d, 5);
+          unsigned* w = sJ + L.start(d, 5);
+          for (int i = tid; i < n; i += kPushThreads) {
+            const long long X = sum_current64(w[i], w[i + n], w[i + 2 * n]);
+            w[i] = (unsigned)X;
+            w[i + n] = (unsigned)(X >> 20);
+            w[i + 2 * n] = (unsigned)(X >> 40);
+          }
+        }
+      }
+      fetch_lists(P, p, c0, nch, (unsigned short*)nullptr);
     }
     __syncthreads();
     // 2 P 2^s = 2 q w jc run 2^s, below 2^63 by the choice of the scale; run at 2^62
@@ -462,26 +488,25 @@ __global__ void __launch_bounds__(kPushThreads, 2)
         }
       }
     }
-    __syncthreads();
+  }
+  __syncthreads();
 
-    // flush: a half warp per (x, y) row, the lanes along z
-    {
-      const int NX = tl.tx + 5, NZ = tl.tz + 5;
-      for (RowWalk r(tl.ty + 5); r.lx < NX; r.next()) {
-        const int lx = r.lx, ly = r.ly;
-        const int gi0 = P.tabx[lx] + P.taby[ly];
-        for (int lz = tid & 15; lz < NZ; lz += 16) {
-          const int i3[3] = {lx, ly, lz};
+  // flush: a half warp per (x, y) row, the lanes along z
+  {
+    const int NX = tl.tx + 5, NZ = tl.tz + 5;
+    for (RowWalk r(tl.ty + 5); r.lx < NX; r.next()) {
+      const int lx = r.lx, ly = r.ly;
+      const int gi0 = P.tabx[lx] + P.taby[ly];
+      for (int lz = tid & 15; lz < NZ; lz += 16) {
+        const int i3[3] = {lx, ly, lz};
 #pragma unroll
-          for (int d = 0; d < 3; ++d) {
-            const unsigned* w = sJ + L.start(d, 5) + i3[d] * L.sd(d, 5) + i3[(d + 1) % 3] * L.se(d, 5) + i3[(d + 2) % 3];
-            const long long X = sum_current64(w[0], w[L.part(d, 5)], w[2 * L.part(d, 5)]);
-            if (X != 0) atomicAdd(f.c[JX + d] + gi0 + P.tabz[lz], fixed_to_double(X, sc[4 + d]));
-          }
+        for (int d = 0; d < 3; ++d) {
+          const unsigned* w = sJ + L.start(d, 5) + i3[d] * L.sd(d, 5) + i3[(d + 1) % 3] * L.se(d, 5) + i3[(d + 2) % 3];
+          const long long X = sum_current64(w[0], w[L.part(d, 5)], w[2 * L.part(d, 5)]);
+          if (X != 0) atomicAdd(f.c[JX + d] + gi0 + P.tabz[lz], fixed_to_double(X, sc[4 + d]));
         }
       }
     }
-    __syncthreads();
   }
   own = __reduce_add_sync(0xffffffffu, own);
   if (lane == 0 && own) atomicAdd(cnt_next + t, own);
