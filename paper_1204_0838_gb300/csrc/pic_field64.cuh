@@ -28,9 +28,6 @@
 
 namespace pic {
 
-constexpr int kFieldBits = 60;    // max|F| 2^s < 2^60
-constexpr int kFieldMinExp = 82;  // smallest biased exponent that sets a scale (s <= 1000)
-
 // Constant weights, split: smoothing centre, two edges, corner per axis at 2^62;
 // dt/2 / d at 2^63 and dt / d at 2^62 per axis.
 struct FieldConst64 {
@@ -55,16 +52,6 @@ __device__ __forceinline__ bool block_scales(const int (&emax)[3], int* sh, int 
     e[c] = max(sh[c], kFieldMinExp);
   }
   return finite;
-}
-
-// round(v 2^s) of a double's bits, s = kFieldBits - 1 + 1023 - emax.
-__device__ __forceinline__ long long block_fixed(long long b, int emax) {
-  const int e = (int)((b >> 52) & 0x7FF);
-  const unsigned long long m = (unsigned long long)(b & 0xFFFFFFFFFFFFFLL) | 0x10000000000000ull;
-  unsigned long long X = (m << 8) >> min(emax - e, 63);  // one bit below the unit
-  X = e == 0 ? 0ull : (X + 1) >> 1;
-  const long long n = b >> 63;
-  return ((long long)X ^ n) - n;
 }
 
 // x w / 2^63 (one product), one bit more than x w / 2^64.
@@ -147,7 +134,7 @@ __global__ void __launch_bounds__(256, 2)
     const int q = tid + 256 * t;
     if (q < EB_N)
 #pragma unroll
-      for (int c = 0; c < 3; ++c) sB[c][q] = block_fixed(raw[t][c], e[c]);
+      for (int c = 0; c < 3; ++c) sB[c][q] = field_fixed(raw[t][c], e[c]);
   }
   __syncthreads();
   int sc[3];  // scale of the products
@@ -267,7 +254,7 @@ __global__ void __launch_bounds__(256, 2)
         const int q = tid + 256 * t;
         if (q < CE_N)
 #pragma unroll
-          for (int c = 0; c < 3; ++c) sE[c * CE_N + q] = block_fixed(raw[t][c], e[c]);
+          for (int c = 0; c < 3; ++c) sE[c * CE_N + q] = field_fixed(raw[t][c], e[c]);
       }
   }
   if (!finite) {  // uniform over the block

@@ -17,9 +17,10 @@
 // add up no drift, and a sum of products of zeros is zero.
 //
 // Scales and the range of M (|M| + 2^31 < 2^63):
-// - gather: fields |x| < 2^58 at 2^sF, weights at 2^63 (at most 2/3, products
-//   of two at most 4/9): a sum of 16 has |sum xh wl| < 16 x 2^26 x 2^31 and
-//   |sum xl wh| <= 2^31 x 2^31, since the weights sum to at most one;
+// - gather: fields |x| < 2^60 at 2^sF, weights at 2^63 (at most 2/3, products
+//   of two at most 4/9): sums of 8 have |sum xh wl| <= 8 x 2^28 x 2^31 = 2^62, and
+//   their high words go to the first accumulator before more is added; sums of
+//   16 have |sum xl wh| <= 2^31 x (2^31 + 16), since the weights sum to one;
 // - deposit factors: S and D = S1 - S of one axis at 2^62, |S| + |D| <= 6/5,
 //   times factors at 2^63 that are at most 2/3 and 1/3:
 //   |M| <= 2^62 (3/5 + 2/3 + 1/3);
@@ -91,12 +92,14 @@ __device__ __forceinline__ long long to_fixed(double v, int k) {
   return b < 0 ? -X : X;
 }
 
-// A staged field value v as round(v 2^k), k = 57 + 1023 - emax for the tile's
-// largest biased exponent emax (below 2047): |v| 2^k < 2^58.
+// A staged field value v as round(v 2^k), k = 59 + 1023 - emax for the largest
+// biased exponent emax of a tile or block (below 2047): |v| 2^k < 2^60.
+constexpr int kFieldBits = 60;
+constexpr int kFieldMinExp = 82;  // smallest biased exponent that sets a scale (k <= 1000)
 __device__ __forceinline__ long long field_fixed(long long b, int emax) {
   const int e = (int)((b >> 52) & 0x7FF);
   const unsigned long long m = (unsigned long long)(b & 0xFFFFFFFFFFFFFLL) | 0x10000000000000ull;
-  unsigned long long X = (m << 6) >> min(emax - e, 63);  // one bit below the unit
+  unsigned long long X = (m << 8) >> min(emax - e, 63);  // one bit below the unit
   X = e == 0 ? 0ull : (X + 1) >> 1;
   const long long n = b >> 63;
   return ((long long)X ^ n) - n;
@@ -168,7 +171,7 @@ __device__ __forceinline__ long long gather64(const int2* __restrict__ s, int sd
     // the two cross sums apart: three chains of multiply-adds instead of two
     long long H = 0, M = kRound2, N = 0;
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < 4; ++i) {
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const int2 v = s[i * sd + j * se + c];
@@ -176,6 +179,11 @@ __device__ __forceinline__ long long gather64(const int2* __restrict__ s, int sd
         M = mad_wide(v.y, wde[i][j].lo, M);
         N = mad_wide(v.x, wde[i][j].hi, N);
       }
+      if (i & 1) {  // M stays below 2^62 + 2^32 (see above)
+        H += M >> 32;
+        M = (long long)(unsigned)M;
+      }
+    }
     const Acc32 a = {H, M + N};
     acc32(sum, split32(acc32_result2(a)), wf[c]);
   }

@@ -3,7 +3,7 @@
 // in 64-bit fixed point on the integer pipes (pic_fixed64.cuh).
 //
 // The staged E and B become int64 at a power of two 2^sF per tile and
-// component with max|F| 2^sF < 2^58, and the J tile holds exact 64-bit sums as
+// component with max|F| 2^sF < 2^60, and the J tile holds exact 64-bit sums as
 // three 32-bit words at 2^s per tile and component with B 2^s < 2^62, B a bound on
 // every node's sum taken from the particles' speeds before the push: a cold or
 // slow tile gets a fine scale, not one sized for moves of a whole cell.
@@ -36,9 +36,7 @@
 
 namespace pic {
 
-constexpr int kField64Range = 58;  // staged fields: 16-term sums need |x| < 2^58
-constexpr int kFieldExpMin = 80;   // smallest biased exponent that sets a scale (sF <= 1000)
-constexpr int kJ64Range = 62;      // J sums
+constexpr int kJ64Range = 62;  // J sums
 
 // Scale exponent of the J tile for component c: B 2^s < 2^62 with B = 1.001 |q|
 // S / (dt d_b d_c), S a bound on sum |w| |running sum|.  A particle moves at
@@ -165,10 +163,10 @@ __global__ void __launch_bounds__(kPushThreads, 2)
       sc[4 + tid] = j64_scale(pc, tid, __int_as_float(sc[2]), __int_as_float(sc[3]), kick);
     }
     if (ps == 0 && tid < 6) {
-      // max|F| 2^sF < 2^58; a non-finite value is reported
+      // max|F| 2^sF < 2^60; a non-finite value is reported
       const int e = sc[50 + tid];
       if (e == 0x7FF) atomicOr(err, 8);
-      sc[56 + tid] = kField64Range - 1 - (max(e, kFieldExpMin) - 1023);
+      sc[56 + tid] = kFieldBits - 1 - (max(e, kFieldMinExp) - 1023);
     }
     __syncthreads();
     rank_order(P, W, nch, sr);
@@ -176,7 +174,7 @@ __global__ void __launch_bounds__(kPushThreads, 2)
       // the staged doubles become split fixed-point words in place
       int emax[6];
 #pragma unroll
-      for (int k = 0; k < 6; ++k) emax[k] = max(sc[50 + k], kFieldExpMin);
+      for (int k = 0; k < 6; ++k) emax[k] = max(sc[50 + k], kFieldMinExp);
       for (RowWalk r(tl.ty + 4); r.lx < SX; r.next()) {
         const int lx = r.lx, ly = r.ly;
         for (int lz = tid & 15; lz < SZ; lz += 16) {
