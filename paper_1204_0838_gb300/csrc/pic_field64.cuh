@@ -61,10 +61,16 @@ __device__ __forceinline__ long long scaled(long long x, S32 w) {
   return acc32_result2(a);
 }
 
-// a - b for a at scale sa, b at sb, at the coarser of the two.
+// a - b for a at scale sa, b at sb, at the coarser of the two; the finer one is
+// rounded to nearest (cut off, it would give the increments of a block a mean error
+// of half a unit that recurs every step).  |a|, |b| < 2^61.
+__device__ __forceinline__ long long coarser(long long a, int sh) {
+  const int r = min(sh, 62);
+  return (a + ((1LL << r) >> 1)) >> r;
+}
 __device__ __forceinline__ long long aligned_diff(long long a, int sa, long long b, int sb) {
   const int s = min(sa, sb);
-  return (a >> min(sa - s, 63)) - (b >> min(sb - s, 63));
+  return coarser(a, sa - s) - coarser(b, sb - s);
 }
 
 // E^{n+1} = E^n + dt (curl B^{n+1/2} - J); hb holds B^{n+1/2}.

@@ -1,7 +1,7 @@
 """The integer arithmetic of staged fields (csrc/pic_fixed64.cuh, pic_field64.cuh) in
 exact integers, on the CPU: the conversion of doubles at a tile's or block's scale, of
-offsets at 2^63, the range of the gather's sums at 60 bits, and the range and the error
-of the smoothing.
+offsets at 2^63, the range of the gather's sums at 60 bits, the range and the error of
+the smoothing, and the rounding of one term of a difference to the other's scale.
 """
 import random
 import struct
@@ -108,3 +108,20 @@ def test_smoothing_stays_in_range():
                 got = 2 * H + (M >> 31)
                 want = F(sum(t * w for t, w in zip(terms, weights)), 1 << 63)
                 assert abs(got - want) <= F(5, 2)  # four dropped products at twice the scale, the shift
+
+
+def coarser(a, sh):
+    r = min(sh, 62)
+    x = a + ((1 << r) >> 1)
+    assert abs(x) < 1 << 63
+    return x >> r
+
+
+def test_the_finer_term_of_a_difference_rounds_to_nearest():
+    rng = random.Random(5)
+    top = (1 << 61) - 1
+    for sh in (0, 1, 2, 20, 59, 60, 61, 62, 63, 900):
+        for a in (0, 1, -1, top, -top, rng.randrange(-top, top), rng.randrange(-top, top)):
+            assert abs(coarser(a, sh) - F(a, 1 << sh)) <= F(1, 2)
+    errs = [coarser(a, 20) - a / 2 ** 20 for a in (rng.randrange(-(1 << 40), 1 << 40) for _ in range(20000))]
+    assert abs(sum(errs) / len(errs)) < 0.02  # 0.29 / sqrt(20000) = 0.002
