@@ -109,10 +109,10 @@ typedef struct pic_grid {
   int precision;        /* PIC_FP64 or PIC_FP32 (FP32: fields, momenta, offsets,
                            currents; the window accumulator and diagnostic
                            reductions stay FP64).  FP64 gathers and deposits
-                           in 64-bit fixed point scaled per cell tile, and
-                           forms the field update's increments so per block
-                           of 4x8x32 cells: the absolute precision of FP64 at
-                           the tile's or block's largest values               */
+                           in 64-bit fixed point scaled per cell tile, with the
+                           absolute precision of FP64 at the tile's largest
+                           values; the field update keeps FP64's relative
+                           precision cell by cell                             */
   int bc_x;             /* PIC_BC_PERIODIC or PIC_BC_OPEN                      */
   int solver;           /* PIC_SOLVER_PERFECT (the paper's method) or
                            PIC_SOLVER_YEE (normal dispersion, for comparison;

@@ -371,7 +371,10 @@ FieldConst64 field_const64(const pic_t* h) {
   const double d[3] = {h->dx, h->dy, h->dz};
   for (int a = 0; a < 3; ++a) {
     const double s[4] = {h->sm_a[a], h->sm_b1[a], h->sm_b2[a], h->sm_g[a]};
-    for (int k = 0; k < 4; ++k) w.s[a][k] = split(s[k], 62);
+    for (int k = 0; k < 4; ++k) {
+      w.s[a][k] = split(s[k], 62);
+      w.s17[a][k] = w.s[a][k].lo >> 17;
+    }
     w.hd[a] = split(0.5 * h->dt / d[a], 63);
     w.fd[a] = split(h->dt / d[a], 62);
   }
@@ -380,11 +383,19 @@ FieldConst64 field_const64(const pic_t* h) {
   return w;
 }
 
-// Blocks of the field kernels over all slabs, or over the two edge slabs.
+// Blocks of the field kernels over all slabs, or over the two edge slabs: FP32 (x, y,
+// z); FP64, whose blocks are shorter along z, (z, y, x), for the launch grid's limits.
+template <typename T>
 dim3 field_blocks(const pic_t* h, bool edges = false) {
+  if (sizeof(T) == 8)
+    return dim3((h->nz + FB_Z - 1) / FB_Z, (h->ny + FB_Y - 1) / FB_Y, edges ? 2 : (h->nx + FB_X - 1) / FB_X);
   return dim3(edges ? 2 : (h->nx + CB_X - 1) / CB_X, (h->ny + CB_Y - 1) / CB_Y, (h->nz + CB_Z - 1) / CB_Z);
 }
-FieldSpan field_span(const pic_t* h, bool edges) { return edges ? FieldSpan{h->nx - 1, 1} : FieldSpan{CB_X, CB_X}; }
+template <typename T>
+FieldSpan field_span(const pic_t* h, bool edges) {
+  const int b = sizeof(T) == 8 ? FB_X : CB_X;
+  return edges ? FieldSpan{h->nx - 1, 1} : FieldSpan{b, b};
+}
 
 // Electric step.
 void launch_e_update(const pic_t* h, const Geom<float>& g, cudaStream_t s) {
@@ -392,20 +403,20 @@ void launch_e_update(const pic_t* h, const Geom<float>& g, cudaStream_t s) {
                                                                     field_coef<float>(h), pml_view<float>(h));
 }
 void launch_e_update(const pic_t* h, const Geom<double>& g, cudaStream_t s) {
-  k_e_update64<<<field_blocks(h), 256, 0, s>>>(g, fields<double>(h), half_b<double>(h), field_coef<double>(h),
+  k_e_update64<<<field_blocks<double>(h), 256, 0, s>>>(g, fields<double>(h), half_b<double>(h), field_coef<double>(h),
                                                       field_const64(h), pml_view<double>(h));
 }
 
 // Magnetic half steps over all slabs or the two edge slabs (see k_curl_tiled).
 void launch_curl(const pic_t* h, const Geom<float>& g, int mode, bool edges, cudaStream_t s) {
-  k_curl_tiled<float><<<field_blocks(h, edges), 256, curl_tiled_smem_bytes<float>(), s>>>(
-      g, smooth<float>(h), fields<float>(h), half_b<float>(h), field_coef<float>(h), mode, field_span(h, edges),
+  k_curl_tiled<float><<<field_blocks<float>(h, edges), 256, curl_tiled_smem_bytes<float>(), s>>>(
+      g, smooth<float>(h), fields<float>(h), half_b<float>(h), field_coef<float>(h), mode, field_span<float>(h, edges),
       pml_view<float>(h));
 }
 void launch_curl(const pic_t* h, const Geom<double>& g, int mode, bool edges, cudaStream_t s) {
-  k_curl64<<<field_blocks(h, edges), 256, kCurl64Smem, s>>>(g, smooth<double>(h), fields<double>(h), half_b<double>(h),
+  k_curl64<<<field_blocks<double>(h, edges), 256, kCurl64Smem, s>>>(g, smooth<double>(h), fields<double>(h), half_b<double>(h),
                                                         field_coef<double>(h), field_const64(h), mode,
-                                                        field_span(h, edges), pml_view<double>(h));
+                                                        field_span<double>(h, edges), pml_view<double>(h));
 }
 
 // H = B - (dt/2) curl'(E) over all slabs or the two edge slabs.

@@ -3,24 +3,24 @@
 //
 // What bounded the FP64 kernels that these replace: the FP64 pipe, 77-83 % busy
 // (about 110 FP64 instructions per cell and step; this GPU retires 0.5 T/s of
-// them).  Here a CTA stages a 4x8x32 block of a field with its halo, converts it
+// them).  Here a CTA stages an 8x8x16 block of a field with its halo, converts it
 // to int64 at a power of two per block and component with max|F| 2^s < 2^60, and
 // forms differences, the smoothing's sums and the products with constant
 // weights as integers (pic_fixed64.cuh); 6 FP64 instructions per cell and kernel
 // are left, which add the increments to the stored fields.
 //
-// Measured: step of a vacuum box of 8.4 M cells 2.00 -> 0.87 ms (magnetic kernel
-// 1.6 -> 0.47, electric kernel 0.45 -> 0.30; the 12 values read and written per
-// cell and kernel are 0.24 ms at the copy rate); 118 M particle step on 101 M cells
-// 93 -> 80 ms.  About 560 (electric) and 990 (magnetic) instructions per 32 cells,
-// issued 40-45 % of the time, bound both; half of them convert between doubles
-// and integers.
+// An increment's error is 2^-60 to 2^-61 of the block's largest value (rms).  Where
+// that is more than FP64 arithmetic would make of the values at hand, the derivative
+// is formed in FP64 (WeakTest): 0.7 % of them in a laser pulse in vacuum, 4 % around a
+// tightly focused one in plasma.  Each component of a curl takes the coarser scale of
+// the two that enter it.  A block that holds a NaN, an infinity or a value above 2^1021
+// takes FP64 arithmetic, cell by cell, so that non-finite values spread as they do in
+// FP64.
 //
-// The increments carry an absolute error of a few units of 2^-59 of the block's
-// largest value, below the 2^-53 rounding of that value itself; each component
-// of a curl takes the coarser scale of the two components that enter it.  A
-// block that holds a NaN or an infinity takes the FP64 arithmetic instead, cell
-// by cell, so that non-finite values spread as they do in FP64.
+// Measured, FP64 arithmetic -> here: step of a vacuum box of 8.4 M cells 2.00 -> 1.03 ms
+// (magnetic kernel 1.6 -> 0.60, electric kernel 0.45 -> 0.35; the 12 values read and
+// written per cell and kernel are 0.24 ms at the copy rate).  Without the test and what
+// it sends to FP64 the two kernels took 0.47 and 0.30 ms.
 #pragma once
 
 #include "pic_fixed64.cuh"
@@ -28,42 +28,90 @@
 
 namespace pic {
 
-// Constant weights, split: smoothing centre, two edges, corner per axis at 2^62;
-// dt/2 / d at 2^63 and dt / d at 2^62 per axis.
+// A block of cells, with the staged fields one cell beyond it, and the points of the
+// smoothed fields S_x Ey, S_x Ez; S_y Ez, S_y Ex; S_z Ex, S_z Ey.  Compact, for one
+// scale to serve it: along z above all, where a pulse falls off.  (4x8x32 blocks, with
+// products two bits coarser and the test's bounds accordingly: four to six times as many
+// derivatives in FP64, vacuum step 1.44 ms instead of 1.09.)
+constexpr int FB_X = 8, FB_Y = 8, FB_Z = 16;
+constexpr int FE_X = FB_X + 2, FE_Y = FB_Y + 2, FE_Z = FB_Z + 2;
+constexpr int FE_N = FE_X * FE_Y * FE_Z;
+constexpr int FXN = (FB_X + 1) * FB_Y * FB_Z, FYN = FB_X * (FB_Y + 1) * FB_Z, FZN = FB_X * FB_Y * (FB_Z + 1);
+static_assert(FB_Z == 16 && FB_Y % 2 == 0, "a warp: two rows of 16 cells in one x slab");
+
+// Constant weights, split: smoothing centre, two edges, corner per axis at 2^62, and
+// the upper 15 bits of their low words; dt/2 / d at 2^63 and dt / d at 2^62 per axis.
 struct FieldConst64 {
   S32 s[3][4];
+  int s17[3][4];
   S32 hd[3], fd[3];
   double idt, ihdt;  // 1 / dt, 2 / dt
 };
 
-// Largest exponent of the block's values, per component (sh: 3 shared ints,
-// zero on entry; barriers inside).  Returns false if a value is not finite.
-__device__ __forceinline__ bool block_scales(const int (&emax)[3], int* sh, int (&e)[3]) {
+// High word of a double's magnitude: its exponent and leading bits.
+__device__ __forceinline__ int high_bits(long long b) { return (int)((unsigned long long)b >> 32) & 0x7FFFFFFF; }
+__device__ __forceinline__ int high_bits(double v) { return __double2hiint(v) & 0x7FFFFFFF; }
+
+// Largest exponent of the block's values per component, from the largest high words
+// (sh: 3 shared ints, zero on entry; barriers inside).  Returns false if a value is
+// not finite, or so large that a sum may not be.
+__device__ __forceinline__ bool block_scales(const int (&hmax)[3], int* sh, int (&e)[3]) {
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    const unsigned m = __reduce_max_sync(0xffffffffu, (unsigned)emax[c]);
+    const unsigned m = __reduce_max_sync(0xffffffffu, (unsigned)hmax[c]);
     if ((threadIdx.x & 31) == 0) atomicMax(sh + c, (int)m);
   }
   __syncthreads();
   bool finite = true;
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    finite = finite && sh[c] != 0x7FF;
-    e[c] = max(sh[c], kFieldMinExp);
+    finite = finite && sh[c] < 0x7FC00000;
+    e[c] = max(sh[c] >> 20, kFieldMinExp);
   }
   return finite;
 }
 
-// x w / 2^63 (one product), one bit more than x w / 2^64.
+// The six derivatives of a curl, in the order of CurlD, are of the components z, y, x,
+// z, y, x; two by two they enter the components x, y, z of the curl.  One that takes
+// part from values far below the block's largest keeps its precision only in FP64.
+// It is strong if one of its operands, at the cell or up to two cells to either side
+// along z, comes within a bound of the largest value M of its component, or if the
+// value that takes the increment does.  The bounds lie where the error in fixed point
+// is that of FP64 in the operands or in the sum (2^-54.3 of it, rms):
+//   magnetic: 2^-61.4 M against 2^-54 of the smoothed operands; 2^-8 to 2^-7 of M, and
+//   2^-7 to 2^-6 for the sum;
+//   electric: 2^-60.2 M against the 2^-53.8 that the operands carry; 2^-7 to 2^-6 both.
+// All lanes of a warp, two rows of cells, call.
+struct WeakTest {
+  unsigned window;
+  int least;      // high word from which an operand is strong
+  int target[3];  // high word from which the sum is strong, per differentiated component
+  __device__ __forceinline__ WeakTest(const int (&e)[3], const int* sh, int least_bit) : least(1 << (least_bit - 32)) {
+    const int lane = threadIdx.x & 15;
+    window = ((0x1Fu << lane >> 2) & 0xFFFFu) << (threadIdx.x & 16);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) target[c] = sh[c] == 0 ? -1 : (e[c] - 6) << 20;  // an all-zero component is exact
+  }
+  // bit n if derivative n, with operands x and y, is weak; hi: high word of the value
+  // that takes the increment (-1: not to be looked at)
+  __device__ __forceinline__ unsigned operator()(int n, long long x, long long y, int hi) const {
+    const int a = (int)(x >> 32), b = (int)(y >> 32);
+    const bool near = __ballot_sync(0xffffffffu, ((a ^ (a >> 31)) | (b ^ (b >> 31))) >= least) & window;
+    return !near && hi < target[2 - n % 3] ? 1u << n : 0u;
+  }
+};
+
+// x w / 2^(64 - K) (one product).
+template <int K>
 __device__ __forceinline__ long long scaled(long long x, S32 w) {
-  Acc32 a = {0LL, kRound2};
+  Acc32 a = {0LL, 1LL << (31 - K)};
   acc32(a, split32(x), w);
-  return acc32_result2(a);
+  return (a.H << K) + (a.M >> (32 - K));
 }
 
 // a - b for a at scale sa, b at sb, at the coarser of the two; the finer one is
 // rounded to nearest (cut off, it would give the increments of a block a mean error
-// of half a unit that recurs every step).  |a|, |b| < 2^61.
+// of half a unit that recurs every step).  |a|, |b| <= 2^61.
 __device__ __forceinline__ long long coarser(long long a, int sh) {
   const int r = min(sh, 62);
   return (a + ((1LL << r) >> 1)) >> r;
@@ -74,20 +122,20 @@ __device__ __forceinline__ long long aligned_diff(long long a, int sa, long long
 }
 
 // E^{n+1} = E^n + dt (curl B^{n+1/2} - J); hb holds B^{n+1/2}.
-constexpr int EB_N = (CB_X + 1) * (CB_Y + 1) * (CB_Z + 1);
+constexpr int EB_N = (FB_X + 1) * (FB_Y + 1) * (FB_Z + 1);
 __global__ void __launch_bounds__(256, 2)
     k_e_update64(Geom<double> g, Fields<double> f, Fields<double> hb, FieldCoef<double> fc, FieldConst64 k64,
                  Pml<double> pm) {
   if (!dyn_prologue(g)) return;
   __shared__ long long sB[3][EB_N];  // origin (bx-1, by-1, bz-1)
   __shared__ int sh[3];
-  const int bx = blockIdx.x * CB_X, by = blockIdx.y * CB_Y, bz = blockIdx.z * CB_Z;
+  const int bx = blockIdx.z * FB_X, by = blockIdx.y * FB_Y, bz = blockIdx.x * FB_Z;
   const int tid = threadIdx.x;
-  constexpr int kIt = (EB_N + 255) / 256, kPer = CB_X * CB_Y * CB_Z / 256;
-  constexpr int NY = CB_Y + 1, NZ = CB_Z + 1;
+  constexpr int kIt = (EB_N + 255) / 256, kPer = FB_X * FB_Y * FB_Z / 256;
+  constexpr int NY = FB_Y + 1, NZ = FB_Z + 1;
   if (tid < 3) sh[tid] = 0;
   long long raw[kIt][3];
-  int emax[3] = {0, 0, 0};
+  int hmax[3] = {0, 0, 0};
 #pragma unroll
   for (int t = 0; t < kIt; ++t) {
     const int q = tid + 256 * t;
@@ -105,7 +153,7 @@ __global__ void __launch_bounds__(256, 2)
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       raw[t][c] = s < 0 ? 0LL : __double_as_longlong(hb.c[c][gi]);
-      emax[c] = max(emax[c], (int)((unsigned long long)raw[t][c] >> 52) & 0x7FF);
+      hmax[c] = max(hmax[c], high_bits(raw[t][c]));
     }
   }
   // E and J of the thread's cells, in flight with the staged values
@@ -113,8 +161,8 @@ __global__ void __launch_bounds__(256, 2)
 #pragma unroll
   for (int t = 0; t < kPer; ++t) {
     const int q = tid + 256 * t;
-    const int lz = q % CB_Z, r = q / CB_Z;
-    const int i = bx + r / CB_Y, j = by + r % CB_Y, k = bz + lz;
+    const int lz = q % FB_Z, r = q / FB_Z;
+    const int i = bx + r / FB_Y, j = by + r % FB_Y, k = bz + lz;
     const bool in = i < g.nx && j < g.ny && k < g.nz;
     const size_t id = in ? (size_t)slab_of(g, i) * g.nyz + (size_t)j * g.nz + k : 0;
 #pragma unroll
@@ -125,12 +173,12 @@ __global__ void __launch_bounds__(256, 2)
   }
   __syncthreads();
   int e[3];
-  const bool finite = block_scales(emax, sh, e);
+  const bool finite = block_scales(hmax, sh, e);
   if (!finite) {  // uniform over the block
     for (int t = 0; t < kPer; ++t) {
       const int q = tid + 256 * t;
-      const int lz = q % CB_Z, r = q / CB_Z;
-      const int i = bx + r / CB_Y, j = by + r % CB_Y, k = bz + lz;
+      const int lz = q % FB_Z, r = q / FB_Z;
+      const int i = bx + r / FB_Y, j = by + r % FB_Y, k = bz + lz;
       if (i < g.nx && j < g.ny && k < g.nz) e_update_cell(g, f, hb, fc, pm, i, j, k);
     }
     return;
@@ -143,89 +191,148 @@ __global__ void __launch_bounds__(256, 2)
       for (int c = 0; c < 3; ++c) sB[c][q] = field_fixed(raw[t][c], e[c]);
   }
   __syncthreads();
+  const WeakTest weak_test(e, sh, kFieldBits - 7);
   int sc[3];  // scale of the products
 #pragma unroll
-  for (int c = 0; c < 3; ++c) sc[c] = kFieldBits - 2 + 1023 - e[c];
+  for (int c = 0; c < 3; ++c) sc[c] = kFieldBits - 1 + 1023 - e[c];
 #pragma unroll
   for (int t = 0; t < kPer; ++t) {
     const int q = tid + 256 * t;
-    const int lz = q % CB_Z, r = q / CB_Z, ly = r % CB_Y, lx = r / CB_Y;
+    const int lz = q % FB_Z, r = q / FB_Z, ly = r % FB_Y, lx = r / FB_Y;
     const int i = bx + lx, j = by + ly, k = bz + lz;
-    if (i >= g.nx || j >= g.ny || k >= g.nz) continue;
+    if (i >= g.nx) continue;  // uniform over a warp
     const int slab = slab_of(g, i);
     const size_t id = (size_t)slab * g.nyz + (size_t)j * g.nz + k;
     const int p = ((lx + 1) * NY + ly + 1) * NZ + lz + 1;
     const long long vx = sB[0][p], vy = sB[1][p], vz = sB[2][p];
-    const long long yBz = scaled(vz - sB[2][p - NZ], k64.fd[1]), zBy = scaled(vy - sB[1][p - 1], k64.fd[2]);
-    const long long zBx = scaled(vx - sB[0][p - 1], k64.fd[2]), xBz = scaled(vz - sB[2][p - NY * NZ], k64.fd[0]);
-    const long long xBy = scaled(vy - sB[1][p - NY * NZ], k64.fd[0]), yBx = scaled(vx - sB[0][p - NZ], k64.fd[1]);
-    double dE[3];
-    const int jr = pm.L ? pml_row(j, g.ny, pm.L) : -1, kr = pm.L ? pml_row(k, g.nz, pm.L) : -1;
-    if (jr >= 0 || kr >= 0) {  // memory variables (times dt): y and z at nodes
-      double dyBz = fixed_to_double(yBz, sc[2]), dzBy = fixed_to_double(zBy, sc[1]);
-      double dzBx = fixed_to_double(zBx, sc[0]), dyBx = fixed_to_double(yBx, sc[0]);
-      if (jr >= 0) {
-        const double a = pm.cy[j] * k64.idt, b = pm.cy[g.ny + j];
-        const size_t pi = ((size_t)slab * pm.rows + jr) * g.nz + k;
-        const double p0 = b * pm.py[0][pi] + a * dyBz, p1 = b * pm.py[1][pi] + a * dyBx;
-        pm.py[0][pi] = p0;
-        pm.py[1][pi] = p1;
-        dyBz += fc.dt * p0;
-        dyBx += fc.dt * p1;
-      }
-      if (kr >= 0) {
-        const double a = pm.cz[k] * k64.idt, b = pm.cz[g.nz + k];
-        const size_t pi = ((size_t)slab * g.ny + j) * pm.rows + kr;
-        const double p0 = b * pm.pz[0][pi] + a * dzBy, p1 = b * pm.pz[1][pi] + a * dzBx;
-        pm.pz[0][pi] = p0;
-        pm.pz[1][pi] = p1;
-        dzBy += fc.dt * p0;
-        dzBx += fc.dt * p1;
-      }
-      dE[0] = dyBz - dzBy;
-      dE[1] = dzBx - fixed_to_double(xBz, sc[2]);
-      dE[2] = fixed_to_double(xBy, sc[1]) - dyBx;
-    } else {
-      dE[0] = fixed_to_double(aligned_diff(yBz, sc[2], zBy, sc[1]), min(sc[2], sc[1]));
-      dE[1] = fixed_to_double(aligned_diff(zBx, sc[0], xBz, sc[2]), min(sc[0], sc[2]));
-      dE[2] = fixed_to_double(aligned_diff(xBy, sc[1], yBx, sc[0]), min(sc[1], sc[0]));
-    }
+    const long long zy = sB[2][p - NZ], zx = sB[2][p - NY * NZ], yz = sB[1][p - 1], yx = sB[1][p - NY * NZ];
+    const long long xz = sB[0][p - 1], xy = sB[0][p - NZ];
+    const bool layer = pm.L && (pml_row(j, g.ny, pm.L) >= 0 || pml_row(k, g.nz, pm.L) >= 0);
+    int hi[3];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) f.c[EX + c][id] = pe[t][c] + fma(-fc.dt, pj[t][c], dE[c]);
+    for (int c = 0; c < 3; ++c) hi[c] = layer ? -1 : high_bits(pe[t][c]);
+    const unsigned weak = weak_test(0, vz, zy, hi[0]) | weak_test(1, vy, yz, hi[0]) | weak_test(2, vx, xz, hi[1]) |
+                          weak_test(3, vz, zx, hi[1]) | weak_test(4, vy, yx, hi[2]) | weak_test(5, vx, xy, hi[2]);
+    if (j >= g.ny || k >= g.nz) continue;
+    const long long yBz = scaled<2>(vz - zy, k64.fd[1]), zBy = scaled<2>(vy - yz, k64.fd[2]);
+    const long long zBx = scaled<2>(vx - xz, k64.fd[2]), xBz = scaled<2>(vz - zx, k64.fd[0]);
+    const long long xBy = scaled<2>(vy - yx, k64.fd[0]), yBx = scaled<2>(vx - xy, k64.fd[1]);
+    const double *Hx = hb.c[0], *Hy = hb.c[1], *Hz = hb.c[2];
+    if (layer) {
+      CurlD<double> d;
+      d.dyEz = weak & 1 ? (Hz[id] - below(Hz, g, slab, j - 1, k)) * fc.idy : fixed_to_double(yBz, sc[2]) * k64.idt;
+      d.dzEy = weak & 2 ? (Hy[id] - below(Hy, g, slab, j, k - 1)) * fc.idz : fixed_to_double(zBy, sc[1]) * k64.idt;
+      d.dzEx = weak & 4 ? (Hx[id] - below(Hx, g, slab, j, k - 1)) * fc.idz : fixed_to_double(zBx, sc[0]) * k64.idt;
+      d.dxEz = weak & 8 ? (Hz[id] - below(Hz, g, slab_of(g, i - 1), j, k)) * fc.idx : fixed_to_double(xBz, sc[2]) * k64.idt;
+      d.dxEy = weak & 16 ? (Hy[id] - below(Hy, g, slab_of(g, i - 1), j, k)) * fc.idx : fixed_to_double(xBy, sc[1]) * k64.idt;
+      d.dyEx = weak & 32 ? (Hx[id] - below(Hx, g, slab, j - 1, k)) * fc.idy : fixed_to_double(yBx, sc[0]) * k64.idt;
+      e_layers(g, pm, slab, j, k, d);
+      f.c[EX][id] = pe[t][0] + fc.dt * ((d.dyEz - d.dzEy) - pj[t][0]);
+      f.c[EY][id] = pe[t][1] + fc.dt * ((d.dzEx - d.dxEz) - pj[t][1]);
+      f.c[EZ][id] = pe[t][2] + fc.dt * ((d.dxEy - d.dyEx) - pj[t][2]);
+      continue;
+    }
+    // the difference of derivatives a and b, a - b; the one of A, B from slab s, row and
+    // column down by one where it is weak
+    auto put = [&](int c, long long a, int ca, const double* A, int sa, int ja, int ka, double ia, long long b, int cb,
+                   const double* B, int sb, int jb, int kb, double ib) {
+      const unsigned w = weak >> (2 * c) & 3u;
+      double v;
+      if (w) {
+        const double da = w & 1 ? (A[id] - below(A, g, sa, ja, ka)) * ia : fixed_to_double(a, sc[ca]) * k64.idt;
+        const double db = w & 2 ? (B[id] - below(B, g, sb, jb, kb)) * ib : fixed_to_double(b, sc[cb]) * k64.idt;
+        v = pe[t][c] + fc.dt * ((da - db) - pj[t][c]);
+      } else {
+        const double dE = fixed_to_double(aligned_diff(a, sc[ca], b, sc[cb]), min(sc[ca], sc[cb]));
+        v = pe[t][c] + fma(-fc.dt, pj[t][c], dE);
+      }
+      f.c[EX + c][id] = v;
+    };
+    const int sm = slab_of(g, i - 1);
+    put(0, yBz, 2, Hz, slab, j - 1, k, fc.idy, zBy, 1, Hy, slab, j, k - 1, fc.idz);
+    put(1, zBx, 0, Hx, slab, j, k - 1, fc.idz, xBz, 2, Hz, sm, j, k, fc.idx);
+    put(2, xBy, 1, Hy, sm, j, k, fc.idx, yBx, 0, Hx, slab, j - 1, k, fc.idy);
   }
 }
 
+// Derivative n of curl'(E) in FP64 from global memory: the same code for every n, so
+// that the lanes of a warp stay together, and the 18 loads in flight at once.
+__device__ __forceinline__ double curl_term(const Geom<double>& g, const Smooth<double>& S, const Fields<double>& f,
+                                            const FieldCoef<double>& fc, int n, int i, int j, int k) {
+  const bool y = n == 0 || n == 5, z = n == 1 || n == 2;  // the axis of the derivative
+  const double* F = n % 3 == 0 ? f.c[EZ] : (n % 3 == 1 ? f.c[EY] : f.c[EX]);
+  int ox[3], oy[3], oz[3];  // offsets of the neighbours at -1, 0, 1; -1 beyond the grid
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const int s = slab_of(g, i + d - 1);
+    int jj = j + d - 1, kk = k + d - 1;
+    if (!g.pml) {
+      jj = jj < 0 ? jj + g.ny : (jj >= g.ny ? jj - g.ny : jj);
+      kk = kk < 0 ? kk + g.nz : (kk >= g.nz ? kk - g.nz : kk);
+    }
+    ox[d] = s < 0 ? -1 : s * g.nyz;
+    oy[d] = (unsigned)jj < (unsigned)g.ny ? jj * g.nz : -1;
+    oz[d] = (unsigned)kk < (unsigned)g.nz ? kk : -1;
+  }
+  double v[2][3][3];  // along the derivative's axis, the first and the second other axis
+#pragma unroll
+  for (int p = 0; p < 2; ++p)
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
+#pragma unroll
+      for (int r = 0; r < 3; ++r) {
+        const int oa = y ? oy[1 + p] : (z ? oz[1 + p] : ox[1 + p]), ob = y || z ? ox[q] : oy[q], oc = z ? oy[r] : oz[r];
+        v[p][q][r] = (oa | ob | oc) >= 0 ? F[oa + ob + oc] : 0.0;
+      }
+  const double wa = y ? S.a[1] : (z ? S.a[2] : S.a[0]), w1 = y ? S.b1[1] : (z ? S.b1[2] : S.b1[0]);
+  const double w2 = y ? S.b2[1] : (z ? S.b2[2] : S.b2[0]), wg = y ? S.g[1] : (z ? S.g[2] : S.g[0]);
+  double m[2];
+#pragma unroll
+  for (int p = 0; p < 2; ++p)
+    m[p] = wa * v[p][1][1] + w1 * (v[p][2][1] + v[p][0][1]) + w2 * (v[p][1][2] + v[p][1][0]) +
+           wg * (v[p][2][2] + v[p][2][0] + v[p][0][2] + v[p][0][0]);
+  return (m[1] - m[0]) * (y ? fc.idy : (z ? fc.idz : fc.idx));
+}
+
 // Smoothed curl and the magnetic half steps, as k_curl_tiled.
-constexpr size_t kCurl64Smem = 8 * (3 * (size_t)CE_N + 2 * (size_t)(SXN + SYN + SZN));
+// The weak derivatives of a block are listed and then computed by as many threads,
+// since a warp takes as long for one of them as for 32; the results take the place of
+// the staged fields.  (A vacuum step with 4x8x32 blocks: 2.35 ms with each lane its own
+// in place, 1.58 with all derivatives of a listed cell, 1.44 with the weak ones.)
+constexpr int kCurlCells = FB_X * FB_Y * FB_Z;
+constexpr int kWeakList = 4096;  // of 6 x 1024; what does not fit, a thread computes in place
+constexpr int kCurlFirst = 3 * FE_N > 6 * kCurlCells ? 3 * FE_N : 6 * kCurlCells;
+constexpr size_t kCurl64Smem = 8 * (kCurlFirst + 2 * (size_t)(FXN + FYN + FZN));
 __global__ void __launch_bounds__(256, 2)
     k_curl64(Geom<double> g, Smooth<double> S, Fields<double> f, Fields<double> hb, FieldCoef<double> fc,
              FieldConst64 k64, int mode, FieldSpan sp, Pml<double> pm) {
   if (!dyn_prologue(g)) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ int sh[3];
-  long long* sE = reinterpret_cast<long long*>(smem_raw);  // [3][CE_X][CE_Y][CE_Z], origin (bx-1, by-1, bz-1)
-  long long* sSxEy = sE + 3 * CE_N;                        // [CB_X+1][CB_Y][CB_Z]
-  long long* sSxEz = sSxEy + SXN;
-  long long* sSyEz = sSxEz + SXN;                          // [CB_X][CB_Y+1][CB_Z]
-  long long* sSyEx = sSyEz + SYN;
-  long long* sSzEx = sSyEx + SYN;                          // [CB_X][CB_Y][CB_Z+1]
-  long long* sSzEy = sSzEx + SZN;
-  const int bx = blockIdx.x * sp.step, bx1 = min(bx + sp.width, g.nx), by = blockIdx.y * CB_Y, bz = blockIdx.z * CB_Z;
+  __shared__ int sh[4];  // largest high words; weak derivatives
+  __shared__ unsigned short list[kWeakList];
+  long long* sE = reinterpret_cast<long long*>(smem_raw);  // [3][FE_X][FE_Y][FE_Z], origin (bx-1, by-1, bz-1)
+  long long* sSxEy = sE + kCurlFirst;                      // [FB_X+1][FB_Y][FB_Z]
+  long long* sSxEz = sSxEy + FXN;
+  long long* sSyEz = sSxEz + FXN;                          // [FB_X][FB_Y+1][FB_Z]
+  long long* sSyEx = sSyEz + FYN;
+  long long* sSzEx = sSyEx + FYN;                          // [FB_X][FB_Y][FB_Z+1]
+  long long* sSzEy = sSzEx + FZN;
+  const int bx = blockIdx.z * sp.step, bx1 = min(bx + sp.width, g.nx), by = blockIdx.y * FB_Y, bz = blockIdx.x * FB_Z;
   const int tid = threadIdx.x;
-  constexpr int kPer = CB_X * CB_Y * CB_Z / 256;
+  constexpr int kPer = FB_X * FB_Y * FB_Z / 256;
   int e[3];
   bool finite;
   double pb[kPer][3];  // H (mode 1) or B (mode 0) of the thread's cells
-  if (tid < 3) sh[tid] = 0;
+  if (tid < 4) sh[tid] = 0;
   {
-    constexpr int kIt = (CE_N + 255) / 256;
+    constexpr int kIt = (FE_N + 255) / 256;
     long long raw[kIt][3];
-    int emax[3] = {0, 0, 0};
+    int hmax[3] = {0, 0, 0};
 #pragma unroll
     for (int t = 0; t < kIt; ++t) {
       const int q = tid + 256 * t;
-      const int lz = q % CE_Z, r = q / CE_Z, ly = r % CE_Y, lx = r / CE_Y;
-      int s = q < CE_N ? slab_of(g, bx - 1 + lx) : -1;
+      const int lz = q % FE_Z, r = q / FE_Z, ly = r % FE_Y, lx = r / FE_Y;
+      int s = q < FE_N ? slab_of(g, bx - 1 + lx) : -1;
       int j = by - 1 + ly, k = bz - 1 + lz;
       if (g.pml) {  // zero beyond the grid
         if (j < 0 || j >= g.ny || k < 0 || k >= g.nz) s = -1;
@@ -239,95 +346,146 @@ __global__ void __launch_bounds__(256, 2)
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         raw[t][c] = s < 0 ? 0LL : __double_as_longlong(f.c[EX + c][gi]);
-        emax[c] = max(emax[c], (int)((unsigned long long)raw[t][c] >> 52) & 0x7FF);
+        hmax[c] = max(hmax[c], high_bits(raw[t][c]));
       }
     }
 #pragma unroll
     for (int t = 0; t < kPer; ++t) {  // in flight with the staged values
       const int q = tid + 256 * t;
-      const int lz = q % CB_Z, r = q / CB_Z;
-      const int i = bx + r / CB_Y, j = by + r % CB_Y, k = bz + lz;
+      const int lz = q % FB_Z, r = q / FB_Z;
+      const int i = bx + r / FB_Y, j = by + r % FB_Y, k = bz + lz;
       const bool in = i < bx1 && j < g.ny && k < g.nz;
       const size_t id = in ? (size_t)slab_of(g, i) * g.nyz + (size_t)j * g.nz + k : 0;
 #pragma unroll
       for (int c = 0; c < 3; ++c) pb[t][c] = mode == 1 ? hb.c[c][id] : f.c[BX + c][id];
     }
     __syncthreads();
-    finite = block_scales(emax, sh, e);
+    finite = block_scales(hmax, sh, e);
     if (finite)
 #pragma unroll
       for (int t = 0; t < kIt; ++t) {
         const int q = tid + 256 * t;
-        if (q < CE_N)
+        if (q < FE_N)
 #pragma unroll
-          for (int c = 0; c < 3; ++c) sE[c * CE_N + q] = field_fixed(raw[t][c], e[c]);
+          for (int c = 0; c < 3; ++c) sE[c * FE_N + q] = field_fixed(raw[t][c], e[c]);
       }
   }
   if (!finite) {  // uniform over the block
     for (int t = 0; t < kPer; ++t) {
       const int q = tid + 256 * t;
-      const int lz = q % CB_Z, r = q / CB_Z;
-      const int i = bx + r / CB_Y, j = by + r % CB_Y, k = bz + lz;
+      const int lz = q % FB_Z, r = q / FB_Z;
+      const int i = bx + r / FB_Y, j = by + r % FB_Y, k = bz + lz;
       if (i < bx1 && j < g.ny && k < g.nz) curl_cell(g, S, f, hb, fc, pm, mode, i, j, k);
     }
     return;
   }
   __syncthreads();
   {
-    auto E = [&](int c, int p) -> long long { return sE[c * CE_N + p]; };
-    // sum over the 3x3 points around p with steps a, b: at 2^(s - 1)
-    auto smooth = [&](int c, int p, int a, int b, const S32(&w)[4]) -> long long {
+    auto E = [&](int c, int p) -> long long { return sE[c * FE_N + p]; };
+    // sum over the 3x3 points around p with steps a, b, at 2^(s + 1); the products' low
+    // words enter with their upper 15 bits
+    auto smooth = [&](int c, int p, int a, int b, const S32(&w)[4], const int(&w17)[4]) -> long long {
       const long long e1 = E(c, p + a) + E(c, p - a), e2 = E(c, p + b) + E(c, p - b);
       const long long cr = (E(c, p + a + b) + E(c, p + a - b)) + (E(c, p - a + b) + E(c, p - a - b));
-      Acc32 s = {0LL, kRound2};
-      acc32(s, split32(E(c, p)), w[0]);
-      acc32(s, split32(e1), w[1]);
-      acc32(s, split32(e2), w[2]);
-      acc32(s, split32(cr), w[3]);
-      return acc32_result2(s);
+      const S32 x[4] = {split32(E(c, p)), split32(e1), split32(e2), split32(cr)};
+      Acc32 s = {0LL, 1LL << 28};
+      int l = 0;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        acc32(s, x[k], w[k]);
+        l += (x[k].lo >> 17) * w17[k];
+      }
+      s.M += (long long)l * 4;
+      return (s.H << 3) + (s.M >> 29);
     };
-    constexpr int PX = CE_Y * CE_Z, PY = CE_Z;
-    for (int q = tid; q < SXN; q += 256) {
-      const int lz = q % CB_Z, r = q / CB_Z;
-      const int p = (r / CB_Y + 1) * PX + (r % CB_Y + 1) * PY + lz + 1;
-      sSxEy[q] = smooth(1, p, PY, 1, k64.s[0]);
-      sSxEz[q] = smooth(2, p, PY, 1, k64.s[0]);
+    constexpr int PX = FE_Y * FE_Z, PY = FE_Z;
+    for (int q = tid; q < FXN; q += 256) {
+      const int lz = q % FB_Z, r = q / FB_Z;
+      const int p = (r / FB_Y + 1) * PX + (r % FB_Y + 1) * PY + lz + 1;
+      sSxEy[q] = smooth(1, p, PY, 1, k64.s[0], k64.s17[0]);
+      sSxEz[q] = smooth(2, p, PY, 1, k64.s[0], k64.s17[0]);
     }
-    for (int q = tid; q < SYN; q += 256) {
-      const int lz = q % CB_Z, r = q / CB_Z;
-      const int p = (r / (CB_Y + 1) + 1) * PX + (r % (CB_Y + 1) + 1) * PY + lz + 1;
-      sSyEz[q] = smooth(2, p, PX, 1, k64.s[1]);
-      sSyEx[q] = smooth(0, p, PX, 1, k64.s[1]);
+    for (int q = tid; q < FYN; q += 256) {
+      const int lz = q % FB_Z, r = q / FB_Z;
+      const int p = (r / (FB_Y + 1) + 1) * PX + (r % (FB_Y + 1) + 1) * PY + lz + 1;
+      sSyEz[q] = smooth(2, p, PX, 1, k64.s[1], k64.s17[1]);
+      sSyEx[q] = smooth(0, p, PX, 1, k64.s[1], k64.s17[1]);
     }
-    for (int q = tid; q < SZN; q += 256) {
-      const int lz = q % (CB_Z + 1), r = q / (CB_Z + 1);
-      const int p = (r / CB_Y + 1) * PX + (r % CB_Y + 1) * PY + lz + 1;
-      sSzEx[q] = smooth(0, p, PX, PY, k64.s[2]);
-      sSzEy[q] = smooth(1, p, PX, PY, k64.s[2]);
+    for (int q = tid; q < FZN; q += 256) {
+      const int lz = q % (FB_Z + 1), r = q / (FB_Z + 1);
+      const int p = (r / FB_Y + 1) * PX + (r % FB_Y + 1) * PY + lz + 1;
+      sSzEx[q] = smooth(0, p, PX, PY, k64.s[2], k64.s17[2]);
+      sSzEy[q] = smooth(1, p, PX, PY, k64.s[2], k64.s17[2]);
     }
   }
   __syncthreads();
+  double* sWeak = reinterpret_cast<double*>(smem_raw);  // [6][kCurlCells]
+  unsigned weak_bits = 0;                               // six per cell of the thread
+  {
+    const WeakTest weak_test(e, sh, kFieldBits - 7);  // the smoothed values have twice the scale
+#pragma unroll
+    for (int t = 0; t < kPer; ++t) {
+      const int q = tid + 256 * t;
+      const int lz = q % FB_Z, r = q / FB_Z, ly = r % FB_Y, lx = r / FB_Y;
+      const int i = bx + lx, j = by + ly, k = bz + lz;
+      if (i >= bx1) continue;  // uniform over a warp
+      const int x0 = (lx * FB_Y + ly) * FB_Z + lz, x1 = x0 + FB_Y * FB_Z;
+      const int y0 = (lx * (FB_Y + 1) + ly) * FB_Z + lz, y1 = y0 + FB_Z;
+      const int z0 = (lx * FB_Y + ly) * (FB_Z + 1) + lz;
+      const bool layer = pm.L && (pml_row(j, g.ny, pm.L) >= 0 || pml_row(k, g.nz, pm.L) >= 0);
+      int hi[3];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) hi[c] = layer ? -1 : high_bits(pb[t][c]);
+      const unsigned weak = weak_test(0, sSyEz[y1], sSyEz[y0], hi[0]) | weak_test(1, sSzEy[z0 + 1], sSzEy[z0], hi[0]) |
+                      weak_test(2, sSzEx[z0 + 1], sSzEx[z0], hi[1]) | weak_test(3, sSxEz[x1], sSxEz[x0], hi[1]) |
+                      weak_test(4, sSxEy[x1], sSxEy[x0], hi[2]) | weak_test(5, sSyEx[y1], sSyEx[y0], hi[2]);
+      if (j < g.ny && k < g.nz) weak_bits |= weak << (6 * t);
+    }
+    if (weak_bits) {
+      int pos = atomicAdd(sh + 3, __popc(weak_bits));
+      for (unsigned m = weak_bits; m; m &= m - 1, ++pos) {
+        const int t = (__ffs(m) - 1) / 6, n = (__ffs(m) - 1) % 6, q = tid + 256 * t, r = q / FB_Z;
+        if (pos < kWeakList)
+          list[pos] = (unsigned short)(n * kCurlCells + q);
+        else
+          sWeak[n * kCurlCells + q] = curl_term(g, S, f, fc, n, bx + r / FB_Y, by + r % FB_Y, bz + q % FB_Z);
+      }
+    }
+    static_assert(6 * kPer <= 32, "six bits per cell");
+    static_assert(6 * kCurlCells <= 65536, "16-bit entries");
+    __syncthreads();
+    const int nweak = min(sh[3], kWeakList);
+    if (nweak > 0) {  // uniform over the block
+#pragma unroll 1
+      for (int m = tid; m < nweak; m += 256) {
+        const int n = list[m] / kCurlCells, q = list[m] % kCurlCells, r = q / FB_Z;
+        sWeak[n * kCurlCells + q] = curl_term(g, S, f, fc, n, bx + r / FB_Y, by + r % FB_Y, bz + q % FB_Z);
+      }
+      __syncthreads();
+    }
+  }
   int sc[3];  // scale of the products
 #pragma unroll
-  for (int c = 0; c < 3; ++c) sc[c] = kFieldBits - 2 + 1023 - e[c];
+  for (int c = 0; c < 3; ++c) sc[c] = kFieldBits + 1023 - e[c];
 #pragma unroll
   for (int t = 0; t < kPer; ++t) {
     const int q = tid + 256 * t;
-    const int lz = q % CB_Z, r = q / CB_Z, ly = r % CB_Y, lx = r / CB_Y;
+    const int lz = q % FB_Z, r = q / FB_Z, ly = r % FB_Y, lx = r / FB_Y;
     const int i = bx + lx, j = by + ly, k = bz + lz;
     if (i >= bx1 || j >= g.ny || k >= g.nz) continue;
-    const int x0 = (lx * CB_Y + ly) * CB_Z + lz, x1 = x0 + CB_Y * CB_Z;
-    const int y0 = (lx * (CB_Y + 1) + ly) * CB_Z + lz, y1 = y0 + CB_Z;
-    const int z0 = (lx * CB_Y + ly) * (CB_Z + 1) + lz;
+    const int x0 = (lx * FB_Y + ly) * FB_Z + lz, x1 = x0 + FB_Y * FB_Z;
+    const int y0 = (lx * (FB_Y + 1) + ly) * FB_Z + lz, y1 = y0 + FB_Z;
+    const int z0 = (lx * FB_Y + ly) * (FB_Z + 1) + lz;
     const int slab = slab_of(g, i);
     const size_t id = (size_t)slab * g.nyz + (size_t)j * g.nz + k;
     // dt/2 times D_y S_y Ez, D_z S_z Ey; D_z S_z Ex, D_x S_x Ez; D_x S_x Ey, D_y S_y Ex
-    const long long yEz = scaled(sSyEz[y1] - sSyEz[y0], k64.hd[1]), zEy = scaled(sSzEy[z0 + 1] - sSzEy[z0], k64.hd[2]);
-    const long long zEx = scaled(sSzEx[z0 + 1] - sSzEx[z0], k64.hd[2]), xEz = scaled(sSxEz[x1] - sSxEz[x0], k64.hd[0]);
-    const long long xEy = scaled(sSxEy[x1] - sSxEy[x0], k64.hd[0]), yEx = scaled(sSyEx[y1] - sSyEx[y0], k64.hd[1]);
+    const long long yEz = scaled<1>(sSyEz[y1] - sSyEz[y0], k64.hd[1]), zEy = scaled<1>(sSzEy[z0 + 1] - sSzEy[z0], k64.hd[2]);
+    const long long zEx = scaled<1>(sSzEx[z0 + 1] - sSzEx[z0], k64.hd[2]), xEz = scaled<1>(sSxEz[x1] - sSxEz[x0], k64.hd[0]);
+    const long long xEy = scaled<1>(sSxEy[x1] - sSxEy[x0], k64.hd[0]), yEx = scaled<1>(sSyEx[y1] - sSyEx[y0], k64.hd[1]);
     double dB[3];
     const int jr = pm.L ? pml_row(j, g.ny, pm.L) : -1, kr = pm.L ? pml_row(k, g.nz, pm.L) : -1;
-    if (jr >= 0 || kr >= 0) {  // memory variables: y and z at half nodes
+    const unsigned weak = (weak_bits >> (6 * t)) & 63u;
+    if (weak || jr >= 0 || kr >= 0) {  // the derivatives as doubles
       CurlD<double> d;
       d.dyEz = fixed_to_double(yEz, sc[2]) * k64.ihdt;
       d.dzEy = fixed_to_double(zEy, sc[1]) * k64.ihdt;
@@ -335,7 +493,13 @@ __global__ void __launch_bounds__(256, 2)
       d.dxEz = fixed_to_double(xEz, sc[2]) * k64.ihdt;
       d.dxEy = fixed_to_double(xEy, sc[1]) * k64.ihdt;
       d.dyEx = fixed_to_double(yEx, sc[0]) * k64.ihdt;
-      curl_layers(g, pm, mode, slab, j, k, d);
+      if (weak & 1) d.dyEz = sWeak[q];
+      if (weak & 2) d.dzEy = sWeak[kCurlCells + q];
+      if (weak & 4) d.dzEx = sWeak[2 * kCurlCells + q];
+      if (weak & 8) d.dxEz = sWeak[3 * kCurlCells + q];
+      if (weak & 16) d.dxEy = sWeak[4 * kCurlCells + q];
+      if (weak & 32) d.dyEx = sWeak[5 * kCurlCells + q];
+      if (jr >= 0 || kr >= 0) curl_layers(g, pm, mode, slab, j, k, d);  // y and z at half nodes
       dB[0] = fc.hdt * (d.dyEz - d.dzEy);
       dB[1] = fc.hdt * (d.dzEx - d.dxEz);
       dB[2] = fc.hdt * (d.dxEy - d.dyEx);

@@ -125,6 +125,38 @@ __device__ __forceinline__ T below(const T* __restrict__ H, const Geom<T>& g, in
   return H[(size_t)s * g.nyz + (size_t)j * g.nz + k];
 }
 
+// The six derivatives of a curl at a cell (of E; of H with H in the place of E).
+template <typename T>
+struct CurlD {
+  T dyEz, dzEy, dzEx, dxEz, dxEy, dyEx;
+};
+
+// Absorbing layers in curl H: Ex (i+1/2, j, k), Ey (i, j+1/2, k), Ez (i, j, k+1/2),
+// y and z at nodes.
+template <typename T>
+__device__ __forceinline__ void e_layers(const Geom<T>& g, const Pml<T>& pm, int s, int j, int k, CurlD<T>& d) {
+  const int jr = pml_row(j, g.ny, pm.L);
+  if (jr >= 0) {
+    const T a = pm.cy[j], b = pm.cy[g.ny + j];
+    const size_t pi = ((size_t)s * pm.rows + jr) * g.nz + k;
+    const T p0 = b * pm.py[0][pi] + a * d.dyEz, p1 = b * pm.py[1][pi] + a * d.dyEx;
+    pm.py[0][pi] = p0;
+    pm.py[1][pi] = p1;
+    d.dyEz += p0;
+    d.dyEx += p1;
+  }
+  const int kr = pml_row(k, g.nz, pm.L);
+  if (kr >= 0) {
+    const T a = pm.cz[k], b = pm.cz[g.nz + k];
+    const size_t pi = ((size_t)s * g.ny + j) * pm.rows + kr;
+    const T p0 = b * pm.pz[0][pi] + a * d.dzEy, p1 = b * pm.pz[1][pi] + a * d.dzEx;
+    pm.pz[0][pi] = p0;
+    pm.pz[1][pi] = p1;
+    d.dzEy += p0;
+    d.dzEx += p1;
+  }
+}
+
 template <typename T>
 __device__ __forceinline__ void e_update_cell(const Geom<T>& g, const Fields<T>& f, const Fields<T>& hb,
                                               const FieldCoef<T>& fc, const Pml<T>& pm, int i, int j, int k) {
@@ -132,37 +164,17 @@ __device__ __forceinline__ void e_update_cell(const Geom<T>& g, const Fields<T>&
   const int s = slab_of(g, i), sm = slab_of(g, i - 1);
   const size_t id = (size_t)s * g.nyz + (size_t)j * g.nz + k;
   const T bx = Hx[id], by = Hy[id], bz = Hz[id];
-  T dyBz = (bz - below(Hz, g, s, j - 1, k)) * fc.idy;
-  T dzBy = (by - below(Hy, g, s, j, k - 1)) * fc.idz;
-  T dzBx = (bx - below(Hx, g, s, j, k - 1)) * fc.idz;
-  const T dxBz = (bz - below(Hz, g, sm, j, k)) * fc.idx;
-  const T dxBy = (by - below(Hy, g, sm, j, k)) * fc.idx;
-  T dyBx = (bx - below(Hx, g, s, j - 1, k)) * fc.idy;
-  if (pm.L) {  // Ex (i+1/2, j, k), Ey (i, j+1/2, k), Ez (i, j, k+1/2): y and z at nodes
-    const int jr = pml_row(j, g.ny, pm.L);
-    if (jr >= 0) {
-      const T a = pm.cy[j], b = pm.cy[g.ny + j];
-      const size_t pi = ((size_t)s * pm.rows + jr) * g.nz + k;
-      const T p0 = b * pm.py[0][pi] + a * dyBz, p1 = b * pm.py[1][pi] + a * dyBx;
-      pm.py[0][pi] = p0;
-      pm.py[1][pi] = p1;
-      dyBz += p0;
-      dyBx += p1;
-    }
-    const int kr = pml_row(k, g.nz, pm.L);
-    if (kr >= 0) {
-      const T a = pm.cz[k], b = pm.cz[g.nz + k];
-      const size_t pi = ((size_t)s * g.ny + j) * pm.rows + kr;
-      const T p0 = b * pm.pz[0][pi] + a * dzBy, p1 = b * pm.pz[1][pi] + a * dzBx;
-      pm.pz[0][pi] = p0;
-      pm.pz[1][pi] = p1;
-      dzBy += p0;
-      dzBx += p1;
-    }
-  }
-  f.c[EX][id] += fc.dt * ((dyBz - dzBy) - f.c[JX][id]);
-  f.c[EY][id] += fc.dt * ((dzBx - dxBz) - f.c[JY][id]);
-  f.c[EZ][id] += fc.dt * ((dxBy - dyBx) - f.c[JZ][id]);
+  CurlD<T> d;
+  d.dyEz = (bz - below(Hz, g, s, j - 1, k)) * fc.idy;
+  d.dzEy = (by - below(Hy, g, s, j, k - 1)) * fc.idz;
+  d.dzEx = (bx - below(Hx, g, s, j, k - 1)) * fc.idz;
+  d.dxEz = (bz - below(Hz, g, sm, j, k)) * fc.idx;
+  d.dxEy = (by - below(Hy, g, sm, j, k)) * fc.idx;
+  d.dyEx = (bx - below(Hx, g, s, j - 1, k)) * fc.idy;
+  if (pm.L) e_layers(g, pm, s, j, k, d);
+  f.c[EX][id] += fc.dt * ((d.dyEz - d.dzEy) - f.c[JX][id]);
+  f.c[EY][id] += fc.dt * ((d.dzEx - d.dxEz) - f.c[JY][id]);
+  f.c[EZ][id] += fc.dt * ((d.dxEy - d.dyEx) - f.c[JZ][id]);
 }
 
 // Launch: grid (ceil(nz / blockDim.x), ny, nx), one thread per cell; k from
@@ -173,12 +185,6 @@ __global__ void __launch_bounds__(256) k_e_update(Geom<T> g, Fields<T> f, Fields
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k < g.nz) e_update_cell(g, f, hb, fc, pm, (int)blockIdx.z, (int)blockIdx.y, k);
 }
-
-// The six derivatives of curl'(E) at a cell.
-template <typename T>
-struct CurlD {
-  T dyEz, dzEy, dzEx, dxEz, dxEy, dyEx;
-};
 
 // Absorbing layers in curl'(E): Bx (i, j+1/2, k+1/2), By (i+1/2, j, k+1/2), Bz
 // (i+1/2, j+1/2, k) at half nodes.  Mode 1 advances the memory variables with

@@ -90,7 +90,7 @@ def smoothing(rb, rc):
     return 1 - 2 * b1 - 2 * b2 - 4 * g, b1, b2, g
 
 
-def test_smoothing_stays_in_range():
+def test_smoothing_stays_in_range_and_close_to_exact():
     rng = random.Random(3)
     big = 1 << BITS
     for rb, rc in ((F(1), F(1)), (F(1), F(1, 9)), (F(1, 10 ** 6), F(1, 10 ** 6)), (F(1, 64), F(1, 64))):
@@ -100,14 +100,33 @@ def test_smoothing_stays_in_range():
                 s = rng.choice((-1, 1))
                 x = [s * big] * 9 if trial < 20 else [rng.randrange(-big, big + 1) for _ in range(9)]
                 terms = [x[0], x[1] + x[2], x[3] + x[4], sum(x[5:])]
-                H, M = 0, 1 << 30
+                H, M, l = 0, 1 << 28, 0
                 for t, w in zip(terms, weights):
                     (th, tl), (wh, wl) = split(t), split(w)
                     H, M = H + th * wh, M + th * wl + tl * wh
-                    assert abs(M) < 1 << 63
-                got = 2 * H + (M >> 31)
-                want = F(sum(t * w for t, w in zip(terms, weights)), 1 << 63)
-                assert abs(got - want) <= F(5, 2)  # four dropped products at twice the scale, the shift
+                    l += (tl >> 17) * (wl >> 17)
+                    assert abs(M) < 1 << 63 and abs(l) <= 1 << 30
+                M += 4 * l
+                got = (H << 3) + (M >> 29)
+                assert abs(M) < 1 << 63 and abs(got) <= 1 << 61  # at twice the scale of x
+                want = F(sum(t * w for t, w in zip(terms, weights)), 1 << 61)
+                # the shift; four low products with 15 of 32 bits each: 2^-14 of at most 2 units
+                assert abs(got - want) <= F(1, 2) + F(1, 1 << 10)
+
+
+def test_products_with_the_step_per_cell():
+    rng = random.Random(4)
+    for K, xmax, wmax in ((1, 1 << 62, 1 << 62), (2, 1 << 61, 1 << 62)):  # magnetic, electric
+        for _ in range(2000):
+            x, w = rng.randrange(-xmax, xmax + 1), rng.randrange(wmax + 1)
+            if rng.random() < 0.1:
+                x, w = rng.choice((-xmax, xmax)), wmax
+            (xh, xl), (wh, wl) = split(x), split(w)
+            H, M = xh * wh, (1 << (31 - K)) + xh * wl + xl * wh
+            assert abs(M) < 1 << 63
+            got = (H << K) + (M >> (32 - K))
+            assert abs(got) <= 1 << 61
+            assert abs(got - F(x * w, 1 << (64 - K))) <= F(1, 2) + F(1 << K, 4)  # the shift and the dropped product
 
 
 def coarser(a, sh):

@@ -2,7 +2,7 @@
 
 Where the two terms of a curl component have different scales, the finer one is
 rounded to the coarser one's unit.  With E = 0 and a strong uniform Bz = 1 (no
-derivative, unit of the products 2^-58) beside weak random Bx, By, the increments of Ex
+derivative, unit of the products 2^-58 or less) beside weak random Bx, By, the increments of Ex
 and Ey are that rounding: uniform on half a unit either way, its mean over 8192 cells
 0 +- 0.29 / sqrt(8192) = 0.003 units.  The bar is 0.03.
 """
