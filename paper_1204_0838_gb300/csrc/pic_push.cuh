@@ -26,6 +26,7 @@ constexpr int kRanks = 32;         // ranks per cell that are ordered; later one
 // bits), cell steps + 1 per axis (6 bits) and two flags
 constexpr unsigned kCross = 1u << 31;  // not with the ordered particles: alone (listed) or not at all
 constexpr unsigned kStray = 1u << 30;  // outside the tile: dropped, error bit set
+constexpr unsigned kSteps = 63u << 24;  // the cell steps; all set (no particle's steps): push again
 
 // The shared-memory region.  Components are stored with their axes rotated,
 // [i_d][i_e][i_f] with (e, f) the axes after d in cyclic order, so that one
@@ -117,7 +118,8 @@ struct PushSmem {
 
 // Pointers into the shared memory of a CTA, and the scalars: [0] particles
 // without an ordered rank, [1] particles that deposit alone, [2, 4) sums or
-// maxima over the tile, [4, 7) J scale per component, [8, 16) scan partials,
+// maxima over the tile, [4, 7) J scale per component, [7] whether particles of the
+// pass are to be pushed again on their own (FP32), [8, 16) scan partials,
 // [16, 33) first pair of each pair of ranks, [33] ordered particles, [34, 50)
 // first position of each pair of ranks, [50, 62) field scales (FP64), [50, 53)
 // scale of P per component and [53] the weight below which a particle is light (FP32).
@@ -177,7 +179,7 @@ __device__ __forceinline__ PushTile push_tile(unsigned char* smem, const Geom<T>
 __device__ __forceinline__ void rank_clear(const PushTile& P, int W) {
   for (int i = threadIdx.x; i < 32 * W; i += kPushThreads) P.hist[i] = 0;
   for (int i = threadIdx.x; i < kRanks * W; i += kPushThreads) P.mask[i] = 0u;
-  if (threadIdx.x < 2) P.sc[threadIdx.x] = 0;
+  if (threadIdx.x < 3) P.sc[threadIdx.x < 2 ? threadIdx.x : 7] = 0;
 }
 
 // Particles [begin, begin + n) of pass ps of npass over a tile of ntile: sizes

@@ -174,6 +174,37 @@ __device__ __forceinline__ float2 boris32(float h, const float2 (&E)[3], const f
   return rsqrt2(fma2(u[2], u[2], fma2(u[1], u[1], fma2(u[0], u[0], one))));
 }
 
+// The push of one particle with the fields of its own 4x4x4 windows (both halves the
+// same particle).  Returns 1 / gamma.
+template <bool FIXED>
+__device__ __forceinline__ float push_own32(const float* sF, const PushLayout<float, FIXED>& L, const int (&l)[3], float h,
+                                            float2 (&o)[3], float2 (&u)[3]) {
+  float2 E[3], B[3];
+  int r[3] = {l[0], l[1], l[2]};
+#pragma unroll 1
+  for (int d = 0; d < 3; ++d) {
+    const int sd = L.sd(d, 4), se = L.se(d, 4);
+    float2 wn[3][4], wh[3][4];
+    int hi[3];  // half-node windows start at c-2 or, from half a cell on, at c-1
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      hi[a] = o[a].x < 0.5f ? 0 : 1;
+      spline32(o[a], wn[a]);
+      spline32(add2(o[a], dup2(hi[a] ? -0.5f : 0.5f)), wh[a]);
+    }
+    const float* b = sF + L.start(d, 4) + r[0] * sd + r[1] * se + r[2];
+    E[0] = E[1], E[1] = E[2];
+    B[0] = B[1], B[1] = B[2];
+    E[2] = gather_pair<4, 4, 4>(b + hi[0] * sd + se + 1, sd, se, wh[0], wn[1], wn[2]);
+    B[2] = gather_pair<4, 4, 4>(b + L.part(d, 4) + sd + hi[1] * se + hi[2], sd, se, wn[0], wh[1], wh[2]);
+    const int r0 = r[0];
+    r[0] = r[1], r[1] = r[2], r[2] = r0;
+    const float2 t = o[0];
+    o[0] = o[1], o[1] = o[2], o[2] = t;
+  }
+  return boris32(h, E, B, u).x;
+}
+
 // New offset and cell step of one particle along one axis.
 __device__ __forceinline__ int step32(float o, float& o1) {
   int k = 0;
@@ -315,6 +346,24 @@ __global__ void __launch_bounds__(kPushThreads, 3)
     const int ranked = sc[33];
     const int nround = sc[16 + kRanks / 2];       // pairs of the ordered ranks
     const int nitem = nround + (nch - ranked);      // the rest goes one by one
+    // Move a particle with momentum u and 1 / gamma; returns its destination tile.
+    auto finish = [&](const int(&l)[3], int idx, int pos, unsigned ent, const float(&u)[3], float ig, bool good) {
+      int dc[3];
+      const int dst = c0 + pos;
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        const float o = p.o[d][idx];
+        float o1;
+        dc[d] = step32(good ? o + pc.dtd[d] * u[d] * ig : o, o1);
+        pn.o[d][dst] = o1;
+        pn.u[d][dst] = u[d];
+      }
+      const float w = p.w[idx];
+      pn.w[dst] = w;
+      if (pn.id) pn.id[dst] = p.id[idx];
+      return place_moved(P, g, tl, t, l, dc, good, good && fabsf(w) < __int_as_float(sc[53]), origin_after, xlo, xhi, pos, ent,
+                         pn.cell + dst, keys + dst);
+    };
     // ---- gather, push, move ----
     int round = 0;
     for (int i0 = 0; i0 < nitem; i0 += kPushThreads) {
@@ -395,27 +444,13 @@ __global__ void __launch_bounds__(kPushThreads, 3)
         for (int k = 0; k < 2; ++k) {
           if (k == 1 && !have[1]) break;
           const float igk = k ? ig.y : ig.x;
-          float uk[3] = {k ? u[0].y : u[0].x, k ? u[1].y : u[1].x, k ? u[2].y : u[2].x};
-          const bool good = igk > 0.0f;
-          if (!good) {  // a non-finite momentum: reported; absorbed without moving or depositing
-            atomicOr(err, 8);
-            uk[0] = uk[1] = uk[2] = 0.0f;
+          if (igk > 0.0f) {
+            const float uk[3] = {k ? u[0].y : u[0].x, k ? u[1].y : u[1].x, k ? u[2].y : u[2].x};
+            key[k] = finish(l, idx[k], pos[k], ent[k], uk, igk, true);
+          } else {  // not finite: once more, alone
+            order[pos[k]] = ent[k] | kCross | kSteps;
+            sc[7] = 1;
           }
-          int dc[3];
-          const int dst = c0 + pos[k];
-#pragma unroll
-          for (int d = 0; d < 3; ++d) {
-            const float o = p.o[d][idx[k]];
-            float o1;
-            dc[d] = step32(good ? o + pc.dtd[d] * uk[d] * igk : o, o1);
-            pn.o[d][dst] = o1;
-            pn.u[d][dst] = uk[d];
-          }
-          const float w = p.w[idx[k]];
-          pn.w[dst] = w;
-          if (pn.id) pn.id[dst] = p.id[idx[k]];
-          key[k] = place_moved(P, g, tl, t, l, dc, good, good && fabsf(w) < __int_as_float(sc[53]), origin_after, xlo, xhi, pos[k],
-                               ent[k], pn.cell + dst, keys + dst);
           if (key[k] == t) own += 1;
         }
       }
@@ -423,6 +458,31 @@ __global__ void __launch_bounds__(kPushThreads, 3)
       for (int k = 0; k < 2; ++k) count_leaving(cnt_next, key[k], t);
     }
     __syncthreads();
+    // A pair's windows also read nodes at weight zero, where a NaN or an infinity is
+    // none of the particle's business: those whose momentum came out not finite are
+    // pushed with their own windows.  What stays so is reported, and absorbed without
+    // moving or depositing.  (Here, and not where it was found: a branch there costs the
+    // others 3 %.)
+    if (sc[7]) {
+      for (int pos = tid; pos < nch; pos += kPushThreads) {
+        if ((order[pos] & (kCross | kStray | kSteps)) != (kCross | kSteps)) continue;
+        const unsigned ent = order[pos] & ~(kCross | kSteps);
+        const int idx = c0 + (int)(ent & 4095);
+        order[pos] = ent;
+        int l[3];
+        L.cell((ent >> 12) & 4095, l);
+        float2 o[3], u2[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) o[d] = dup2(p.o[d][idx]), u2[d] = dup2(p.u[d][idx]);
+        const float ig = push_own32(sF, L, l, pc.h, o, u2);
+        const bool good = ig > 0.0f;
+        if (!good) atomicOr(err, 8);
+        const float u[3] = {good ? u2[0].x : 0.0f, good ? u2[1].x : 0.0f, good ? u2[2].x : 0.0f};
+        const int key = finish(l, idx, pos, ent, u, ig, good);
+        if (key >= 0) atomicAdd(cnt_next + key, 1);
+      }
+      __syncthreads();
+    }
     if (npass > 1) {
       keep_lists(P, p, c0, nch, nitem, pairB);
       __syncthreads();
