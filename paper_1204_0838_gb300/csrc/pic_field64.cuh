@@ -14,8 +14,8 @@
 // is formed in FP64 (WeakTest): 0.7 % of them in a laser pulse in vacuum, 4 % around a
 // tightly focused one in plasma.  Each component of a curl takes the coarser scale of
 // the two that enter it.  A block that holds a NaN, an infinity or a value above 2^1021
-// takes FP64 arithmetic, cell by cell, so that non-finite values spread as they do in
-// FP64.
+// takes FP64 arithmetic as a whole, so that non-finite values spread as they do in
+// FP64; so does, in the magnetic kernel, one that is mostly weak.
 //
 // Measured, FP64 arithmetic -> here: step of a vacuum box of 8.4 M cells 2.00 -> 1.03 ms
 // (magnetic kernel 1.6 -> 0.60, electric kernel 0.45 -> 0.35; the 12 values read and
@@ -298,11 +298,96 @@ __device__ __forceinline__ double curl_term(const Geom<double>& g, const Smooth<
 // The weak derivatives of a block are listed and then computed by as many threads,
 // since a warp takes as long for one of them as for 32; the results take the place of
 // the staged fields.  (A vacuum step with 4x8x32 blocks: 2.35 ms with each lane its own
-// in place, 1.58 with all derivatives of a listed cell, 1.44 with the weak ones.)
+// in place, 1.58 with all derivatives of a listed cell, 1.44 with the weak ones.)  A
+// block with more of them than the list takes (ahead of a front, where values fall by
+// decades per cell), or one that is not finite, is done in FP64 as a whole, with the
+// smoothed values shared.
 constexpr int kCurlCells = FB_X * FB_Y * FB_Z;
-constexpr int kWeakList = 4096;  // of 6 x 1024; what does not fit, a thread computes in place
+constexpr int kWeakList = 3072;  // of 6 x 1024
 constexpr int kCurlFirst = 3 * FE_N > 6 * kCurlCells ? 3 * FE_N : 6 * kCurlCells;
 constexpr size_t kCurl64Smem = 8 * (kCurlFirst + 2 * (size_t)(FXN + FYN + FZN));
+
+// Index of the staged value q of a block at (bx, by, bz), or -1: beyond the grid, or
+// beyond the slabs that nx cells need.
+__device__ __forceinline__ int staged_index(const Geom<double>& g, int q, int bx, int by, int bz, int nx) {
+  const int lz = q % FE_Z, r = q / FE_Z, ly = r % FE_Y, lx = r / FE_Y;
+  int s = lx < nx + 2 ? slab_of(g, bx - 1 + lx) : -1;
+  int j = by - 1 + ly, k = bz - 1 + lz;
+  if (g.pml) {  // zero beyond the grid
+    if (j < 0 || j >= g.ny || k < 0 || k >= g.nz) s = -1;
+  } else {      // periodic; a block may exceed a small ny or nz more than once
+    j = j < 0 ? j + g.ny : (j >= g.ny ? j - g.ny : j);
+    k = k < 0 ? k + g.nz : (k >= g.nz ? k - g.nz : k);
+    if ((unsigned)j >= (unsigned)g.ny) j = wrapi(j, g.ny);
+    if ((unsigned)k >= (unsigned)g.nz) k = wrapi(k, g.nz);
+  }
+  return s < 0 ? -1 : s * g.nyz + j * g.nz + k;
+}
+
+// The smoothed fields of a block of nx slabs from staged values E(component, point),
+// as smooth(component, point, steps along the two other axes, axis) gives them.
+template <typename V, typename F>
+__device__ __forceinline__ void smooth_block(V* out, int nx, F smooth) {
+  constexpr int PX = FE_Y * FE_Z, PY = FE_Z;
+  V *sxEy = out, *sxEz = sxEy + FXN, *syEz = sxEz + FXN, *syEx = syEz + FYN, *szEx = syEx + FYN, *szEy = szEx + FZN;
+  const int tid = threadIdx.x;
+  for (int q = tid; q < (nx + 1) * FB_Y * FB_Z; q += 256) {
+    const int lz = q % FB_Z, r = q / FB_Z;
+    const int p = (r / FB_Y + 1) * PX + (r % FB_Y + 1) * PY + lz + 1;
+    sxEy[q] = smooth(1, p, PY, 1, 0);
+    sxEz[q] = smooth(2, p, PY, 1, 0);
+  }
+  for (int q = tid; q < nx * (FB_Y + 1) * FB_Z; q += 256) {
+    const int lz = q % FB_Z, r = q / FB_Z;
+    const int p = (r / (FB_Y + 1) + 1) * PX + (r % (FB_Y + 1) + 1) * PY + lz + 1;
+    syEz[q] = smooth(2, p, PX, 1, 1);
+    syEx[q] = smooth(0, p, PX, 1, 1);
+  }
+  for (int q = tid; q < nx * FB_Y * (FB_Z + 1); q += 256) {
+    const int lz = q % (FB_Z + 1), r = q / (FB_Z + 1);
+    const int p = (r / FB_Y + 1) * PX + (r % FB_Y + 1) * PY + lz + 1;
+    szEx[q] = smooth(0, p, PX, PY, 2);
+    szEy[q] = smooth(1, p, PX, PY, 2);
+  }
+}
+
+// A whole block of k_curl64 in FP64 arithmetic, in the same shared memory.
+__device__ __forceinline__ void curl_block64(const Geom<double>& g, const Smooth<double>& S, const Fields<double>& f,
+                                             const Fields<double>& hb, const FieldCoef<double>& fc, const Pml<double>& pm,
+                                             int mode, int bx, int nx, int by, int bz, double* sE,
+                                             const double (&pb)[kCurlCells / 256][3]) {
+  const int tid = threadIdx.x;
+  __syncthreads();
+  for (int q = tid; q < FE_N; q += 256) {
+    const int gi = staged_index(g, q, bx, by, bz, nx);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) sE[c * FE_N + q] = gi < 0 ? 0.0 : f.c[EX + c][gi];
+  }
+  __syncthreads();
+  double* sS = sE + kCurlFirst;
+  smooth_block(sS, nx, [&](int c, int p, int a, int b, int ax) {
+    const double* E = sE + c * FE_N + p;
+    return S.a[ax] * E[0] + S.b1[ax] * (E[a] + E[-a]) + S.b2[ax] * (E[b] + E[-b]) +
+           S.g[ax] * (E[a + b] + E[a - b] + E[-a + b] + E[-a - b]);
+  });
+  __syncthreads();
+  const double *sxEy = sS, *sxEz = sxEy + FXN, *syEz = sxEz + FXN, *syEx = syEz + FYN, *szEx = syEx + FYN, *szEy = szEx + FZN;
+#pragma unroll
+  for (int t = 0; t < kCurlCells / 256; ++t) {
+    const int q = tid + 256 * t;
+    const int lz = q % FB_Z, r = q / FB_Z, ly = r % FB_Y, lx = r / FB_Y;
+    const int j = by + ly, k = bz + lz;
+    if (lx >= nx || j >= g.ny || k >= g.nz) continue;
+    const int x0 = (lx * FB_Y + ly) * FB_Z + lz, x1 = x0 + FB_Y * FB_Z;
+    const int y0 = (lx * (FB_Y + 1) + ly) * FB_Z + lz, y1 = y0 + FB_Z;
+    const int z0 = (lx * FB_Y + ly) * (FB_Z + 1) + lz;
+    const CurlD<double> d = {(syEz[y1] - syEz[y0]) * fc.idy,     (szEy[z0 + 1] - szEy[z0]) * fc.idz,
+                             (szEx[z0 + 1] - szEx[z0]) * fc.idz, (sxEz[x1] - sxEz[x0]) * fc.idx,
+                             (sxEy[x1] - sxEy[x0]) * fc.idx,     (syEx[y1] - syEx[y0]) * fc.idy};
+    curl_store(g, f, hb, fc, pm, mode, slab_of(g, bx + lx), j, k, d, pb[t]);
+  }
+}
+
 __global__ void __launch_bounds__(256, 2)
     k_curl64(Geom<double> g, Smooth<double> S, Fields<double> f, Fields<double> hb, FieldCoef<double> fc,
              FieldConst64 k64, int mode, FieldSpan sp, Pml<double> pm) {
@@ -330,22 +415,10 @@ __global__ void __launch_bounds__(256, 2)
     int hmax[3] = {0, 0, 0};
 #pragma unroll
     for (int t = 0; t < kIt; ++t) {
-      const int q = tid + 256 * t;
-      const int lz = q % FE_Z, r = q / FE_Z, ly = r % FE_Y, lx = r / FE_Y;
-      int s = q < FE_N ? slab_of(g, bx - 1 + lx) : -1;
-      int j = by - 1 + ly, k = bz - 1 + lz;
-      if (g.pml) {  // zero beyond the grid
-        if (j < 0 || j >= g.ny || k < 0 || k >= g.nz) s = -1;
-      } else {      // periodic; a block may exceed a small ny or nz more than once
-        j = j < 0 ? j + g.ny : (j >= g.ny ? j - g.ny : j);
-        k = k < 0 ? k + g.nz : (k >= g.nz ? k - g.nz : k);
-        if ((unsigned)j >= (unsigned)g.ny) j = wrapi(j, g.ny);
-        if ((unsigned)k >= (unsigned)g.nz) k = wrapi(k, g.nz);
-      }
-      const size_t gi = s < 0 ? 0 : (size_t)s * g.nyz + (size_t)j * g.nz + k;
+      const int gi = staged_index(g, tid + 256 * t, bx, by, bz, bx1 - bx);
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        raw[t][c] = s < 0 ? 0LL : __double_as_longlong(f.c[EX + c][gi]);
+        raw[t][c] = gi < 0 ? 0LL : __double_as_longlong(f.c[EX + c][gi]);
         hmax[c] = max(hmax[c], high_bits(raw[t][c]));
       }
     }
@@ -371,53 +444,27 @@ __global__ void __launch_bounds__(256, 2)
       }
   }
   if (!finite) {  // uniform over the block
-    for (int t = 0; t < kPer; ++t) {
-      const int q = tid + 256 * t;
-      const int lz = q % FB_Z, r = q / FB_Z;
-      const int i = bx + r / FB_Y, j = by + r % FB_Y, k = bz + lz;
-      if (i < bx1 && j < g.ny && k < g.nz) curl_cell(g, S, f, hb, fc, pm, mode, i, j, k);
-    }
+    curl_block64(g, S, f, hb, fc, pm, mode, bx, bx1 - bx, by, bz, reinterpret_cast<double*>(smem_raw), pb);
     return;
   }
   __syncthreads();
-  {
-    auto E = [&](int c, int p) -> long long { return sE[c * FE_N + p]; };
-    // sum over the 3x3 points around p with steps a, b, at 2^(s + 1); the products' low
-    // words enter with their upper 15 bits
-    auto smooth = [&](int c, int p, int a, int b, const S32(&w)[4], const int(&w17)[4]) -> long long {
-      const long long e1 = E(c, p + a) + E(c, p - a), e2 = E(c, p + b) + E(c, p - b);
-      const long long cr = (E(c, p + a + b) + E(c, p + a - b)) + (E(c, p - a + b) + E(c, p - a - b));
-      const S32 x[4] = {split32(E(c, p)), split32(e1), split32(e2), split32(cr)};
-      Acc32 s = {0LL, 1LL << 28};
-      int l = 0;
+  // sum over the 3x3 points around p with steps a, b, at 2^(s + 1); the products' low
+  // words enter with their upper 15 bits
+  smooth_block(sSxEy, bx1 - bx, [&](int c, int p, int a, int b, int ax) -> long long {
+    const long long* E = sE + c * FE_N + p;
+    const long long e1 = E[a] + E[-a], e2 = E[b] + E[-b];
+    const long long cr = (E[a + b] + E[a - b]) + (E[-a + b] + E[-a - b]);
+    const S32 x[4] = {split32(E[0]), split32(e1), split32(e2), split32(cr)};
+    Acc32 s = {0LL, 1LL << 28};
+    int l = 0;
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        acc32(s, x[k], w[k]);
-        l += (x[k].lo >> 17) * w17[k];
-      }
-      s.M += (long long)l * 4;
-      return (s.H << 3) + (s.M >> 29);
-    };
-    constexpr int PX = FE_Y * FE_Z, PY = FE_Z;
-    for (int q = tid; q < FXN; q += 256) {
-      const int lz = q % FB_Z, r = q / FB_Z;
-      const int p = (r / FB_Y + 1) * PX + (r % FB_Y + 1) * PY + lz + 1;
-      sSxEy[q] = smooth(1, p, PY, 1, k64.s[0], k64.s17[0]);
-      sSxEz[q] = smooth(2, p, PY, 1, k64.s[0], k64.s17[0]);
+    for (int k = 0; k < 4; ++k) {
+      acc32(s, x[k], k64.s[ax][k]);
+      l += (x[k].lo >> 17) * k64.s17[ax][k];
     }
-    for (int q = tid; q < FYN; q += 256) {
-      const int lz = q % FB_Z, r = q / FB_Z;
-      const int p = (r / (FB_Y + 1) + 1) * PX + (r % (FB_Y + 1) + 1) * PY + lz + 1;
-      sSyEz[q] = smooth(2, p, PX, 1, k64.s[1], k64.s17[1]);
-      sSyEx[q] = smooth(0, p, PX, 1, k64.s[1], k64.s17[1]);
-    }
-    for (int q = tid; q < FZN; q += 256) {
-      const int lz = q % (FB_Z + 1), r = q / (FB_Z + 1);
-      const int p = (r / FB_Y + 1) * PX + (r % FB_Y + 1) * PY + lz + 1;
-      sSzEx[q] = smooth(0, p, PX, PY, k64.s[2], k64.s17[2]);
-      sSzEy[q] = smooth(1, p, PX, PY, k64.s[2], k64.s17[2]);
-    }
-  }
+    s.M += (long long)l * 4;
+    return (s.H << 3) + (s.M >> 29);
+  });
   __syncthreads();
   double* sWeak = reinterpret_cast<double*>(smem_raw);  // [6][kCurlCells]
   unsigned weak_bits = 0;                               // six per cell of the thread
@@ -444,18 +491,19 @@ __global__ void __launch_bounds__(256, 2)
     if (weak_bits) {
       int pos = atomicAdd(sh + 3, __popc(weak_bits));
       for (unsigned m = weak_bits; m; m &= m - 1, ++pos) {
-        const int t = (__ffs(m) - 1) / 6, n = (__ffs(m) - 1) % 6, q = tid + 256 * t, r = q / FB_Z;
-        if (pos < kWeakList)
-          list[pos] = (unsigned short)(n * kCurlCells + q);
-        else
-          sWeak[n * kCurlCells + q] = curl_term(g, S, f, fc, n, bx + r / FB_Y, by + r % FB_Y, bz + q % FB_Z);
+        const int t = (__ffs(m) - 1) / 6, n = (__ffs(m) - 1) % 6, q = tid + 256 * t;
+        if (pos < kWeakList) list[pos] = (unsigned short)(n * kCurlCells + q);
       }
     }
     static_assert(6 * kPer <= 32, "six bits per cell");
     static_assert(6 * kCurlCells <= 65536, "16-bit entries");
     __syncthreads();
-    const int nweak = min(sh[3], kWeakList);
-    if (nweak > 0) {  // uniform over the block
+    const int nweak = sh[3];  // uniform over the block
+    if (nweak > kWeakList) {
+      curl_block64(g, S, f, hb, fc, pm, mode, bx, bx1 - bx, by, bz, reinterpret_cast<double*>(smem_raw), pb);
+      return;
+    }
+    if (nweak > 0) {
 #pragma unroll 1
       for (int m = tid; m < nweak; m += 256) {
         const int n = list[m] / kCurlCells, q = list[m] % kCurlCells, r = q / FB_Z;

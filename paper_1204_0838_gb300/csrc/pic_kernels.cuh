@@ -242,25 +242,6 @@ __device__ __forceinline__ void curl_store(const Geom<T>& g, const Fields<T>& f,
   }
 }
 
-// One cell of k_curl_tiled from global memory.
-template <typename T>
-__device__ __forceinline__ void curl_cell(const Geom<T>& g, const Smooth<T>& S, const Fields<T>& f, const Fields<T>& hb,
-                                          const FieldCoef<T>& fc, const Pml<T>& pm, int mode, int i, int j, int k) {
-  const int s = slab_of(g, i), sm = slab_of(g, i - 1), sp = slab_of(g, i + 1);
-  const T *Ex = f.c[EX], *Ey = f.c[EY], *Ez = f.c[EZ];
-  CurlD<T> d;
-  d.dyEz = (smooth_y(Ez, g, S, sm, s, sp, j + 1, k) - smooth_y(Ez, g, S, sm, s, sp, j, k)) * fc.idy;
-  d.dzEy = (smooth_z(Ey, g, S, sm, s, sp, j, k + 1) - smooth_z(Ey, g, S, sm, s, sp, j, k)) * fc.idz;
-  d.dzEx = (smooth_z(Ex, g, S, sm, s, sp, j, k + 1) - smooth_z(Ex, g, S, sm, s, sp, j, k)) * fc.idz;
-  d.dxEz = (smooth_x(Ez, g, S, sp, j, k) - smooth_x(Ez, g, S, s, j, k)) * fc.idx;
-  d.dxEy = (smooth_x(Ey, g, S, sp, j, k) - smooth_x(Ey, g, S, s, j, k)) * fc.idx;
-  d.dyEx = (smooth_y(Ex, g, S, sm, s, sp, j + 1, k) - smooth_y(Ex, g, S, sm, s, sp, j, k)) * fc.idy;
-  const size_t id = (size_t)s * g.nyz + (size_t)j * g.nz + k;
-  const T* const* src = mode == 1 ? hb.c : f.c + BX;
-  const T b[3] = {src[0][id], src[1][id], src[2][id]};
-  curl_store(g, f, hb, fc, pm, mode, s, j, k, d, b);
-}
-
 // ---------------------------------------------------------------------------
 // Smoothed curl, shared-memory tiled.  A CTA covers a block of CB_X x CB_Y x
 // CB_Z cells (window-relative slabs i0 + blockIdx.x * CB_X ...).  It stages E
