@@ -45,13 +45,13 @@ ALG_BYTES_PER_PARTICLE = {"fp64": lambda ppc: 112 + 72 / ppc, "fp32": lambda ppc
 # precision on a 256x128x128 window in a run's own state (run for 256 steps past
 # a load at rest), 8x8x8 tiles; traffic per launch scales with the particles
 # processed.
-NCU_TRAFFIC_PER_PARTICLE = {"fp64": (822.058752e6 + 625.361664e6) / 8336282,
-                            "fp32": (419.947264e6 + 309.271552e6) / 8336282}
+NCU_TRAFFIC_PER_PARTICLE = {"fp64": (812.474368e6 + 600.525824e6) / 8336282,
+                            "fp32": (419.928064e6 + 309.740288e6) / 8336282}
 TRAFFIC_SOURCE = ("ncu dram__bytes_read.sum + dram__bytes_write.sum per particle (c1 spacings, 256x128x128 "
                   "window in a run's state) x particles per launch")
-LIMITER = {"fp64": ("latency at 16 warps per SM (ncu: issue active 39 %, shared-memory pipe 54 %, integer ALU 30 %, "
-                    "FMA 26 %, FP64 pipe 25 %; DRAM 4 %)"),
-           "fp32": ("shared-memory pipe (ncu: L1tex 76 %, issue active 48 %, FMA 37 %, 24 warps per SM; "
+LIMITER = {"fp64": ("latency at 16 warps per SM (ncu: issue active 40 %, shared-memory pipe 54 %, integer ALU 31 %, "
+                    "FMA 27 %, FP64 pipe 26 %; DRAM 4 %)"),
+           "fp32": ("shared-memory pipe (ncu: L1tex 76 %, issue active 49 %, FMA 37 %, 24 warps per SM; "
                     "DRAM 7 %)")}
 
 

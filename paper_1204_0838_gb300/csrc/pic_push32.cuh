@@ -17,8 +17,7 @@
 //   neighbouring cells.
 // - Two phases over one shared-memory region: all particles gather and move
 //   first (staged E, B), then the region becomes the J tile and all deposit.
-//   Two CTAs of 256 threads fit an SM, and each phase's code is short enough
-//   for the instruction cache.
+//   Each phase's code is short enough for the instruction cache.
 // - Particles that leave their cell deposit on other windows; they are listed
 //   and deposit one per lane after the pairs, so that no warp runs the wide
 //   window for a few lanes.
@@ -32,14 +31,14 @@
 //   again for every rotation instead of kept; two particles' arithmetic goes in
 //   packed FP32 instructions.
 //
-// Measured (whole step, before -> after the two kernels' steps): 118 M particles,
-// 1536x256x256 cells, 2 per cell 41.3 -> 26.2 ms; 14 M particles, 4 per cell,
-// absorbing layers 4.85 -> 2.53 ms; 3.1 M at random places, a quarter leaving
+// Measured (whole step, the one-pass kernel -> this one): 118 M particles,
+// 1536x256x256 cells, 2 per cell 41.3 -> 26.1 ms; 14 M particles, 4 per cell,
+// absorbing layers 4.85 -> 2.51 ms; 3.1 M at random places, a quarter leaving
 // their cell each step, 1.01 -> 0.72 ms.  With the bodies unrolled the first took
-// 38.6 ms, with two CTAs at 128 registers 27.6.  Now about 2,600 instructions per
-// 32 particles (4 per cell), issued 54 % of the time; shared-memory wavefronts
-// take 65 % of the cycles; barriers and the latency of the particle loads share
-// the rest.
+// 38.6 ms, with two CTAs at 128 registers 27.6.  In a run's state, 2 per cell: 3,370
+// instructions per 32 particles, issued 49 % of the time, the shared-memory pipe 76 %
+// busy; waits at barriers (uneven last rounds of a tile) and for shared memory are the
+// largest stalls.
 //
 // Current: sums of integers at 2^s per tile and component, with s the largest
 // for which B 2^s < 2^42, B = |q jc| sum |w|.  A contribution is a product of

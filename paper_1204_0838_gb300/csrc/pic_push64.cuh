@@ -24,12 +24,12 @@
 // - a current word pair with a carry became three overlapping words added by
 //   reductions that return nothing.
 //
-// Measured (whole step, before -> after): 118 M particles, 1536x256x256 cells
-// 183 -> 93 ms; 7 M, 384x96x96 10.6 -> 5.26 ms; 436 k at random places 0.97 ->
-// 0.62 ms.  About 9,000 instructions per particle, issued 43 % of the time; the
-// gather takes 42 % of the kernel, the ordered deposit 32 %, particles that left
-// their cell 6 %, the flush 4 %; no pipe is above a third (integer ALU, FMA,
-// FP64) and shared memory is at 45 %: fixed latencies at 16 warps per SM bound it.
+// Measured (the push of a step, the one-pass kernel -> this one): 119 M particles,
+// 1536x256x256 cells 167 -> 69 ms; whole steps, with the field update's change: 118 M
+// 183 -> 78.6 ms, 7 M, 384x96x96 10.6 -> 4.8 ms, 436 k at random places 0.97 -> 0.54 ms.
+// In a run's state 9,380 instructions per 32 particles, issued 40 % of the time; the
+// shared-memory pipe is 54 % busy, no other above a third (integer ALU 31 %, FMA 27 %,
+// FP64 26 %): fixed latencies at 16 warps per SM bound it.
 #pragma once
 
 #include "pic_push.cuh"
