@@ -256,8 +256,8 @@ __device__ __forceinline__ void curl_store(const Geom<T>& g, const Fields<T>& f,
 // ---------------------------------------------------------------------------
 constexpr int CB_X = 4, CB_Y = 8, CB_Z = 32;
 // Window-relative slabs of a launch: block b covers [b step, b step + width).
-// All slabs: step = width = CB_X; the two at the window's edges: step = nx - 1,
-// width 1.
+// All slabs: step = width = the blocks' extent (CB_X; FP64 FB_X); the two at the
+// window's edges: step = nx - 1, width 1.
 struct FieldSpan {
   int step, width;
 };
