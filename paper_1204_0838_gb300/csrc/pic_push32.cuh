@@ -55,7 +55,9 @@
 // - 2^-31 of its own |q w jc| for a lighter particle or one that left its cell:
 //   these deposit one per lane, with a kp of their own.  (With one kp for all, the
 //   current of particles at 1e-4 of the largest weight was off by 1e-4 of itself,
-//   of those at 1e-6 by 1e-2.)
+//   of those at 1e-6 by 1e-2.  A step of 1.6 M particles takes 414 us with equal
+//   weights, 493 with one in a hundred a hundred times heavier, so that nearly all
+//   others are light.)
 #pragma once
 
 #include "pic_push.cuh"
